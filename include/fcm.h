@@ -30,15 +30,7 @@
  *   - Arithmetic: memberships and per-thread sums in FP32; the sums across
  *     threads and blocks (center numerators/denominators and J) in
  *     compensated FP32 (double-float, about 44 bits) or FP64, in a fixed
- *     order. A run is deterministic, with one exception: on images large
- *     enough that every warp of the default whole-run kernel (stored U)
- *     holds more than a ring of tiles (about 4 million pixels), 40% of each
- *     pass's tiles go to whichever warps ask first, so SMs that stream
- *     faster take more of them (about 11% faster on a 256^3 volume). Which
- *     block sums which tile then depends on timing, and so does the FP32
- *     rounding of the block sums: results agree to rounding, and the
- *     iteration count can differ by one when delta_k lands at eps.
- *     FCM_OPT_DETERMINISTIC keeps fixed shares for bit-reproducible runs.
+ *     order. A run is deterministic: the same call gives the same bits.
  *     The histogram-domain entry points form V^1 the same way from the
  *     pixels; their loop over the 256 bins sums non-negative terms in FP32
  *     within each warp (a fixed tree, at most five roundings) and combines
@@ -93,13 +85,13 @@ extern "C" {
 #define FCM_OPT_NO_TMA 4   /* plain-load pass kernel instead of the TMA-fed one */
 #define FCM_OPT_NO_PERSISTENT 8 /* one launch per pass (graph or host loop) instead of
                                     one cooperative launch for the whole run */
-#define FCM_OPT_RECOMPUTE 16 /* do not store U between iterations: recompute U^{k-1}
-                                 from V^{k-1}, so an iteration reads only x; U^k is
-                                 written once at the end (one cooperative launch;
-                                 needs n % 4 == 0 and 16-byte-aligned rows) */
-#define FCM_OPT_DETERMINISTIC 32 /* whole-run kernel: every tile in fixed warp
-                                     shares, so the result does not depend on
-                                     timing (see the arithmetic note above) */
+#define FCM_OPT_RECOMPUTE 16 /* insist on the whole-run launch, which keeps no U
+                                 between iterations (an iteration reads only x; U^k
+                                 is written once at the end): refused unless
+                                 n % 4 == 0 and the rows are 16-byte aligned; takes
+                                 precedence over the three options above */
+#define FCM_OPT_DETERMINISTIC 32 /* bit-reproducible results; every run is (kept for
+                                     callers that ask for it) */
 
 typedef struct fcm_ctx* fcm_handle;
 
@@ -138,9 +130,9 @@ void fcm_destroy(fcm_handle h);
  * of times and then gives up: the run ends with FCM_ERR_TIMEOUT (U and V
  * unspecified) and the handle stays usable.
  *
- *   grid_wait_spins   polls, about 128 ns apart, of a grid-wide barrier
- *                     (whole-run, U-free, multi-feature and round-schedule
- *                     kernels). 0 = the default 2^23 (about 1 s). The
+ *   grid_wait_spins   polls, a fraction of a microsecond apart, of a grid-wide
+ *                     wait (whole-run, multi-feature and round-schedule
+ *                     kernels). 0 = the default 2^23 (a few seconds). The
  *                     environment variable FCM_TIMEOUT_SPINS sets the default
  *                     of new handles.
  *   tma_wait_polls    suspensions, up to about 1 ms each, of a wait for a TMA
@@ -181,16 +173,19 @@ int fcm_get_limits(fcm_handle h, fcm_limits* lim);
  *             With FCM_INIT_U and U0 != NULL the initial membership is read
  *             from U0 and left unchanged; with U0 == NULL (or U0 == U) it is
  *             read from U. Ignored with FCM_INIT_V.
- *   U         C*n floats, cluster-major, device or host. Out: U^k (the run
- *             updates it in place from the first iteration on).
+ *   U         C*n floats, cluster-major, device or host. Out: U^k.
  *   V         C floats, device or host. In: V^0 when init_mode == FCM_INIT_V.
  *             Out: V^k.
- *   options   FCM_OPT_* bits. By default, when n % 4 == 0 and the buffers are
- *             16-byte aligned, the whole run is one cooperative kernel launch
- *             (grid-wide exchange of the per-block sums after each pass);
- *             otherwise, or with FCM_OPT_NO_PERSISTENT, one launch per pass
- *             inside a CUDA graph WHILE loop (or a host loop with
- *             FCM_OPT_NO_GRAPH).
+ *   options   FCM_OPT_* bits. By default the whole run is one cooperative
+ *             kernel launch (grid-wide exchange of the per-block sums after
+ *             each pass). It keeps no U between iterations: an iteration takes
+ *             max|U^k - U^{k-1}| over a sample of the pixels, which bounds
+ *             delta_k from below, and over every pixel only when that bound
+ *             does not already reach eps, at max_iter, or for a trace; the stop
+ *             decision and the reported delta_k and J_k are exact. With
+ *             FCM_OPT_NO_PERSISTENT, FCM_OPT_NO_GRAPH or FCM_OPT_NO_TMA, one
+ *             launch per pass inside a CUDA graph WHILE loop (or a host loop
+ *             with FCM_OPT_NO_GRAPH), with U^{k-1} stored.
  *   rep       nullable; filled on return.
  *
  * Returns FCM_OK, FCM_NOT_CONVERGED, or an error. On FCM_ERR_BAD_INPUT the
@@ -575,8 +570,8 @@ int fcm_time_pass(fcm_handle h, const float* x, int64_t n, int C, float m, float
  * acceptable. fcm_run keeps its scratch in a handle that allocates on first
  * use; this entry point needs no handle and allocates nothing (no cudaMalloc,
  * cudaFree or allocating library call). Its scratch — the device-side run
- * state and the per-block partial sums — lives in one fixed array inside the
- * library image (about 80 KB plus the state) that every GPU which loads the
+ * state and the blocks' exchange slots — lives in one fixed array inside the
+ * library image (about 150 KB plus the state) that every GPU which loads the
  * library holds until the process exits.
  *
  *   x, n, C, m, eps, max_iter, init_mode, U0, U, V: as for fcm_run, except
@@ -587,7 +582,7 @@ int fcm_time_pass(fcm_handle h, const float* x, int64_t n, int C, float m, float
  *             on the current device. The call synchronises that stream.
  *   rep       nullable; filled on return.
  *
- * Limit: the scratch holds partial sums for at most FCM_NOALLOC_MAX_BLOCKS
+ * Limit: the scratch holds exchange slots for at most FCM_NOALLOC_MAX_BLOCKS
  * thread blocks; a device that would need more (more SMs than any current
  * GPU) gets FCM_ERR_TOO_LARGE. Other bad arguments give FCM_ERR_INVALID_ARG.
  *

@@ -27,7 +27,7 @@
 #include "fcm.h"
 #include "fcm_device.cuh"
 #include "fcm_internal.h"
-#include "fcm_recompute.h"
+#include "fcm_run.h"
 #include "fcm_runtime.h"
 
 using namespace fcm;
@@ -36,19 +36,19 @@ namespace {
 
 SingleTable g_table;
 std::once_flag g_table_once;
-RcTable g_rc;
+RunTable g_run;
 
 void init_table() {
     std::memset(&g_table, 0, sizeof(g_table));
-    std::memset(&g_rc, 0, sizeof(g_rc));
-    register_rc_c1(g_rc);
-    register_rc_c2(g_rc);
-    register_rc_c3(g_rc);
-    register_rc_c4(g_rc);
-    register_rc_c5(g_rc);
-    register_rc_c6(g_rc);
-    register_rc_c7(g_rc);
-    register_rc_c8(g_rc);
+    std::memset(&g_run, 0, sizeof(g_run));
+    register_run_c1(g_run);
+    register_run_c2(g_run);
+    register_run_c3(g_run);
+    register_run_c4(g_run);
+    register_run_c5(g_run);
+    register_run_c6(g_run);
+    register_run_c7(g_run);
+    register_run_c8(g_run);
     register_single_c1(g_table);
     register_single_c2(g_table);
     register_single_c3(g_table);
@@ -70,28 +70,6 @@ WaitLimits default_limits() {
     return w;
 }
 
-// Percent of a pass's tiles the whole-run kernel deals in fixed warp shares;
-// FCM_RUN_STATIC_PCT overrides the default (100: fixed shares only).
-int default_static_pct() {
-    if (const char* e = std::getenv("FCM_RUN_STATIC_PCT")) {
-        const long v = std::atol(e);
-        if (v >= 1 && v <= 100) return (int)v;
-    }
-    return DEFAULT_STATIC_PCT;
-}
-
-// Grid of a whole-run kernel for n pixels when at most max_blocks blocks are
-// co-resident: the fewest blocks that keep the largest number of 128-pixel
-// tiles per warp that max_blocks would give, so every warp holds about the
-// same number of tiles (8,192 tiles on 304 blocks would leave a third of the
-// warps one tile more than the rest; 256 blocks give each warp 4).
-int run_grid(int64_t n, int64_t max_blocks) {
-    if (max_blocks < 1) return 0;
-    const int64_t ntiles = (n + WARP_TILE - 1) / WARP_TILE;
-    const int64_t per_warp = (ntiles + max_blocks * NWARP - 1) / (max_blocks * NWARP);
-    return (int)std::max<int64_t>(1, (ntiles + per_warp * NWARP - 1) / (per_warp * NWARP));
-}
-
 bool is_device_pointer(const void* p) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -105,9 +83,20 @@ bool is_device_pointer(const void* p) {
 
 namespace fcm {
 
-const SingleTable& single_table() {
+const RunTable& run_table() {
     std::call_once(g_table_once, init_table);
-    return g_table;
+    return g_run;
+}
+
+// Every thread of the whole-run kernel takes four pixels at a time: the fewest
+// blocks that keep the largest number of such steps per thread that max_blocks
+// would give, so the threads hold about the same number of pixels (a 1 M-pixel
+// image: 128 blocks with 4 steps each; 152 blocks would also need 4).
+int run_grid(int64_t n, int64_t max_blocks) {
+    if (max_blocks < 1) return 0;
+    const int64_t quads = (n + 3) / 4;
+    const int64_t steps = (quads + max_blocks * RUN_NT - 1) / (max_blocks * RUN_NT);
+    return (int)std::max<int64_t>(1, (quads + steps * RUN_NT - 1) / (steps * RUN_NT));
 }
 
 int ctx_fail(fcm_ctx* h, cudaError_t e, const char* what) {
@@ -172,6 +161,10 @@ int ctx_grow(fcm_ctx* h, void** p, size_t* cap, size_t bytes, const char* what) 
 
 namespace {
 
+size_t run_slot_bytes(const fcm_ctx* h) {
+    return (size_t)RUN_SLOT_BYTES * run_slots(FCM_MAX_CLUSTERS) * h->num_sms;
+}
+
 // Each buffer is allocated when missing, so a call after a failed allocation
 // completes the workspace.
 int ensure_single_workspace(fcm_ctx* h) {
@@ -181,10 +174,42 @@ int ensure_single_workspace(fcm_ctx* h) {
     }
     if (!h->h_st) CK(host_malloc(h, &h->h_st, sizeof(RunState)));
     if (!h->d_partials) {
+        // the pass kernels' partials, then the exchange slots of the whole-run
+        // kernel, zero before its first run (no tag is 0)
         h->partial_blocks = h->num_sms * 32;
-        CK(dev_malloc(h, &h->d_partials, sizeof(double) * SLOTS_MAX * h->partial_blocks));
+        const size_t bytes = sizeof(double) * SLOTS_MAX * h->partial_blocks;
+        CK(dev_malloc(h, &h->d_partials, bytes + run_slot_bytes(h)));
+        h->d_slots = reinterpret_cast<char*>(h->d_partials) + bytes;
+        h->run_nonce = 0xffffffffu;  // the first run zeroes the slots
     }
     return 0;
+}
+
+// The number of the next whole run of the handle: the upper half of its
+// exchanges' tags. The slots are zeroed when the numbers start over, so no slot
+// can show a tag of an earlier run of the same number.
+int next_nonce(fcm_ctx* h, unsigned* nonce) {
+    if (++h->run_nonce == 0) {
+        CK(cudaMemsetAsync(h->d_slots, 0, run_slot_bytes(h), h->stream));
+        h->run_nonce = 1;
+    }
+    *nonce = h->run_nonce;
+    return 0;
+}
+
+// Co-resident blocks of the whole-run kernel (one per SM), or 0 when it does
+// not fit.
+int64_t max_run_blocks(fcm_ctx* h, const void* k) {
+    auto it = h->occupancy.find(k);
+    if (it == h->occupancy.end()) {
+        int nb = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, RUN_NT, 0) != cudaSuccess) {
+            cudaGetLastError();
+            nb = 0;
+        }
+        it = h->occupancy.emplace(k, nb).first;
+    }
+    return it->second > 0 ? h->num_sms : 0;
 }
 
 // Blocks per SM of a pass kernel with `smem` bytes of dynamic shared memory;
@@ -339,7 +364,6 @@ int fcm_create(fcm_handle* out, int device, void* cuda_stream) {
     h->max_smem_optin = (int)prop.sharedMemPerBlockOptin;
     h->device_name = prop.name;
     h->limits = default_limits();
-    h->static_pct = default_static_pct();
     *out = h;
     return FCM_OK;
 }
@@ -495,7 +519,7 @@ int fcm_run(fcm_handle h, const float* x, int64_t n, int C, float m, float eps, 
     hs->C = C;
     hs->status = STATUS_RUNNING;
     hs->lim = h->limits;
-    hs->static_pct = (options & FCM_OPT_DETERMINISTIC) ? 100 : h->static_pct;
+    hs->from_u = init_mode == FCM_INIT_U;
     if (init_mode == FCM_INIT_V && !V_dev) std::memcpy(hs->V0, V, sizeof(float) * C);
     CK(cudaMemcpyAsync(h->d_st, hs, sizeof(RunState), cudaMemcpyHostToDevice, h->stream));
     if (init_mode == FCM_INIT_V && V_dev)
@@ -507,19 +531,17 @@ int fcm_run(fcm_handle h, const float* x, int64_t n, int C, float m, float eps, 
                          ((uintptr_t)hs->Uprev % 16 == 0);
     int run_blocks = 0;
     const bool recompute = (options & FCM_OPT_RECOMPUTE) != 0;
-    const int iu = init_mode == FCM_INIT_U ? 0 : 1;
-    const void* krun = recompute ? (const void*)g_rc.run[C][mk][iu] : (const void*)g_table.run[C][mk][iu];
-    const int run_smem = recompute ? g_rc.smem[C][iu] : g_table.run_smem[C];
+    const void* krun = (const void*)g_run.run[C][mk];
     if (recompute && !(aligned && h->coop))
         return ctx_invalid(h, "FCM_OPT_RECOMPUTE needs n % 4 == 0, 16-byte-aligned rows and cooperative launch");
-    if (recompute ||
-        (aligned && h->coop && !(options & (FCM_OPT_NO_TMA | FCM_OPT_NO_PERSISTENT | FCM_OPT_NO_GRAPH)))) {
-        run_blocks = run_grid(n, (int64_t)h->num_sms * blocks_per_sm(h, krun, run_smem));
-    }
+    if (recompute || (h->coop && !(options & (FCM_OPT_NO_TMA | FCM_OPT_NO_PERSISTENT | FCM_OPT_NO_GRAPH))))
+        run_blocks = run_grid(n, max_run_blocks(h, krun));
     if (run_blocks > 0) {
         // the whole run: one cooperative launch (all blocks co-resident)
-        void* args[2] = {&h->d_st, &h->d_partials};
-        CK(cudaLaunchCooperativeKernel(krun, dim3(run_blocks), dim3(NT), args, run_smem, h->stream));
+        unsigned nonce;
+        if ((rc = next_nonce(h, &nonce))) return rc;
+        void* args[3] = {&h->d_st, &h->d_slots, &nonce};
+        CK(cudaLaunchCooperativeKernel(krun, dim3(run_blocks), dim3(RUN_NT), args, 0, h->stream));
         h->last_blocks = run_blocks;
         h->last_path = 2;
     } else {
@@ -616,10 +638,8 @@ int fcm_run_stream(fcm_handle h, int n_images, const float* const* x, int64_t n,
     cudaEvent_t ev_start = h->pipe_ev[3 * NS], ev_end = h->pipe_ev[3 * NS + 1];
 
     const int mk = mkind_of(m);
-    const bool recompute = (options & FCM_OPT_RECOMPUTE) != 0;
-    const void* krun = recompute ? (const void*)g_rc.run[C][mk][0] : (const void*)g_table.run[C][mk][0];
-    const int run_smem = recompute ? g_rc.smem[C][0] : g_table.run_smem[C];
-    const int run_blocks = run_grid(n, (int64_t)h->num_sms * blocks_per_sm(h, krun, run_smem));
+    const void* krun = (const void*)g_run.run[C][mk];
+    const int run_blocks = run_grid(n, max_run_blocks(h, krun));
     if (run_blocks < 1) return ctx_invalid(h, "the whole-run kernel does not fit on this device");
 
     // the copy streams start behind the work already queued on the handle's stream
@@ -645,7 +665,7 @@ int fcm_run_stream(fcm_handle h, int n_images, const float* const* x, int64_t n,
         hs->C = C;
         hs->status = STATUS_RUNNING;
         hs->lim = h->limits;
-        hs->static_pct = (options & FCM_OPT_DETERMINISTIC) ? 100 : h->static_pct;
+        hs->from_u = 1;
         const float* u0 = (U0 && U0[i]) ? U0[i] : U[i];
         // upload, once the download of image i - NS has drained this set
         if (i >= NS) e = cudaStreamWaitEvent(h->pipe_in, out_done[b], 0);
@@ -655,9 +675,11 @@ int fcm_run_stream(fcm_handle h, int n_images, const float* const* x, int64_t n,
         // the run, with its state uploaded before and read back after
         if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, in_done[b], 0);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_st, hs, sizeof(RunState), cudaMemcpyHostToDevice, h->stream);
-        void* args[2] = {&h->d_st, &h->d_partials};
+        unsigned nonce = 0;
+        if (e == cudaSuccess && next_nonce(h, &nonce)) e = cudaErrorUnknown;
+        void* args[3] = {&h->d_st, &h->d_slots, &nonce};
         if (e == cudaSuccess)
-            e = cudaLaunchCooperativeKernel(krun, dim3(run_blocks), dim3(NT), args, run_smem, h->stream);
+            e = cudaLaunchCooperativeKernel(krun, dim3(run_blocks), dim3(RUN_NT), args, 0, h->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(hs, h->d_st, sizeof(RunState), cudaMemcpyDeviceToHost, h->stream);
         if (e == cudaSuccess) e = cudaEventRecord(run_done[b], h->stream);
         // download
@@ -734,7 +756,6 @@ int fcm_time_pass(fcm_handle h, const float* x, int64_t n, int C, float m, float
     hs->k = 1;
     hs->status = STATUS_RUNNING;
     hs->lim = h->limits;
-    hs->static_pct = (options & FCM_OPT_DETERMINISTIC) ? 100 : h->static_pct;
     const bool V_dev = is_device_pointer(V);
     if (!V_dev)
         for (int j = 0; j < C; ++j) {

@@ -258,6 +258,131 @@ __device__ __forceinline__ f2 membership_pair(f2 x2, const f2 (&v2)[C], float m,
     return pack2(ja, jb);
 }
 
+// ---------------------------------------------------------------------------
+// u^m alone, for passes that only add up Eq. 3's sums.
+// ---------------------------------------------------------------------------
+
+// u^m of two pixels by the scalar weight form, for the pairs that the packed
+// forms below cannot take. Not inlined: it is rare, and the packed loop keeps
+// its registers.
+template <int C>
+struct Powers {
+    float a[C], b[C];
+};
+template <int C, int MK>
+__device__ __noinline__ Powers<C> powers_scalar(float xa, float xb, const float* vs, float m, float inv_m1) {
+    float v[C], u[C];
+    Powers<C> w;
+#pragma unroll
+    for (int j = 0; j < C; ++j) v[j] = vs[j];
+    membership<C, MK>(xa, v, m, inv_m1, u, w.a);
+    membership<C, MK>(xb, v, m, inv_m1, u, w.b);
+    return w;
+}
+
+// Power-of-two factor that brings the centers' spread to [1, 2), for the
+// products of powers_pair at m = 1.5 (1 when the spread is 0 or extreme).
+// Scaling by it is exact, so it changes the products' range and nothing else.
+template <int C>
+__device__ __forceinline__ float spread_scale(const f2 (&v2)[C]) {
+    float lo = lo2(v2[0]), hi = lo;
+#pragma unroll
+    for (int j = 1; j < C; ++j) {
+        lo = fminf(lo, lo2(v2[j]));
+        hi = fmaxf(hi, lo2(v2[j]));
+    }
+    const int e = (__float_as_int(hi - lo) >> 23) - 127;
+    return (e < -60 || e > 60) ? 1.0f : __int_as_float((127 - e) << 23);
+}
+
+// Products P_j = prod_{k != j} b_k.
+template <int C>
+__device__ __forceinline__ void co_products(const f2 (&b)[C], f2 (&P)[C]) {
+    if (C == 1) {
+        P[0] = pack2(1.0f, 1.0f);
+        return;
+    }
+    f2 pre[C], suf[C];
+#pragma unroll
+    for (int j = 1; j < C; ++j) pre[j] = (j == 1) ? b[0] : mul2(pre[j - 1], b[j - 1]);
+#pragma unroll
+    for (int j = C - 2; j >= 0; --j) suf[j] = (j == C - 2) ? b[C - 1] : mul2(suf[j + 1], b[j + 1]);
+#pragma unroll
+    for (int j = 0; j < C; ++j) P[j] = (j == 0) ? suf[0] : (j == C - 1) ? pre[C - 1] : mul2(pre[j], suf[j]);
+}
+
+// True when a is a normal positive float (not 0, subnormal, infinite or NaN).
+__device__ __forceinline__ bool normal_pos(float a) {
+    return (unsigned)(__float_as_int(a) - 0x00800000) < 0x7f000000u;
+}
+
+// um2[j] = u_j^m and d2[j] = x - v_j of two pixels (packed x2). vs: the C
+// centers in memory, for the scalar form. vq2, xs: the centers and the pair as
+// the differences d2 use them (scaled by spread_scale at m = 1.5, unscaled
+// otherwise).
+//   m = 2, 3  the product form of membership_pair.
+//   m = 1.5   with p_j = prod_{k != j} d_k^2, sqrt(u_j) = p_j / sqrt(sum_k
+//             p_k^2): one reciprocal square root per pixel where the weight form
+//             takes C reciprocals and C square roots; u^1.5 is its cube.
+//   other m   w_j = 2^t_j, t_j = (log2 d2min - log2 d2_j) / (m - 1), S = sum w:
+//             u_j^m = 2^(m (t_j - log2 S)), without the C logarithms of u_j.
+template <int C, int MK>
+__device__ __forceinline__ void powers_pair(f2 x2, f2 xs, const f2 (&vq2)[C], float m, float inv_m1,
+                                            const float* vs, f2 (&um2)[C], f2 (&d2)[C]) {
+#pragma unroll
+    for (int j = 0; j < C; ++j) d2[j] = sub2(xs, vq2[j]);
+    if (MK == M_TWO || MK == M_THREE || MK == M_ONE_HALF) {
+        f2 b[C], P[C];
+#pragma unroll
+        for (int j = 0; j < C; ++j) b[j] = (MK == M_THREE) ? abs2(d2[j]) : mul2(d2[j], d2[j]);
+        co_products<C>(b, P);
+        f2 S = (MK == M_ONE_HALF) ? mul2(P[0], P[0]) : P[0];
+#pragma unroll
+        for (int j = 1; j < C; ++j) S = (MK == M_ONE_HALF) ? fma2(P[j], P[j], S) : add2(S, P[j]);
+        float s0, s1;
+        unpack2(S, s0, s1);
+        if (normal_pos(s0) && normal_pos(s1)) {
+            const f2 r = (MK == M_ONE_HALF) ? pack2(rsqrt_approx(s0), rsqrt_approx(s1))
+                                            : pack2(rcp_approx(s0), rcp_approx(s1));
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                const f2 u = mul2(P[j], r);
+                um2[j] = mul2(u, u);
+                if (MK != M_TWO) um2[j] = mul2(um2[j], u);
+            }
+            return;
+        }
+    } else {
+        float ta[C], tb[C];
+        float la = __int_as_float(0x7f800000), lb = la;
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            float da, db;
+            unpack2(mul2(d2[j], d2[j]), da, db);
+            ta[j] = lg2_approx(da);  // a squared distance below 2^-126 reads as 0: -inf
+            tb[j] = lg2_approx(db);
+            la = fminf(la, ta[j]);
+            lb = fminf(lb, tb[j]);
+        }
+        if (la >= -126.0f && lb >= -126.0f) {
+            f2 S = pack2(0.0f, 0.0f);
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                ta[j] = inv_m1 * (la - ta[j]);
+                tb[j] = inv_m1 * (lb - tb[j]);
+                S = add2(S, pack2(ex2_approx(ta[j]), ex2_approx(tb[j])));
+            }
+            const float ga = lg2_approx(lo2(S)), gb = lg2_approx(hi2(S));
+#pragma unroll
+            for (int j = 0; j < C; ++j) um2[j] = pack2(ex2_approx(m * (ta[j] - ga)), ex2_approx(m * (tb[j] - gb)));
+            return;
+        }
+    }
+    const Powers<C> w = powers_scalar<C, MK>(lo2(x2), hi2(x2), vs, m, inv_m1);
+#pragma unroll
+    for (int j = 0; j < C; ++j) um2[j] = pack2(w.a[j], w.b[j]);
+}
+
 // Compensated FP32 ("double-float") sum, hi + lo, with Knuth's TwoSum: long
 // sums of the center numerators/denominators and of J carry about 44 bits
 // while using only FP32 instructions.

@@ -20,4 +20,6 @@ __device__ __forceinline__ DF df_div(DF a, DF b) {
     return DF{s, q1 - (s - q0)};
 }
 
+__device__ __forceinline__ double df_to_double(DF d) { return (double)d.hi + (double)d.lo; }
+
 }  // namespace fcm

@@ -11,16 +11,6 @@ namespace fcm {
 constexpr int NT = 256;                                  // threads per block of the pass
 constexpr int NWARP = NT / 32;
 constexpr int WARP_TILE = 128;                           // pixels per warp tile of the TMA kernels
-constexpr int DCHUNK = 4;  // tiles per grab from the shared part of a pass (stored-U whole-run kernel)
-// Issue-side state of one warp's TMA ring in the stored-U whole-run kernel
-// (lane 0 only, kept in shared memory): copies issued, next tile of the chunk being
-// issued, pass, index in the fixed share, ring slot, tiles left in the chunk,
-// and the counter value grabbed for the next chunk.
-struct IssueState {
-    int64_t issued, cb;
-    int ip, ik, is, cl;
-    unsigned grab;
-};
 constexpr int SLOTS_MAX = 2 * FCM_MAX_CLUSTERS + 4;      // num[C], den[C], J, delta, 2 flags
 constexpr int STATUS_RUNNING = 2;
 
@@ -77,33 +67,19 @@ struct alignas(128) RunState {
     unsigned int ticket;  // last-block-done counter of the current pass
     int launches;         // passes started in this run (loop guard)
     WaitLimits lim;
-    // stored-U whole-run kernel: percent of each pass's tiles dealt to the
-    // warps in fixed shares (100: all of them); the rest is taken in chunks from
-    // dyn[pass & 1] (zeroed by the upload of this state, re-zeroed on the
-    // device two passes before each reuse)
-    int static_pct;
-    unsigned int dyn[2];
+    int from_u;           // whole-run kernel: 1 from U^0, 0 from V^0
     unsigned int bounds;  // FCM_FLAG_BOUNDS from a FCM_DEBUG_BOUNDS build's guards
 };
-constexpr int DEFAULT_STATIC_PCT = 60;
 
 typedef void (*PassFn)(RunState*, double*, cudaGraphConditionalHandle, int);
 
 // Kernel table: [C][m kind][pass][variant], variant 0 = grid-stride scalar
 // loads (any n), 1 = TMA ring (n % 4 == 0, 16-byte aligned rows); smem holds
 // each kernel's dynamic shared memory in bytes.
-typedef void (*RunFn)(RunState*, double*);
-
 struct SingleTable {
     PassFn k[FCM_MAX_CLUSTERS + 1][4][P_COUNT][2];
     int smem[FCM_MAX_CLUSTERS + 1][4][P_COUNT][2];
-    // the whole run in one cooperative launch: [C][m kind][0 = from U^0, 1 = from V^0]
-    RunFn run[FCM_MAX_CLUSTERS + 1][4][2];
-    int run_smem[FCM_MAX_CLUSTERS + 1];
 };
-
-// The kernel table, filled on first use.
-const SingleTable& single_table();
 
 void register_single_c1(SingleTable&);
 void register_single_c2(SingleTable&);

@@ -10,10 +10,9 @@
 // that is part of the library image and exists on every GPU that loads the
 // library until the process exits.
 //
-// The scratch holds the device-side run state and the per-block partial sums
-// of the cooperative whole-run kernel (the same kernel fcm_run launches for
-// aligned inputs). Its size is fixed: partial sums for at most
-// FCM_NOALLOC_MAX_BLOCKS thread blocks. Every call shares it, so calls whose
+// The scratch holds the device-side run state and the blocks' exchange slots
+// of the cooperative whole-run kernel (the kernel fcm_run launches). Its size is
+// fixed: slots for at most FCM_NOALLOC_MAX_BLOCKS thread blocks. Every call shares it, so calls whose
 // work overlaps on the GPU (from several host threads, or on several streams
 // without ordering between them) race and give wrong results.
 #include <cuda_runtime.h>
@@ -26,18 +25,19 @@
 #include "fcm.h"
 #include "fcm_device.cuh"
 #include "fcm_internal.h"
+#include "fcm_run.h"
 
 using namespace fcm;
 
 namespace {
 
 constexpr size_t kStateBytes = (sizeof(RunState) + 255) / 256 * 256;
-constexpr size_t kPartialBytes = sizeof(float) * 2 * SLOTS_MAX * FCM_NOALLOC_MAX_BLOCKS;
+constexpr size_t kSlotBytes = (size_t)RUN_SLOT_BYTES * run_slots(FCM_MAX_CLUSTERS) * FCM_NOALLOC_MAX_BLOCKS;
 
-// The scratch: run state, then two buffers of per-block partial sums.
+// The scratch: run state, then the blocks' exchange slots (zero at load).
 // In host code this name is only a stand-in for the device array; its device
 // address comes from cudaGetSymbolAddress, once per device.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kStateBytes + kPartialBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kStateBytes + kSlotBytes];
 
 constexpr int kMaxDevices = 64;
 
@@ -46,8 +46,8 @@ struct DeviceSetup {
     int status = FCM_OK;
     unsigned char* scratch = nullptr;  // device address of g_noalloc_scratch
     int num_sms = 0;
-    // blocks per SM of the whole-run kernel: [C][m kind][from U^0 / from V^0]
-    int bps[FCM_MAX_CLUSTERS + 1][4][2] = {};
+    unsigned nonce = 0;  // number of the last run on this device (the tag of its exchanges)
+    bool fits[FCM_MAX_CLUSTERS + 1][4] = {};  // the whole-run kernel of [C][m kind] can be launched
 };
 
 std::mutex g_mu;
@@ -72,20 +72,16 @@ int setup_device(int dev) {
         cudaGetLastError();
         return d.status = FCM_ERR_CUDA;
     }
-    const SingleTable& t = single_table();
+    const RunTable& t = run_table();
     for (int C = 1; C <= FCM_MAX_CLUSTERS; ++C)
-        for (int mk = 0; mk < 4; ++mk)
-            for (int init = 0; init < 2; ++init) {
-                const void* k = (const void*)t.run[C][mk][init];
-                const int smem = t.run_smem[C];
-                int nb = 0;
-                if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, NT, smem) != cudaSuccess) {
-                    cudaGetLastError();
-                    nb = 0;
-                }
-                d.bps[C][mk][init] = nb;
+        for (int mk = 0; mk < 4; ++mk) {
+            int nb = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)t.run[C][mk], RUN_NT, 0) != cudaSuccess) {
+                cudaGetLastError();
+                nb = 0;
             }
+            d.fits[C][mk] = nb > 0;
+        }
     return d.status = FCM_OK;
 }
 
@@ -134,18 +130,14 @@ extern "C" int fcm_run_noalloc(const float* x, int64_t n, int C, float m, float 
     cudaStream_t stream = (cudaStream_t)cuda_stream;
 
     const int mk = mkind_of(m);
-    const int init = init_mode == FCM_INIT_U ? 0 : 1;
-    const int bps = d.bps[C][mk][init];
-    if (bps < 1) return FCM_ERR_CUDA;
-    const int64_t want = (n + (int64_t)WARP_TILE * NWARP - 1) / ((int64_t)WARP_TILE * NWARP);
-    const int64_t blocks = std::min<int64_t>(want, (int64_t)d.num_sms * bps);
+    if (!d.fits[C][mk]) return FCM_ERR_CUDA;
+    const int blocks = run_grid(n, d.num_sms);
     if (blocks > FCM_NOALLOC_MAX_BLOCKS) return FCM_ERR_TOO_LARGE;
 
     RunState* st = reinterpret_cast<RunState*>(d.scratch);
-    double* partials = reinterpret_cast<double*>(d.scratch + kStateBytes);
+    char* slots = reinterpret_cast<char*>(d.scratch + kStateBytes);
 
-    // A fresh state for every call: the grid-barrier counter and the status
-    // must start at zero; the partial sums are always written before read.
+    // A fresh state for every call: the status must start at running.
     RunState hs;
     std::memset(&hs, 0, sizeof(hs));
     hs.x = x;
@@ -159,17 +151,26 @@ extern "C" int fcm_run_noalloc(const float* x, int64_t n, int C, float m, float 
     hs.C = C;
     hs.status = STATUS_RUNNING;
     hs.lim = WaitLimits{DEFAULT_GRID_SPINS, DEFAULT_TMA_POLLS, 0u, 0u};
-    hs.static_pct = DEFAULT_STATIC_PCT;
+    hs.from_u = init_mode == FCM_INIT_U;
     const bool V_dev = on_device(V);
     if (init_mode == FCM_INIT_V && !V_dev) std::memcpy(hs.V0, V, sizeof(float) * C);
 
     cudaError_t e = cudaMemcpyAsync(st, &hs, sizeof(RunState), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess && init_mode == FCM_INIT_V && V_dev)
         e = cudaMemcpyAsync(&st->V0, V, sizeof(float) * C, cudaMemcpyDeviceToDevice, stream);
+    // the run's number, and zeroed slots when the numbers start over (no slot
+    // then shows a tag of an earlier run of the same number)
+    unsigned nonce;
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        nonce = ++g_dev[dev].nonce;
+        if (nonce == 0) nonce = g_dev[dev].nonce = 1;
+    }
+    if (e == cudaSuccess && nonce == 1) e = cudaMemsetAsync(slots, 0, kSlotBytes, stream);
     if (e == cudaSuccess) {
-        void* args[2] = {&st, &partials};
-        e = cudaLaunchCooperativeKernel((const void*)single_table().run[C][mk][init], dim3((unsigned)blocks),
-                                        dim3(NT), args, single_table().run_smem[C], stream);
+        void* args[3] = {&st, &slots, &nonce};
+        e = cudaLaunchCooperativeKernel((const void*)run_table().run[C][mk], dim3((unsigned)blocks), dim3(RUN_NT), args,
+                                        0, stream);
     }
     RunState out;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&out, st, sizeof(RunState), cudaMemcpyDeviceToHost, stream);

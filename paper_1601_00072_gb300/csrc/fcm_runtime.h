@@ -63,9 +63,6 @@ struct fcm_ctx {
     // run's state; alloc_fail_in > 0 makes the allocation that many calls
     // from now fail once (fault injection for tests, 0 = off)
     fcm::WaitLimits limits{fcm::DEFAULT_GRID_SPINS, fcm::DEFAULT_TMA_POLLS, 0u, 0u};
-    // whole-run kernel: percent of a pass's tiles dealt in fixed warp shares
-    // (FCM_RUN_STATIC_PCT in the environment overrides it, 1..100)
-    int static_pct = fcm::DEFAULT_STATIC_PCT;
     int alloc_fail_in = 0;
 
     // single-image path
@@ -74,6 +71,8 @@ struct fcm_ctx {
     int h_done = 0;
     double* d_partials = nullptr;
     int partial_blocks = 0;
+    char* d_slots = nullptr;    // whole-run kernel's exchange slots, behind the partials
+    unsigned run_nonce = 0;     // number of the handle's last whole run
     double* d_trace = nullptr;
     size_t trace_cap = 0;
     int last_trace_iters = 0;

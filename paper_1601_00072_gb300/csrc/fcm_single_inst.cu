@@ -29,11 +29,8 @@
 // block order, forms V^{k+1}, decides convergence on the device (the paper
 // does this on the host, Sec. 4.3) and sets the CUDA-graph WHILE condition.
 // No block waits for another: the ticket only elects the finisher.
-#include <climits>
-
 #include "fcm_bounds.cuh"
 #include "fcm_device.cuh"
-#include "fcm_exchange.cuh"
 #include "fcm_internal.h"
 #include "fcm_tma.cuh"
 
@@ -488,362 +485,6 @@ __global__ void __launch_bounds__(NT, 2) k_fcm_pass_tma(RunState* __restrict__ s
     finish_pass<C, PASS>(st, partials, cond, use_cond, a.num, a.den, a.J, a.dmax, a.bad, tmo);
 }
 
-// ---------------------------------------------------------------------------
-// The whole run in one cooperative launch (n % 4 == 0, aligned rows).
-// ---------------------------------------------------------------------------
-
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// The grid barrier polls at most st->lim.grid_spins times, 128 ns apart
-// (2^23, about 1 s, by default), and waits for st->lim.phantoms arrivals
-// beyond the grid's own (0 unless a test injects a barrier that never fills).
-
-// Tiles are dealt in two parts. Every warp keeps the same fixed share of tiles
-// in every pass (tile gw + k * nwarps, k < ks), so the U tile it reads from
-// that share in pass p + 1 is one it wrote itself in pass p. Its ring
-// therefore streams one sequence of loads across passes (a proxy fence orders
-// the warp's stores before its own TMA re-read) and keeps DRAM busy while the
-// grid exchanges the 2C + 4 sums of a pass. The rest of each pass is taken in
-// chunks of DCHUNK consecutive tiles from a per-pass counter, so warps on SMs
-// that stream faster take more of it and the warps finish a pass together
-// (with fixed shares alone, the slowest SMs took about 1.5x as long as the
-// fastest). A warp reaches the shared part of pass p only after its fixed
-// share of pass p, which it starts after the grid barrier of pass p - 1, so
-// every tile it takes was written before that barrier. The counter grab is
-// issued one chunk ahead, so its latency hides behind the chunk's copies. After each pass every block
-// publishes its FP32 totals, waits at a bounded grid barrier (co-residency is
-// guaranteed by the cooperative launch), and computes the cross-block sums in
-// the same fixed order as every other block, so all blocks derive the same
-// V^{k+1} and the same stop decision. Pass 0 is INIT (V^1 from U^0, or U^0
-// from V^0); pass p >= 1 is iteration p of Algorithm 1.
-template <int C, int MK, int INIT>
-__global__ void __launch_bounds__(NT, 2) k_fcm_run_tma(RunState* __restrict__ st,
-                                                                      double* __restrict__ partials_raw) {
-    using Sh = TmaShape<P_ITER, C>;
-    constexpr int S = 2 * C + 4;
-    extern __shared__ __align__(128) float ring_all[];
-    __shared__ __align__(8) uint64_t full_all[NWARP][Sh::STAGES];
-    __shared__ float s_red[NWARP][S];
-    __shared__ DF s_df[2 * C + 1];
-    __shared__ float s_mx[3];
-    __shared__ DF s_vq[C];
-    __shared__ int s_empty[C];
-    __shared__ int s_err;
-    // what each ring stage holds: tile and pass (pass INT_MAX: nothing)
-    __shared__ int64_t s_tile[NWARP][Sh::STAGES];
-    __shared__ int s_pass[NWARP][Sh::STAGES];
-    __shared__ IssueState s_iss[NWARP];
-
-    const float* __restrict__ x = st->x;
-    const float* U0 = st->Uprev;
-    float* U = st->U;
-    const int64_t n = st->n;
-    const float m = st->m, inv_m1 = st->inv_m1, eps = st->eps;
-    const int max_iter = st->max_iter;
-    unsigned* gbar = &st->ticket;
-    float* partials = reinterpret_cast<float*>(partials_raw);
-
-    float v[C];
-    f2 v2[C];
-    DF v64[C];  // the double-float quotients behind v, converted to FP64 only when written
-#pragma unroll
-    for (int j = 0; j < C; ++j) {
-        v[j] = st->V0[j];
-        v2[j] = pack2(v[j], v[j]);
-        v64[j] = DF{v[j], 0.0f};
-    }
-    int flags = 0;
-
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float* ring = ring_all + warp * (Sh::STAGES * Sh::STAGE_FLOATS);
-    uint64_t* full = full_all[warp];
-    const int64_t nwarps = (int64_t)gridDim.x * NWARP;
-    const int64_t gw = (int64_t)blockIdx.x * NWARP + warp;
-    const int64_t ntiles = (n + WTILE - 1) / WTILE;
-    // fixed share: ks tiles per warp, when every warp has more than a ring of
-    // them; otherwise every tile is dealt in fixed shares (nk per warp)
-    const int64_t ks = ntiles * (int64_t)st->static_pct / 100 / nwarps;
-    const bool shared_part = st->static_pct < 100 && ks > Sh::STAGES;
-    const int nk = shared_part ? (int)ks : (int)(ntiles > gw ? (ntiles - 1 - gw) / nwarps + 1 : 0);
-    const int64_t n_fixed = shared_part ? ks * nwarps : ntiles;
-    const int64_t n_chunks = (ntiles - n_fixed + DCHUNK - 1) / DCHUNK;
-    const int look = nk < Sh::STAGES ? nk : Sh::STAGES;
-    const int npass = 1 + max_iter;  // passes the run can take
-    const uint32_t wait_limit = st->lim.tma_polls, grid_spins = st->lim.grid_spins;
-    const unsigned phantoms = st->lim.phantoms;
-    const uint64_t pol_x = policy_evict_last();
-    const uint64_t pol_u = policy_evict_first();
-
-    if (lane == 0) {
-#pragma unroll
-        for (int s = 0; s < Sh::STAGES; ++s) {
-            mbar_init(&full[s], 1);
-            s_pass[warp][s] = INT_MAX;
-        }
-        mbar_fence_init();
-    }
-    if (threadIdx.x == 0) s_err = 0;
-    __syncthreads();
-
-    // Issue side (lane 0), kept in shared memory so that it takes no
-    // registers during the tile work: pass ip, index ik in the fixed share,
-    // the chunk being issued (next tile cb, cl tiles left), the grab for the
-    // next chunk, ring slot is, and the copies issued so far.
-    IssueState& q = s_iss[warp];
-    if (lane == 0) q = IssueState{0, 0, 0, 0, 0, 0, 0u};
-    auto issue_tile = [&](int64_t tile, int ip) {
-        const int64_t i0 = tile * WTILE;
-        const uint32_t bytes = (uint32_t)min((int64_t)WTILE, n - i0) * 4u;  // multiple of 16
-        const bool with_u = !(ip == 0 && INIT == P_INITV);
-        const float* Usrc = (ip == 0 || (ip == 1 && INIT == P_ACCUM0)) ? U0 : U;
-        const int is = q.is;
-        float* dst = ring + is * Sh::STAGE_FLOATS;
-        s_pass[warp][is] = ip;
-        if (!in_bounds(tile >= 0 && tile < ntiles && is < Sh::STAGES, &st->bounds)) {
-            s_tile[warp][is] = -1;  // the consumer skips it
-            mbar_expect_tx(&full[is], 0u);  // arrive without copies
-            ++q.issued;
-            q.is = is + 1 == Sh::STAGES ? 0 : is + 1;
-            return;
-        }
-        s_tile[warp][is] = tile;
-        mbar_expect_tx(&full[is], bytes * (with_u ? 1 + C : 1));
-        bulk_g2s(dst, x + i0, bytes, &full[is], pol_x);
-        if (with_u) {
-#pragma unroll
-            for (int j = 0; j < C; ++j)
-                bulk_g2s(dst + (1 + j) * WTILE, Usrc + (int64_t)j * n + i0, bytes, &full[is], pol_u);
-        }
-        ++q.issued;
-        q.is = is + 1 == Sh::STAGES ? 0 : is + 1;
-    };
-    auto issue_next = [&]() {
-        while (q.ip < npass && nk > 0) {
-            const int ip = q.ip;
-            if (q.ik < nk) {
-                const int64_t tile = gw + (int64_t)q.ik * nwarps;
-                if (++q.ik == nk && shared_part) q.grab = atomicAdd(&st->dyn[ip & 1], 1u);  // first chunk, ahead
-                issue_tile(tile, ip);
-                return;
-            }
-            if (q.cl == 0) {
-                if (shared_part && (int64_t)q.grab < n_chunks) {
-                    q.cb = n_fixed + (int64_t)q.grab * DCHUNK;
-                    q.cl = (int)min((int64_t)DCHUNK, ntiles - q.cb);
-                    q.grab = atomicAdd(&st->dyn[ip & 1], 1u);  // the chunk after this one, ahead
-                } else {
-                    ++q.ip;  // pass ip is dealt out: on to the next pass's fixed share
-                    q.ik = 0;
-                    continue;
-                }
-            }
-            --q.cl;
-            issue_tile(q.cb++, ip);
-            return;
-        }
-        s_pass[warp][q.is] = INT_MAX;  // nothing more to load
-    };
-    if (lane == 0)
-        for (int t = 0; t < look; ++t) issue_next();
-    __syncwarp();
-
-    int cs = 0;  // consume side: ring slot and phase parity
-    uint32_t parity = 0;
-    int64_t consumed = 0;
-    bool stop = false, err = false;
-    int status = FCM_NOT_CONVERGED, iters = 0;
-    Acc<C> a;
-
-    for (int p = 0; !stop; ++p) {
-        a.reset();
-        if (p == 0 && INIT == P_INITV) {
-#pragma unroll
-            for (int j = 0; j < C; ++j) a.bad |= !finite_f(v[j]);
-        }
-        // ---- the pass over this warp's tiles: the ring's items of pass p ----
-        while (s_pass[warp][cs] == p) {
-            const bool ok = mbar_wait_bounded(&full[cs], parity, wait_limit);
-            if (__any_sync(0xffffffffu, !ok)) {
-                err = true;
-                break;
-            }
-            const int64_t tile = s_tile[warp][cs];
-            const int64_t i0 = tile * WTILE;
-            const int cnt = (int)min((int64_t)WTILE, n - i0);
-            const float* sb = ring + cs * Sh::STAGE_FLOATS;
-            if (kBoundsChecks && tile < 0) {
-                // a copy the guards skipped: nothing to compute or store
-            } else if (p == 0) {
-                tile_work<C, MK, INIT>(sb, cnt, i0, lane, U, n, v, v2, m, inv_m1, pol_u, a);
-            } else {
-                tile_work<C, MK, P_ITER>(sb, cnt, i0, lane, U, n, v, v2, m, inv_m1, pol_u, a);
-            }
-            // this lane's stores of U must precede any TMA re-read of the tile:
-            // the warp's own (fixed share, next pass) or another warp's after
-            // the grid barrier (shared part)
-            asm volatile("fence.proxy.async.global;" ::: "memory");
-            __syncwarp();
-            ++consumed;
-            if (lane == 0) issue_next();
-            __syncwarp();  // the stage records written by lane 0
-            if (++cs == Sh::STAGES) {
-                cs = 0;
-                parity ^= 1u;
-            }
-        }
-        if (!(p == 0 && INIT == P_ACCUM0)) a.fold();
-
-        // ---- block totals (FP32 over the 8 warps) -> partials[p & 1] ----
-        {
-            float vals[S];
-#pragma unroll
-            for (int j = 0; j < C; ++j) {
-                vals[j] = a.num[j];
-                vals[C + j] = a.den[j];
-            }
-            vals[2 * C] = a.J;
-            vals[2 * C + 1] = a.dmax;
-            vals[2 * C + 2] = a.bad ? 1.0f : 0.0f;
-            vals[2 * C + 3] = err ? 1.0f : 0.0f;
-#pragma unroll
-            for (int s = 0; s < S; ++s) vals[s] = (s <= 2 * C) ? warp_sum(vals[s]) : warp_max(vals[s]);
-            if (lane == 0) {
-#pragma unroll
-                for (int s = 0; s < S; ++s) s_red[warp][s] = vals[s];
-            }
-        }
-        __syncthreads();
-        float* part = partials + (int64_t)(p & 1) * S * gridDim.x;
-        if (threadIdx.x < S) {
-            const int s = threadIdx.x;
-            float t = s_red[0][s];
-#pragma unroll
-            for (int w = 1; w < NWARP; ++w) t = (s <= 2 * C) ? t + s_red[w][s] : fmaxf(t, s_red[w][s]);
-            __stcg(part + (int64_t)s * gridDim.x + blockIdx.x, t);
-        }
-        __syncthreads();
-        // ---- bounded grid barrier ----
-        if (threadIdx.x == 0) {
-            __threadfence();
-            atomicAdd(gbar, 1u);
-            const unsigned target = (unsigned)(p + 1) * gridDim.x + phantoms;
-            uint32_t spins = 0;
-            while (ld_acquire_u32(gbar) < target) {
-                if (++spins > grid_spins) {
-                    s_err = 1;
-                    break;
-                }
-                __nanosleep(128);
-            }
-            __threadfence();
-        }
-        __syncthreads();
-        if (s_err) {
-            status = FCM_ERR_TIMEOUT;
-            iters = p;
-            break;
-        }
-        // ---- cross-block sums and V^{p+1}, the same fixed order in every block ----
-        grid_totals<S, 2 * C + 1, NWARP>(part, (int)gridDim.x, s_df, s_mx);
-        __syncthreads();
-        grid_centers<C>(s_df, s_vq, s_empty);
-        __syncthreads();
-        const float delta = s_mx[0];
-        const bool bad = s_mx[1] != 0.0f, tmo = s_mx[2] != 0.0f;
-        // the loads this warp issues from here on may read U tiles that other
-        // warps wrote before the barrier
-        if (lane == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
-        // every chunk of pass p was taken before this barrier; its counter
-        // serves pass p + 2, whose first grab follows the next barrier
-        if (blockIdx.x == 0 && threadIdx.x == 0) st->dyn[p & 1] = 0u;
-        bool update = false;
-        if (tmo) {
-            status = FCM_ERR_TIMEOUT;
-            iters = p;
-            stop = true;
-        } else if (p == 0) {
-            if (bad) {
-                status = FCM_ERR_BAD_INPUT;
-                iters = 0;
-                stop = true;
-            } else {
-                update = true;
-            }
-        } else {
-            if (blockIdx.x == 0 && threadIdx.x == 0 && st->trace) {
-                double* t = st->trace + (int64_t)(p - 1) * (2 + C);
-                t[0] = delta;
-                t[1] = df_to_double(s_df[2 * C]);
-#pragma unroll
-                for (int j = 0; j < C; ++j) t[2 + j] = df_to_double(v64[j]);
-            }
-            if (delta < eps) {
-                status = FCM_OK;
-                iters = p;
-                stop = true;
-            } else if (p >= max_iter) {
-                status = FCM_NOT_CONVERGED;
-                iters = p;
-                stop = true;
-            } else {
-                update = true;
-            }
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                st->delta = delta;
-                st->J = df_to_double(s_df[2 * C]);
-            }
-        }
-        if (update) {
-#pragma unroll
-            for (int j = 0; j < C; ++j) {
-                if (s_empty[j]) {
-                    // an empty cluster keeps its center (first pass: V^0, or 0 from a U^0)
-                    flags |= FCM_FLAG_EMPTY_CLUSTER;
-                    if (p == 0 && INIT == P_ACCUM0) {
-                        v[j] = 0.0f;
-                        v64[j] = DF{0.0f, 0.0f};
-                    }
-                } else {
-                    v[j] = s_vq[j].hi;
-                    v64[j] = s_vq[j];
-                }
-                v2[j] = pack2(v[j], v[j]);
-            }
-        }
-        __syncthreads();  // s_df / s_vq are rewritten by the next pass
-    }
-
-    // copies issued for passes that will not run: let them land
-    if (lane == 0) {
-        int ds = cs;
-        uint32_t dp = parity;
-        for (int64_t t = consumed; t < q.issued; ++t) {
-            mbar_wait_bounded(&full[ds], dp, wait_limit);
-            if (++ds == Sh::STAGES) {
-                ds = 0;
-                dp ^= 1u;
-            }
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            st->V[j] = v[j];
-            st->V64[j] = df_to_double(v64[j]);
-        }
-        st->status = status;
-        st->iters = iters;
-        st->k = iters;
-        st->flags = flags;
-        st->done = 1;
-        st->Uprev = st->U;
-    }
-}
-
 template <int C, int MK, int PASS>
 void fill_pass(SingleTable& t) {
     t.k[C][MK][PASS][0] = k_fcm_pass_ldg<C, MK, PASS>;
@@ -857,9 +498,6 @@ void fill_mk(SingleTable& t) {
     fill_pass<C, MK, P_ACCUM0>(t);
     fill_pass<C, MK, P_INITV>(t);
     fill_pass<C, MK, P_ITER>(t);
-    t.run[C][MK][0] = k_fcm_run_tma<C, MK, P_ACCUM0>;
-    t.run[C][MK][1] = k_fcm_run_tma<C, MK, P_INITV>;
-    t.run_smem[C] = TmaShape<P_ITER, C>::SMEM_BYTES;
 }
 
 }  // namespace

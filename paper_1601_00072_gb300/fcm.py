@@ -174,11 +174,10 @@ class FCM:
         Start from memberships: ``U0`` [C, n] (read only), or no ``U0`` and
         ``U`` holding U^0 (updated in place). Start from centers: ``V0`` [C].
         ``U`` (allocated when None) receives U^k and ``V`` (allocated when
-        None, or V0 itself) receives V^k. ``recompute=True`` keeps no U
-        between iterations (``FCM_OPT_RECOMPUTE``). ``deterministic=True``
-        deals every tile of the whole-run kernel in fixed warp shares, so
-        large images give bit-identical results run after run
-        (``FCM_OPT_DETERMINISTIC``).
+        None, or V0 itself) receives V^k. ``recompute=True`` insists on the
+        launch that keeps no U between iterations (``FCM_OPT_RECOMPUTE``).
+        ``deterministic=True`` asks for bit-identical results run after run
+        (``FCM_OPT_DETERMINISTIC``; every run gives them).
         """
         import torch
         n = _numel(x)
