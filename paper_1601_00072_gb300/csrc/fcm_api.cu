@@ -88,15 +88,35 @@ const RunTable& run_table() {
     return g_run;
 }
 
-// Every thread of the whole-run kernel takes four pixels at a time: the fewest
-// blocks that keep the largest number of such steps per thread that max_blocks
-// would give, so the threads hold about the same number of pixels (a 1 M-pixel
-// image: 128 blocks with 4 steps each; 152 blocks would also need 4).
-int run_grid(int64_t n, int64_t max_blocks) {
-    if (max_blocks < 1) return 0;
+bool run_kernel_fits(const void* k, int C) {
+    const int pt = run_max_pt(C), smem = run_smem(C, pt, run_max_resident(C, pt));
+    int nb = 0;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, pt + 32, smem) != cudaSuccess) {
+        cudaGetLastError();
+        nb = 0;
+    }
+    return nb > 0;
+}
+
+// A pixel thread takes a quad of pixels per step. A large image fills every SM
+// with the most pixel threads: the fewest blocks that keep the largest number of
+// steps that max_blocks would give (a 1 M-pixel image: 137 blocks with 4 steps;
+// 152 would also need 4). A small one, a single step of which would not fill the
+// SMs, is spread over them with fewer threads each, at least RUN_FEW_PT (and one
+// warp per cluster, for the exchange).
+RunShape run_shape(int64_t n, int C, int64_t max_blocks) {
+    if (max_blocks < 1) return RunShape{0, 0, 0, 0};
     const int64_t quads = (n + 3) / 4;
-    const int64_t steps = (quads + max_blocks * RUN_NT - 1) / (max_blocks * RUN_NT);
-    return (int)std::max<int64_t>(1, (quads + steps * RUN_NT - 1) / (steps * RUN_NT));
+    int64_t pt = run_max_pt(C);
+    const int64_t steps = (quads + max_blocks * pt - 1) / (max_blocks * pt);
+    if (steps == 1) {
+        const int64_t even = (quads + max_blocks - 1) / max_blocks;
+        pt = std::min<int64_t>(pt, std::max<int64_t>(std::max(RUN_FEW_PT, 32 * C), (even + 31) / 32 * 32));
+    }
+    const int64_t blocks = std::max<int64_t>(1, (quads + steps * pt - 1) / (steps * pt));
+    const int resident = (int)std::min<int64_t>((quads + blocks * pt - 1) / (blocks * pt), run_max_resident(C, (int)pt));
+    return RunShape{(int)blocks, (int)pt + 32, resident, run_smem(C, (int)pt, resident)};
 }
 
 int ctx_fail(fcm_ctx* h, cudaError_t e, const char* what) {
@@ -161,9 +181,7 @@ int ctx_grow(fcm_ctx* h, void** p, size_t* cap, size_t bytes, const char* what) 
 
 namespace {
 
-size_t run_slot_bytes(const fcm_ctx* h) {
-    return (size_t)RUN_SLOT_BYTES * run_slots(FCM_MAX_CLUSTERS) * h->num_sms;
-}
+int max_run_sms(const fcm_ctx* h) { return std::min(h->num_sms, RUN_MAX_BLOCKS); }
 
 // Each buffer is allocated when missing, so a call after a failed allocation
 // completes the workspace.
@@ -174,42 +192,37 @@ int ensure_single_workspace(fcm_ctx* h) {
     }
     if (!h->h_st) CK(host_malloc(h, &h->h_st, sizeof(RunState)));
     if (!h->d_partials) {
-        // the pass kernels' partials, then the exchange slots of the whole-run
-        // kernel, zero before its first run (no tag is 0)
+        // the pass kernels' partials, then the exchange scratch of the whole-run
+        // kernel, zero before its first run
         h->partial_blocks = h->num_sms * 32;
         const size_t bytes = sizeof(double) * SLOTS_MAX * h->partial_blocks;
-        CK(dev_malloc(h, &h->d_partials, bytes + run_slot_bytes(h)));
+        CK(dev_malloc(h, &h->d_partials, bytes + run_scratch_bytes(max_run_sms(h))));
         h->d_slots = reinterpret_cast<char*>(h->d_partials) + bytes;
-        h->run_nonce = 0xffffffffu;  // the first run zeroes the slots
+        h->run_nonce = 0xffffffffu;  // the first run zeroes the scratch
     }
     return 0;
 }
 
 // The number of the next whole run of the handle: the upper half of its
-// exchanges' tags. The slots are zeroed when the numbers start over, so no slot
-// can show a tag of an earlier run of the same number.
+// exchanges' tags, and which bank of words it uses. The scratch is zeroed when
+// the numbers start over, so no slot can show a tag of an earlier run of the
+// same number.
 int next_nonce(fcm_ctx* h, unsigned* nonce) {
     if (++h->run_nonce == 0) {
-        CK(cudaMemsetAsync(h->d_slots, 0, run_slot_bytes(h), h->stream));
-        h->run_nonce = 1;
+        CK(cudaMemsetAsync(h->d_slots, 0, run_scratch_bytes(max_run_sms(h)), h->stream));
+        h->run_nonce = 2;  // even, as 0: the banks go on alternating
     }
     *nonce = h->run_nonce;
     return 0;
 }
 
 // Co-resident blocks of the whole-run kernel (one per SM), or 0 when it does
-// not fit.
-int64_t max_run_blocks(fcm_ctx* h, const void* k) {
+// not fit; the first call also raises the kernel's dynamic shared memory limit.
+int64_t max_run_blocks(fcm_ctx* h, const void* k, int C) {
     auto it = h->occupancy.find(k);
-    if (it == h->occupancy.end()) {
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, RUN_NT, 0) != cudaSuccess) {
-            cudaGetLastError();
-            nb = 0;
-        }
-        it = h->occupancy.emplace(k, nb).first;
-    }
-    return it->second > 0 ? h->num_sms : 0;
+    if (it == h->occupancy.end())
+        it = h->occupancy.emplace(k, run_kernel_fits(k, C) ? 1 : 0).first;
+    return it->second ? max_run_sms(h) : 0;
 }
 
 // Blocks per SM of a pass kernel with `smem` bytes of dynamic shared memory;
@@ -529,20 +542,26 @@ int fcm_run(fcm_handle h, const float* x, int64_t n, int C, float m, float eps, 
     const int pass0 = init_mode == FCM_INIT_U ? P_ACCUM0 : P_INITV;
     const bool aligned = (n % 4 == 0) && ((uintptr_t)dx % 16 == 0) && ((uintptr_t)dU % 16 == 0) &&
                          ((uintptr_t)hs->Uprev % 16 == 0);
-    int run_blocks = 0;
+    RunShape shape{0, 0, 0, 0};
     const bool recompute = (options & FCM_OPT_RECOMPUTE) != 0;
     const void* krun = (const void*)g_run.run[C][mk];
     if (recompute && !(aligned && h->coop))
         return ctx_invalid(h, "FCM_OPT_RECOMPUTE needs n % 4 == 0, 16-byte-aligned rows and cooperative launch");
     if (recompute || (h->coop && !(options & (FCM_OPT_NO_TMA | FCM_OPT_NO_PERSISTENT | FCM_OPT_NO_GRAPH))))
-        run_blocks = run_grid(n, max_run_blocks(h, krun));
-    if (run_blocks > 0) {
+        shape = run_shape(n, C, max_run_blocks(h, krun, C));
+    if (shape.blocks > 0) {
         // the whole run: one cooperative launch (all blocks co-resident)
         unsigned nonce;
         if ((rc = next_nonce(h, &nonce))) return rc;
-        void* args[3] = {&h->d_st, &h->d_slots, &nonce};
-        CK(cudaLaunchCooperativeKernel(krun, dim3(run_blocks), dim3(RUN_NT), args, 0, h->stream));
-        h->last_blocks = run_blocks;
+        int resident = shape.resident;
+        void* args[4] = {&h->d_st, &h->d_slots, &nonce, &resident};
+        const cudaError_t le =
+            cudaLaunchCooperativeKernel(krun, dim3(shape.blocks), dim3(shape.threads), args, shape.smem, h->stream);
+        if (le != cudaSuccess) {
+            h->run_nonce = 0xffffffffu;  // the number was not used: the next run zeroes the scratch
+            return ctx_fail(h, le, "launching the whole run");
+        }
+        h->last_blocks = shape.blocks;
         h->last_path = 2;
     } else {
     Launch L;
@@ -639,8 +658,8 @@ int fcm_run_stream(fcm_handle h, int n_images, const float* const* x, int64_t n,
 
     const int mk = mkind_of(m);
     const void* krun = (const void*)g_run.run[C][mk];
-    const int run_blocks = run_grid(n, max_run_blocks(h, krun));
-    if (run_blocks < 1) return ctx_invalid(h, "the whole-run kernel does not fit on this device");
+    const RunShape shape = run_shape(n, C, max_run_blocks(h, krun, C));
+    if (shape.blocks < 1) return ctx_invalid(h, "the whole-run kernel does not fit on this device");
 
     // the copy streams start behind the work already queued on the handle's stream
     CK(cudaEventRecord(ev_start, h->stream));
@@ -677,9 +696,11 @@ int fcm_run_stream(fcm_handle h, int n_images, const float* const* x, int64_t n,
         if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_st, hs, sizeof(RunState), cudaMemcpyHostToDevice, h->stream);
         unsigned nonce = 0;
         if (e == cudaSuccess && next_nonce(h, &nonce)) e = cudaErrorUnknown;
-        void* args[3] = {&h->d_st, &h->d_slots, &nonce};
+        int resident = shape.resident;
+        void* args[4] = {&h->d_st, &h->d_slots, &nonce, &resident};
         if (e == cudaSuccess)
-            e = cudaLaunchCooperativeKernel(krun, dim3(run_blocks), dim3(RUN_NT), args, 0, h->stream);
+            e = cudaLaunchCooperativeKernel(krun, dim3(shape.blocks), dim3(shape.threads), args, shape.smem, h->stream);
+        if (e != cudaSuccess) h->run_nonce = 0xffffffffu;  // a number may not have been used
         if (e == cudaSuccess) e = cudaMemcpyAsync(hs, h->d_st, sizeof(RunState), cudaMemcpyDeviceToHost, h->stream);
         if (e == cudaSuccess) e = cudaEventRecord(run_done[b], h->stream);
         // download
@@ -701,7 +722,7 @@ int fcm_run_stream(fcm_handle h, int n_images, const float* const* x, int64_t n,
     }
     if (e != cudaSuccess) return ctx_fail(h, e, what);
 
-    h->last_blocks = run_blocks;
+    h->last_blocks = shape.blocks;
     h->last_path = 2;
     h->last_C = C;
     h->last_trace_iters = 0;

@@ -259,37 +259,43 @@ __device__ __forceinline__ f2 membership_pair(f2 x2, const f2 (&v2)[C], float m,
 }
 
 // ---------------------------------------------------------------------------
-// u^m alone, for passes that only add up Eq. 3's sums.
+// Two pixels at once for every fuzzifier, u^m alone (the passes that only add
+// up Eq. 3's sums) or u with the J terms. The scalar weight form above is called,
+// not inlined, for the rare pair that the packed forms cannot take: the packed
+// code keeps its registers and stays small.
 // ---------------------------------------------------------------------------
 
-// u^m of two pixels by the scalar weight form, for the pairs that the packed
-// forms below cannot take. Not inlined: it is rare, and the packed loop keeps
-// its registers.
 template <int C>
-struct Powers {
-    float a[C], b[C];
+struct PixelPair {
+    float a[C], b[C];  // u^m or u of the two pixels
+    float Ja, Jb;
 };
-template <int C, int MK>
-__device__ __noinline__ Powers<C> powers_scalar(float xa, float xb, const float* vs, float m, float inv_m1) {
-    float v[C], u[C];
-    Powers<C> w;
+template <int C, int MK, bool POWERS>
+__device__ __noinline__ PixelPair<C> scalar_pair(float xa, float xb, const float* vs, float m, float inv_m1) {
+    float v[C], t[C];
+    PixelPair<C> w;
 #pragma unroll
     for (int j = 0; j < C; ++j) v[j] = vs[j];
-    membership<C, MK>(xa, v, m, inv_m1, u, w.a);
-    membership<C, MK>(xb, v, m, inv_m1, u, w.b);
+    if (POWERS) {
+        w.Ja = membership<C, MK>(xa, v, m, inv_m1, t, w.a);
+        w.Jb = membership<C, MK>(xb, v, m, inv_m1, t, w.b);
+    } else {
+        w.Ja = membership<C, MK>(xa, v, m, inv_m1, w.a, t);
+        w.Jb = membership<C, MK>(xb, v, m, inv_m1, w.b, t);
+    }
     return w;
 }
 
 // Power-of-two factor that brings the centers' spread to [1, 2), for the
-// products of powers_pair at m = 1.5 (1 when the spread is 0 or extreme).
-// Scaling by it is exact, so it changes the products' range and nothing else.
+// products at m = 1.5 (1 when the spread is 0 or extreme). Scaling by it is
+// exact, so it changes the products' range and nothing else.
 template <int C>
-__device__ __forceinline__ float spread_scale(const f2 (&v2)[C]) {
-    float lo = lo2(v2[0]), hi = lo;
+__device__ __forceinline__ float spread_scale(const float* v) {
+    float lo = v[0], hi = lo;
 #pragma unroll
     for (int j = 1; j < C; ++j) {
-        lo = fminf(lo, lo2(v2[j]));
-        hi = fmaxf(hi, lo2(v2[j]));
+        lo = fminf(lo, v[j]);
+        hi = fmaxf(hi, v[j]);
     }
     const int e = (__float_as_int(hi - lo) >> 23) - 127;
     return (e < -60 || e > 60) ? 1.0f : __int_as_float((127 - e) << 23);
@@ -311,76 +317,178 @@ __device__ __forceinline__ void co_products(const f2 (&b)[C], f2 (&P)[C]) {
     for (int j = 0; j < C; ++j) P[j] = (j == 0) ? suf[0] : (j == C - 1) ? pre[C - 1] : mul2(pre[j], suf[j]);
 }
 
-// True when a is a normal positive float (not 0, subnormal, infinite or NaN).
-__device__ __forceinline__ bool normal_pos(float a) {
-    return (unsigned)(__float_as_int(a) - 0x00800000) < 0x7f000000u;
-}
+// What the packed forms read of the centers: the centers themselves in memory
+// (vs, for the scalar form), and as the differences use them (v2; at m = 1.5
+// times the power of two `scale`, see spread_scale).
+template <int C, int MK>
+struct PackedCenters {
+    f2 v2[C], scale;
+    const float* vs;
+    static constexpr bool SCALED = MK == M_ONE_HALF;
+    __device__ __forceinline__ void set(const float* v) {
+        vs = v;
+        float s = 1.0f;
+        if (SCALED) {
+            s = spread_scale<C>(v);
+            scale = pack2(s, s);
+        }
+#pragma unroll
+        for (int j = 0; j < C; ++j) v2[j] = pack2(v[j] * s, v[j] * s);
+    }
+    __device__ __forceinline__ f2 of(f2 x) const { return SCALED ? mul2(x, scale) : x; }
+};
 
-// um2[j] = u_j^m and d2[j] = x - v_j of two pixels (packed x2). vs: the C
-// centers in memory, for the scalar form. vq2, xs: the centers and the pair as
-// the differences d2 use them (scaled by spread_scale at m = 1.5, unscaled
-// otherwise).
+// N pairs at once (N = 1 or 2: two pairs share one test for the scalar form, and
+// their chains overlap). POWERS: w2[j] = u_j^m of each pair, and d2[j] = x - v_j
+// (scaled). Otherwise w2[j] = u_j, and J2 each pair's J terms.
 //   m = 2, 3  the product form of membership_pair.
-//   m = 1.5   with p_j = prod_{k != j} d_k^2, sqrt(u_j) = p_j / sqrt(sum_k
-//             p_k^2): one reciprocal square root per pixel where the weight form
-//             takes C reciprocals and C square roots; u^1.5 is its cube.
+//   m = 1.5   for u^m, with p_j = prod_{k != j} d_k^2: sqrt(u_j) = p_j / sqrt(
+//             sum_k p_k^2), one reciprocal square root per pixel where the weight
+//             form takes C reciprocals and C square roots; u^1.5 is its cube.
+//             The products' roundings average out in the sums, but not in a
+//             pixel's u (at C = 8 up to 7e-7, against 2e-7): u itself takes the
+//             weight form, w_j = (d2min / d2_j)^2.
 //   other m   w_j = 2^t_j, t_j = (log2 d2min - log2 d2_j) / (m - 1), S = sum w:
 //             u_j^m = 2^(m (t_j - log2 S)), without the C logarithms of u_j.
-template <int C, int MK>
-__device__ __forceinline__ void powers_pair(f2 x2, f2 xs, const f2 (&vq2)[C], float m, float inv_m1,
-                                            const float* vs, f2 (&um2)[C], f2 (&d2)[C]) {
+template <int C, int MK, bool POWERS, int N>
+__device__ __forceinline__ void packed_pairs(const f2 (&x2)[N], const PackedCenters<C, MK>& c, float m, float inv_m1,
+                                             f2 (&w2)[N][C], f2 (&d2)[N][C], f2 (&J2)[N]) {
 #pragma unroll
-    for (int j = 0; j < C; ++j) d2[j] = sub2(xs, vq2[j]);
-    if (MK == M_TWO || MK == M_THREE || MK == M_ONE_HALF) {
-        f2 b[C], P[C];
+    for (int p = 0; p < N; ++p) {
+        const f2 xs = c.of(x2[p]);
 #pragma unroll
-        for (int j = 0; j < C; ++j) b[j] = (MK == M_THREE) ? abs2(d2[j]) : mul2(d2[j], d2[j]);
-        co_products<C>(b, P);
-        f2 S = (MK == M_ONE_HALF) ? mul2(P[0], P[0]) : P[0];
+        for (int j = 0; j < C; ++j) d2[p][j] = sub2(xs, c.v2[j]);
+    }
+    if (MK == M_ONE_HALF && !POWERS) {
+        float mn[2 * N], low = __int_as_float(0x7f800000);
+        f2 b[N][C];
 #pragma unroll
-        for (int j = 1; j < C; ++j) S = (MK == M_ONE_HALF) ? fma2(P[j], P[j], S) : add2(S, P[j]);
-        float s0, s1;
-        unpack2(S, s0, s1);
-        if (normal_pos(s0) && normal_pos(s1)) {
-            const f2 r = (MK == M_ONE_HALF) ? pack2(rsqrt_approx(s0), rsqrt_approx(s1))
-                                            : pack2(rcp_approx(s0), rcp_approx(s1));
+        for (int p = 0; p < N; ++p) {
+            mn[2 * p] = mn[2 * p + 1] = __int_as_float(0x7f800000);
 #pragma unroll
             for (int j = 0; j < C; ++j) {
-                const f2 u = mul2(P[j], r);
-                um2[j] = mul2(u, u);
-                if (MK != M_TWO) um2[j] = mul2(um2[j], u);
+                b[p][j] = mul2(d2[p][j], d2[p][j]);
+                mn[2 * p] = fminf(mn[2 * p], lo2(b[p][j]));
+                mn[2 * p + 1] = fminf(mn[2 * p + 1], hi2(b[p][j]));
+            }
+            low = fminf(low, fminf(mn[2 * p], mn[2 * p + 1]));
+        }
+        if (low >= flt_min()) {
+#pragma unroll
+            for (int p = 0; p < N; ++p) {
+                const f2 mn2 = pack2(mn[2 * p], mn[2 * p + 1]);
+                f2 S = pack2(0.0f, 0.0f);
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                    const f2 q = mul2(mn2, pack2(rcp_approx(lo2(b[p][j])), rcp_approx(hi2(b[p][j]))));
+                    w2[p][j] = mul2(q, q);
+                    S = add2(S, w2[p][j]);
+                }
+                const float ra = rcp_approx(lo2(S)), rb = rcp_approx(hi2(S));
+#pragma unroll
+                for (int j = 0; j < C; ++j) w2[p][j] = mul2(w2[p][j], pack2(ra, rb));
+                // d2min S^(-1/2), back from scaled differences
+                const float q = rcp_approx(lo2(c.scale));  // of a power of two: exact
+                J2[p] = mul2(mul2(mn2, pack2(sqrt_approx(ra), sqrt_approx(rb))), pack2(q * q, q * q));
+            }
+            return;
+        }
+    } else if (MK == M_TWO || MK == M_THREE || MK == M_ONE_HALF) {
+        f2 b0[N], P[N][C];
+        unsigned worst = 0u;  // of the sums' distances from the smallest normal float
+        float s0[N], s1[N];
+#pragma unroll
+        for (int p = 0; p < N; ++p) {
+            f2 b[C];
+#pragma unroll
+            for (int j = 0; j < C; ++j) b[j] = (MK == M_THREE) ? abs2(d2[p][j]) : mul2(d2[p][j], d2[p][j]);
+            b0[p] = b[0];
+            co_products<C>(b, P[p]);
+            f2 S = (MK == M_ONE_HALF) ? mul2(P[p][0], P[p][0]) : P[p][0];
+#pragma unroll
+            for (int j = 1; j < C; ++j) S = (MK == M_ONE_HALF) ? fma2(P[p][j], P[p][j], S) : add2(S, P[p][j]);
+            unpack2(S, s0[p], s1[p]);
+            // a normal positive float has bits in [0x00800000, 0x7f800000): not
+            // zero, subnormal, infinite or NaN
+            worst = max(worst, max(__float_as_uint(s0[p]) - 0x00800000u, __float_as_uint(s1[p]) - 0x00800000u));
+        }
+        if (worst < 0x7f000000u) {
+#pragma unroll
+            for (int p = 0; p < N; ++p) {
+                const f2 r = (MK == M_ONE_HALF) ? pack2(rsqrt_approx(s0[p]), rsqrt_approx(s1[p]))
+                                                : pack2(rcp_approx(s0[p]), rcp_approx(s1[p]));
+                if (!POWERS) {
+                    // u_j d_j^2 (m = 2), (u_j |d_j|)^2 (m = 3), any j
+                    J2[p] = mul2(mul2(P[p][0], r), b0[p]);
+                    if (MK == M_THREE) J2[p] = mul2(J2[p], J2[p]);
+                }
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                    const f2 u = mul2(P[p][j], r);
+                    if (POWERS) {
+                        w2[p][j] = mul2(u, u);
+                        if (MK != M_TWO) w2[p][j] = mul2(w2[p][j], u);
+                    } else {
+                        w2[p][j] = u;
+                    }
+                }
             }
             return;
         }
     } else {
-        float ta[C], tb[C];
-        float la = __int_as_float(0x7f800000), lb = la;
+        float t[2 * N][C], l[2 * N], mn[2 * N], low = __int_as_float(0x7f800000);
 #pragma unroll
-        for (int j = 0; j < C; ++j) {
-            float da, db;
-            unpack2(mul2(d2[j], d2[j]), da, db);
-            ta[j] = lg2_approx(da);  // a squared distance below 2^-126 reads as 0: -inf
-            tb[j] = lg2_approx(db);
-            la = fminf(la, ta[j]);
-            lb = fminf(lb, tb[j]);
-        }
-        if (la >= -126.0f && lb >= -126.0f) {
-            f2 S = pack2(0.0f, 0.0f);
+        for (int p = 0; p < N; ++p) {
+            l[2 * p] = l[2 * p + 1] = mn[2 * p] = mn[2 * p + 1] = __int_as_float(0x7f800000);
 #pragma unroll
             for (int j = 0; j < C; ++j) {
-                ta[j] = inv_m1 * (la - ta[j]);
-                tb[j] = inv_m1 * (lb - tb[j]);
-                S = add2(S, pack2(ex2_approx(ta[j]), ex2_approx(tb[j])));
-            }
-            const float ga = lg2_approx(lo2(S)), gb = lg2_approx(hi2(S));
+                float q[2];
+                unpack2(mul2(d2[p][j], d2[p][j]), q[0], q[1]);
 #pragma unroll
-            for (int j = 0; j < C; ++j) um2[j] = pack2(ex2_approx(m * (ta[j] - ga)), ex2_approx(m * (tb[j] - gb)));
+                for (int h = 0; h < 2; ++h) {
+                    if (!POWERS) mn[2 * p + h] = fminf(mn[2 * p + h], q[h]);
+                    t[2 * p + h][j] = lg2_approx(q[h]);  // a square below 2^-126 reads as 0: -inf
+                    l[2 * p + h] = fminf(l[2 * p + h], t[2 * p + h][j]);
+                }
+            }
+            low = fminf(low, fminf(l[2 * p], l[2 * p + 1]));
+        }
+        if (low >= -126.0f) {
+#pragma unroll
+            for (int p = 0; p < N; ++p) {
+                const float la = l[2 * p], lb = l[2 * p + 1];
+                f2 S = pack2(0.0f, 0.0f);
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                    t[2 * p][j] = inv_m1 * (la - t[2 * p][j]);
+                    t[2 * p + 1][j] = inv_m1 * (lb - t[2 * p + 1][j]);
+                    w2[p][j] = pack2(ex2_approx(t[2 * p][j]), ex2_approx(t[2 * p + 1][j]));
+                    S = add2(S, w2[p][j]);
+                }
+                const float ga = lg2_approx(lo2(S)), gb = lg2_approx(hi2(S));
+                if (POWERS) {
+#pragma unroll
+                    for (int j = 0; j < C; ++j)
+                        w2[p][j] = pack2(ex2_approx(m * (t[2 * p][j] - ga)), ex2_approx(m * (t[2 * p + 1][j] - gb)));
+                } else {
+                    const f2 r = pack2(rcp_approx(lo2(S)), rcp_approx(hi2(S)));
+#pragma unroll
+                    for (int j = 0; j < C; ++j) w2[p][j] = mul2(w2[p][j], r);
+                    // d2min S^(1-m)
+                    J2[p] = mul2(pack2(mn[2 * p], mn[2 * p + 1]),
+                                 pack2(ex2_approx((1.0f - m) * ga), ex2_approx((1.0f - m) * gb)));
+                }
+            }
             return;
         }
     }
-    const Powers<C> w = powers_scalar<C, MK>(lo2(x2), hi2(x2), vs, m, inv_m1);
 #pragma unroll
-    for (int j = 0; j < C; ++j) um2[j] = pack2(w.a[j], w.b[j]);
+    for (int p = 0; p < N; ++p) {
+        const PixelPair<C> w = scalar_pair<C, MK, POWERS>(lo2(x2[p]), hi2(x2[p]), c.vs, m, inv_m1);
+#pragma unroll
+        for (int j = 0; j < C; ++j) w2[p][j] = pack2(w.a[j], w.b[j]);
+        if (!POWERS) J2[p] = pack2(w.Ja, w.Jb);
+    }
 }
 
 // Compensated FP32 ("double-float") sum, hi + lo, with Knuth's TwoSum: long
@@ -405,6 +513,19 @@ __device__ __forceinline__ DF df_merge(DF a, DF b) {
     return DF{hi, __fsub_rn(lo, __fsub_rn(hi, s))};
 }
 
+// The same without the renormalisation (two dependent steps shorter): for a
+// few merges in a row, followed by df_norm.
+__device__ __forceinline__ DF df_merge_raw(DF a, DF b) {
+    const float s = __fadd_rn(a.hi, b.hi);
+    const float bb = __fsub_rn(s, a.hi);
+    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
+    return DF{s, __fadd_rn(__fadd_rn(a.lo, b.lo), e)};
+}
+__device__ __forceinline__ DF df_norm(DF a) {
+    const float hi = __fadd_rn(a.hi, a.lo);
+    return DF{hi, __fsub_rn(a.lo, __fsub_rn(hi, a.hi))};
+}
+
 // Warp-wide double-float sum (xor tree, fixed order).
 __device__ __forceinline__ DF warp_sum_df(DF d) {
     const int lane = threadIdx.x & 31;
@@ -414,23 +535,6 @@ __device__ __forceinline__ DF warp_sum_df(DF d) {
         d = (lane & o) ? df_merge(e, d) : df_merge(d, e);
     }
     return d;
-}
-
-// N warp-wide double-float sums at once: every level of the xor tree issues
-// the shuffles of all N sums before their merges, so the N chains of five
-// dependent levels overlap instead of running one after another. Each sum is
-// the same as warp_sum_df's (same operands, same order).
-template <int N>
-__device__ __forceinline__ void warp_sum_df_n(DF (&d)[N]) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        DF e[N];
-#pragma unroll
-        for (int q = 0; q < N; ++q) e[q] = DF{__shfl_xor_sync(0xffffffffu, d[q].hi, o), __shfl_xor_sync(0xffffffffu, d[q].lo, o)};
-#pragma unroll
-        for (int q = 0; q < N; ++q) d[q] = (lane & o) ? df_merge(e[q], d[q]) : df_merge(d[q], e[q]);
-    }
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

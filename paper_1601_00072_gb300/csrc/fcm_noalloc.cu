@@ -32,9 +32,9 @@ using namespace fcm;
 namespace {
 
 constexpr size_t kStateBytes = (sizeof(RunState) + 255) / 256 * 256;
-constexpr size_t kSlotBytes = (size_t)RUN_SLOT_BYTES * run_slots(FCM_MAX_CLUSTERS) * FCM_NOALLOC_MAX_BLOCKS;
+constexpr size_t kSlotBytes = run_scratch_bytes(FCM_NOALLOC_MAX_BLOCKS);
 
-// The scratch: run state, then the blocks' exchange slots (zero at load).
+// The scratch: run state, then the blocks' exchange scratch (zero at load).
 // In host code this name is only a stand-in for the device array; its device
 // address comes from cudaGetSymbolAddress, once per device.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kStateBytes + kSlotBytes];
@@ -74,14 +74,7 @@ int setup_device(int dev) {
     }
     const RunTable& t = run_table();
     for (int C = 1; C <= FCM_MAX_CLUSTERS; ++C)
-        for (int mk = 0; mk < 4; ++mk) {
-            int nb = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)t.run[C][mk], RUN_NT, 0) != cudaSuccess) {
-                cudaGetLastError();
-                nb = 0;
-            }
-            d.fits[C][mk] = nb > 0;
-        }
+        for (int mk = 0; mk < 4; ++mk) d.fits[C][mk] = run_kernel_fits((const void*)t.run[C][mk], C);
     return d.status = FCM_OK;
 }
 
@@ -131,8 +124,8 @@ extern "C" int fcm_run_noalloc(const float* x, int64_t n, int C, float m, float 
 
     const int mk = mkind_of(m);
     if (!d.fits[C][mk]) return FCM_ERR_CUDA;
-    const int blocks = run_grid(n, d.num_sms);
-    if (blocks > FCM_NOALLOC_MAX_BLOCKS) return FCM_ERR_TOO_LARGE;
+    const RunShape shape = run_shape(n, C, std::min(d.num_sms, RUN_MAX_BLOCKS));
+    if (shape.blocks > FCM_NOALLOC_MAX_BLOCKS) return FCM_ERR_TOO_LARGE;
 
     RunState* st = reinterpret_cast<RunState*>(d.scratch);
     char* slots = reinterpret_cast<char*>(d.scratch + kStateBytes);
@@ -168,9 +161,14 @@ extern "C" int fcm_run_noalloc(const float* x, int64_t n, int C, float m, float 
     }
     if (e == cudaSuccess && nonce == 1) e = cudaMemsetAsync(slots, 0, kSlotBytes, stream);
     if (e == cudaSuccess) {
-        void* args[3] = {&st, &slots, &nonce};
-        e = cudaLaunchCooperativeKernel((const void*)run_table().run[C][mk], dim3((unsigned)blocks), dim3(RUN_NT), args,
-                                        0, stream);
+        int resident = shape.resident;
+        void* args[4] = {&st, &slots, &nonce, &resident};
+        e = cudaLaunchCooperativeKernel((const void*)run_table().run[C][mk], dim3(shape.blocks), dim3(shape.threads), args, shape.smem,
+                                        stream);
+    }
+    if (e != cudaSuccess) {
+        std::lock_guard<std::mutex> lock(g_mu);
+        g_dev[dev].nonce = 0;  // the number was not used: the next run zeroes the scratch
     }
     RunState out;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&out, st, sizeof(RunState), cudaMemcpyDeviceToHost, stream);

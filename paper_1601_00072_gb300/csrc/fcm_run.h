@@ -6,8 +6,17 @@
 
 namespace fcm {
 
-constexpr int RUN_NT = 512;  // threads per block of the whole-run kernel, one block per SM
-constexpr int RUN_NW = RUN_NT / 32;
+// Threads per block of the whole-run kernel (one block per SM): pt pixel
+// threads, then one control warp. At most 15 pixel warps at C <= 5 (128
+// registers each; a 17th warp would leave 96) and 11 above (168 registers).
+constexpr int run_max_pt(int C) { return C <= 5 ? 480 : 352; }
+constexpr int RUN_MAX_PW = 15;
+constexpr int RUN_FEW_PT = 128;
+// Dynamic shared memory: the second set of the sums (2 C pairs per pixel
+// thread), then `resident` quads of x per pixel thread.
+constexpr int run_smem(int C, int pt, int resident) { return pt * 16 * (C + resident); }
+constexpr int RUN_SMEM_MAX = 222 * 1024;
+constexpr int run_max_resident(int C, int pt) { return RUN_SMEM_MAX / (pt * 16) - C; }
 
 // One 16-byte exchange slot: two values and the 64-bit tag of the exchange
 // they belong to, written and read as a unit.
@@ -16,7 +25,17 @@ constexpr int RUN_SLOT_BYTES = 16;
 // maximum and the flags; two exchanges are live at a time.
 constexpr int run_slots(int C) { return 2 * (C + 1); }
 
-typedef void (*WholeRunFn)(RunState*, void* slots, unsigned nonce);
+// The scratch of the exchanges: the words of two banks (runs alternate), each
+// [parity][cluster or control], a 128-byte line each; then the slots.
+constexpr int RUN_WORD_BYTES = 128;
+constexpr int RUN_WORDS_BYTES = 2 * 2 * (FCM_MAX_CLUSTERS + 1) * RUN_WORD_BYTES;
+constexpr int RUN_MAX_BLOCKS = 255;  // a word's top byte counts them
+constexpr size_t run_scratch_bytes(int blocks) {
+    return RUN_WORDS_BYTES + (size_t)RUN_SLOT_BYTES * run_slots(FCM_MAX_CLUSTERS) * blocks;
+}
+
+// nonce: the run's number on its scratch, counting up by one from run to run.
+typedef void (*WholeRunFn)(RunState*, char* scratch, unsigned nonce, int resident);
 
 struct RunTable {
     WholeRunFn run[FCM_MAX_CLUSTERS + 1][4];
@@ -34,7 +53,15 @@ void register_run_c8(RunTable&);
 // The kernel table, filled on first use.
 const RunTable& run_table();
 
-// Grid of a run of n pixels when at most max_blocks blocks are co-resident.
-int run_grid(int64_t n, int64_t max_blocks);
+// Raises the kernel's dynamic shared memory limit; whether it can be launched.
+bool run_kernel_fits(const void* kernel, int C);
+
+// Launch shape of a run of n pixels when at most max_blocks blocks are
+// co-resident (0 blocks: none): blocks, threads per block, quads of x per pixel
+// thread kept in shared memory, and the dynamic shared memory that takes.
+struct RunShape {
+    int blocks, threads, resident, smem;
+};
+RunShape run_shape(int64_t n, int C, int64_t max_blocks);
 
 }  // namespace fcm

@@ -9,35 +9,50 @@
 //  * A sums pass (iteration k) reads x, forms u^m from V^k (Eq. 4) and adds up
 //    the numerators and denominators of V^{k+1} (Eq. 3): 4 bytes per pixel
 //    instead of 4 + 8C.
-//  * In the same pass a few warps take max |U^k - U^{k-1}| over a sample of the
-//    pixels (U^{k-1} again from V^{k-1}, or from U^0 at k = 1). The maximum over
-//    a sample is a lower bound of delta_k: when it reaches eps the run cannot
-//    stop at k, and the exact delta_k is not needed.
+//  * A control warp beside the pixel warps takes max |U^k - U^{k-1}| over a
+//    sample of the pixels (U^{k-1} again from V^{k-1}, or from U^0 at k = 1). The
+//    maximum over a sample is a lower bound of delta_k: when it reaches eps in any
+//    block the run cannot stop at k, and the exact delta_k is not needed.
 //  * When it does not, or k is max_iter, or a trace wants every iteration, a
-//    full pass takes delta_k over every pixel and J_k (Eq. 1), and writes U^k
-//    unless the sample has already shown that the run goes on. If the run goes
-//    on all the same, the next samples hold the pixel of largest change that
-//    every thread saw.
+//    full pass takes delta_k over every pixel and J_k (Eq. 1), and writes U^k. If
+//    the run goes on all the same, the next samples hold the pairs of largest
+//    change that the pixel warps saw.
 // The iterates, the stop decision and the outputs are those of the loop that
 // takes delta_k in every iteration; U is written once instead of k times.
 //
-// What bounds it: on a large image the FP32 pipe (about 33 operations per pixel
-// and iteration at C = 4, m = 2, in packed FP32x2 pairs); x comes from the L2
-// (67 MB for a 256^3 volume) or, up to about 10 million pixels, partly from L1.
-// On a small image the exchange between the blocks. 60 iterations on a GB300,
-// before (U stored; plain loads and a launch per pass where n % 4 != 0) and
-// after: 200x200 371 -> 215 us, 199x201 907 -> 247 us, 1024x1024 716 -> 413 us,
-// 256^3 6.02 -> 1.85 ms.
+// What bounds it: on a large image the FP32 pipe (33 operations per pixel and
+// iteration at C = 4, m = 2, in packed FP32x2 pairs: 14 us per iteration of a
+// 256^3 volume at the pipe's rate, 27 measured; 15 pixel warps per SM, two pairs
+// in flight each: 23 or 31 warps with fewer registers were slower). x is kept in
+// shared memory up to 7 million pixels; beyond that, the rest of x comes from the
+// L2, two steps ahead of its use. On a small image it is the latency of an
+// iteration (1.9 us at 40,000 pixels): about 1 us of dependent steps in a block
+// and as much for the exchange. 60 iterations on a GB300, before (U stored; plain
+// loads and a launch per pass where n % 4 != 0) and after: 200x200 371 -> 160 us,
+// 199x201 907 -> 195 us, 1024x1024 713 -> 283 us, 256^3 6.02 -> 1.79 ms.
 //
-// The exchange carries its own arrival: every block publishes (num_j, den_j)
-// with a 64-bit tag (the run's number and the exchange's index) in one 16-byte
-// store, and the warp that needs cluster j's totals polls the slots of all
-// blocks until each shows the tag. That is one L2 round trip after the slowest
-// block's store, where a barrier counter followed by reads of the partial sums
-// takes three. Every block adds the blocks' totals in the same order in
-// compensated FP32, so all derive the same V^{k+1} and the same decision.
+// The exchange. Between iterations every block adds its totals of (num_j, den_j)
+// as 64-bit fixed-point numbers to one word each, with a reduction in the L2; the
+// top byte of a word counts the arrivals, so the word itself says when the sum
+// is complete, and the warp that needs cluster j polls these two words and
+// nothing else. Integer sums do not depend on the order of arrival: every block
+// reads the same totals and forms the same V^{k+1}. (Slots that every block
+// polls for every other one cost 5,000 cycles per exchange at 152 blocks, most
+// of it contention of the polls: 7.5 us per iteration of a 1 M-pixel image.)
+// The words are never cleared within a run: those of even and odd exchanges
+// alternate, and a sum is the difference from the word's value two exchanges
+// ago, which no block can have moved on from before all have read it. The
+// fixed-point unit comes from n and the largest |x|, |V^0|, known after pass 0;
+// it is 2^-53 of the largest total possible. A cluster whose den_j is below
+// 2^-16 n could lose precision to it: then (the same decision in every block) the
+// totals go through the slots instead, as do pass 0's and J's.
+// Slots: a block's values with a 64-bit tag (the run's number and the exchange's
+// index) in one 16-byte store, polled until each block's shows the tag, added in
+// block order in compensated FP32.
 // Every poll loop is bounded (fcm_set_limits): the run then ends with
 // FCM_ERR_TIMEOUT.
+#include <type_traits>
+
 #include "fcm_device.cuh"
 #include "fcm_df.cuh"
 #include "fcm_internal.h"
@@ -49,8 +64,6 @@
 
 namespace fcm {
 namespace {
-
-constexpr int SAMPLE_WARPS = 4;  // warps per block that sample delta_k: one per SM sub-partition
 
 // ---- exchange slots: {float a, float b, u64 tag} moved as one 128-bit unit ----
 
@@ -115,6 +128,34 @@ __device__ __forceinline__ bool collect(const char* slots, int nb, uint64_t tag,
     return ok;
 }
 
+// ---- exchange words ----
+
+constexpr uint64_t ARRIVAL = 1ull << 56;  // the top byte counts blocks (at most 255)
+
+__device__ __forceinline__ void red_add_u64(uint64_t* p, uint64_t v) {
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ void ld_words(const uint64_t* p, uint64_t& a, uint64_t& b) {
+    asm volatile(
+        "{\n\t.reg .b128 t;\n\t"
+        "ld.relaxed.gpu.global.b128 t, [%2];\n\t"
+        "mov.b128 {%0, %1}, t;\n\t}"
+        : "=l"(a), "=l"(b)
+        : "l"(p)
+        : "memory");
+}
+// The arrivals in a word's change since an earlier value; the sum in it may be
+// negative, but is below 2^55 in magnitude.
+__device__ __forceinline__ unsigned arrivals(uint64_t change) { return (unsigned)((change + (ARRIVAL >> 1)) >> 56); }
+__device__ __forceinline__ DF fixed_to_df(int64_t v, float unit) {
+    // the upper 24 bits exactly, the lower 31 rounded; then renormalised
+    const float a = (float)(int)(v >> 31) * 2147483648.0f, b = (float)(int)(v & 0x7fffffff);
+    const float hi = __fadd_rn(a, b);
+    return DF{hi * unit, __fsub_rn(b, __fsub_rn(hi, a)) * unit};
+}
+// 2^e for e in [-126, 127].
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
+
 // ---- warp totals of N values: log-step halving, N - 1 + (5 - log2 N) shuffles ----
 
 constexpr int pow2_at_least(int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : 16; }
@@ -148,38 +189,31 @@ __device__ __forceinline__ int slot_of_lane(int lane) {
     return s;
 }
 
-// ---- one pair of pixels in a sums pass ----
+// ---- the sums of a sums pass ----
 
 // The numerators are centered: num_j = sum u_j^m (x - v_j^k), so that
 // v_j^{k+1} = v_j^k + num_j / den_j. The differences are at hand, and the FP32
 // rounding of the sums is then relative to the pixels' distance from the center
 // and not to their grey level, and vanishes from den as the run converges.
 //
-// Sums in two levels: pairs into num2/den2, those into num/den after every
-// FOLD quads. A thread's share of a 256^3 volume is 54 quads; many of its terms
-// are equal (a constant background), so a single chain of 108 additions rounds
-// the same way again and again, in all threads alike. Uncentered and in one
-// chain, the sums moved the iteration at which a random start of that volume
-// breaks its symmetry by three.
+// Sums in two levels: pairs into num2/den2, those into a second set after every
+// FOLD quads. A thread's share of a 256^3 volume is 27 quads; many of its terms
+// are equal (a constant background), so a single chain of additions rounds the
+// same way again and again, in all threads alike. Uncentered and in one chain of
+// 108, the sums moved the iteration at which a random start of that volume
+// breaks its symmetry by three. The second set is touched once in FOLD quads
+// and lives in shared memory, not in registers.
 constexpr int FOLD = 8;
+static_assert(RUN_MAX_PW <= 16, "the block's totals are a tree over 16 lanes");
+// Pairs of pixels whose arithmetic overlaps: as many as fit in the registers.
+constexpr int run_pairs(int C) { return C <= 6 ? 2 : 1; }
 
 template <int C>
 struct SumAcc {
-    f2 num2[C], den2[C], num[C], den[C];
-    int held;
+    f2 num2[C], den2[C];
     __device__ __forceinline__ void reset() {
 #pragma unroll
-        for (int j = 0; j < C; ++j) num2[j] = den2[j] = num[j] = den[j] = pack2(0.0f, 0.0f);
-        held = 0;
-    }
-    __device__ __forceinline__ void fold() {
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            num[j] = add2(num[j], num2[j]);
-            den[j] = add2(den[j], den2[j]);
-            num2[j] = den2[j] = pack2(0.0f, 0.0f);
-        }
-        held = 0;
+        for (int j = 0; j < C; ++j) num2[j] = den2[j] = pack2(0.0f, 0.0f);
     }
     __device__ __forceinline__ void add(const f2 (&d2)[C], const f2 (&um2)[C]) {
 #pragma unroll
@@ -188,302 +222,502 @@ struct SumAcc {
             den2[j] = add2(den2[j], um2[j]);
         }
     }
-};
-
-// What the passes read of the run.
-struct Px {
-    const float* __restrict__ x;
-    int64_t n;
-    bool vec_x;   // x 16-byte aligned: quads of pixels
-    bool vec_u;   // n % 4 == 0 and U, U^0 aligned too: quads of memberships
-};
-
-// Calls f(xa, xb) on packed pairs, the pixels (i, i+1) of a quad; tail(i) on
-// the pixels past the last whole quad (at most three, on one thread). The
-// loads run two steps ahead of their use.
-template <typename F, typename T>
-__device__ __forceinline__ void for_quads(const Px& px, int64_t t0, int64_t nt, F&& f, T&& tail) {
-    const int64_t nq = px.n >> 2;
-    const float4* x4 = reinterpret_cast<const float4*>(px.x);
-    float4 a = t0 < nq ? __ldg(x4 + t0) : make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 b = t0 + nt < nq ? __ldg(x4 + t0 + nt) : make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t q = t0; q < nq; q += nt) {
-        const float4 c = a;
-        a = b;
-        if (q + 2 * nt < nq) b = __ldg(x4 + q + 2 * nt);
-        f(c, 4 * q);
+    // Into the second set (of this thread: stride threads apart), or from it.
+    __device__ __forceinline__ void fold(f2* set, int stride, bool first) {
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            f2* const a = set + (2 * j) * stride;
+            f2* const b = a + stride;
+            *a = first ? num2[j] : add2(*a, num2[j]);
+            *b = first ? den2[j] : add2(*b, den2[j]);
+        }
+        reset();
     }
-    if (t0 == nq % nt)
-        for (int64_t i = 4 * nq; i < px.n; ++i) tail(i);
-}
-
-// The same for unaligned x or rows: a warp takes 128 consecutive pixels, a
-// lane the pixels base + lane + 32 p, p = 0..3 (coalesced 32-bit accesses);
-// whole tiles through f, the last partial one pixel by pixel through tail.
-template <typename F, typename T>
-__device__ __forceinline__ void for_tiles(const Px& px, int64_t t0, int64_t nt, F&& f, T&& tail) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = nt >> 5, w0 = t0 >> 5, tiles = (px.n + 127) >> 7;
-    for (int64_t w = w0; w < tiles; w += nw) {
-        const int64_t i = (w << 7) + lane;
-        if ((w << 7) + 128 <= px.n) {
-            const float4 c = make_float4(__ldg(px.x + i), __ldg(px.x + i + 32), __ldg(px.x + i + 64), __ldg(px.x + i + 96));
-            f(c, i);
-        } else {
-#pragma unroll 1
-            for (int64_t k = i; k < px.n; k += 32) tail(k);
+    __device__ __forceinline__ void finish(const f2* set, int stride, bool folded) {
+        if (!folded) return;
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            num2[j] = add2(num2[j], set[(2 * j) * stride]);
+            den2[j] = add2(den2[j], set[(2 * j + 1) * stride]);
         }
     }
-}
+};
+
+// The pixels of a pass. Pixel thread t0 of nt takes the quads (four consecutive
+// pixels) t0, t0 + nt, ...; the first `resident` of them stay in shared memory
+// for the whole run (at xs[step * pt], this thread's own place), the others are
+// read again in every pass.
+struct Px {
+    const float* __restrict__ x;
+    float4* xs;
+    int64_t n, t0, nt;
+    int pt;               // pixel threads of the block
+    int steps, resident;  // this thread's quads; how many of them are kept
+    bool vec_x;           // x is 16-byte aligned
+    bool vec_u;           // so are the rows of U and U^0, and n % 4 == 0
+
+    __device__ __forceinline__ float4 load(int step) const {
+        const int64_t q = t0 + (int64_t)step * nt;
+        if (vec_x) return __ldg(reinterpret_cast<const float4*>(x) + q);
+        const float* p = x + 4 * q;
+        return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+    }
+    // tail(i) on the pixels past the last whole quad (at most three, on one thread)
+    template <typename T>
+    __device__ __forceinline__ void tail(T&& f) const {
+        if (t0 == (n >> 2) % nt) {
+#pragma unroll 1
+            for (int64_t i = n & ~(int64_t)3; i < n; ++i) f(i);
+        }
+    }
+    // Reads the quads from global memory, two steps ahead, keeps the resident
+    // ones and calls f(quad, index of its first pixel).
+    template <typename F>
+    __device__ __forceinline__ void stage(F&& f) const {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+        if (steps > 0) a = load(0);
+        if (steps > 1) b = load(1);
+#pragma unroll 1
+        for (int s = 0; s < steps; ++s) {
+            const float4 c = a;
+            a = b;
+            if (s + 2 < steps) b = load(s + 2);
+            if (s < resident) xs[s * pt] = c;
+            f(c, 4 * (t0 + (int64_t)s * nt));
+        }
+    }
+    // The same, once the resident quads are in place.
+    template <typename F>
+    __device__ __forceinline__ void quads(F&& f) const {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+        if (resident < steps) {
+            a = load(resident);
+            if (resident + 1 < steps) b = load(resident + 1);
+        }
+#pragma unroll 1
+        for (int s = 0; s < steps; ++s) {
+            float4 c;
+            if (s < resident) {
+                c = xs[s * pt];
+            } else {
+                c = a;
+                a = b;
+                if (s + 2 < steps) b = load(s + 2);
+            }
+            f(c, 4 * (t0 + (int64_t)s * nt));
+        }
+    }
+    // For unaligned rows of U: a warp takes 128 consecutive pixels, a lane the
+    // pixels i + 32 p, p = 0..3 (coalesced 32-bit accesses); whole tiles through f,
+    // the last partial one pixel by pixel through g.
+    template <typename F, typename G>
+    __device__ __forceinline__ void tiles(F&& f, G&& g) const {
+        const int64_t nw = nt >> 5, all = (n + 127) >> 7;
+#pragma unroll 1
+        for (int64_t w = t0 >> 5; w < all; w += nw) {
+            const int64_t i = (w << 7) + (threadIdx.x & 31);
+            if ((w << 7) + 128 <= n) {
+                f(make_float4(__ldg(x + i), __ldg(x + i + 32), __ldg(x + i + 64), __ldg(x + i + 96)), i);
+            } else {
+#pragma unroll 1
+                for (int64_t k = i; k < n; k += 32) g(k);
+            }
+        }
+    }
+};
 
 template <int C>
 struct RunShared {
-    float red[RUN_NW][2 * C];  // warp totals of a sums pass; row 0..: J in red[w][0] of a full pass
-    float mx[RUN_NW];
-    unsigned bad[RUN_NW];
-    DF vq[C];                  // V^{k+1} as double-float quotients
-    int empty[C];
+    float red[RUN_MAX_PW][2 * C];  // warp totals of a sums pass; J in red[w][0] of a full pass
+    float mx[RUN_MAX_PW];
+    unsigned bad[RUN_MAX_PW];      // bit 0: bad input; bit 1: wit holds a pair of the image
+    f2 wit[RUN_MAX_PW];            // each warp's pair of largest change in a full pass
+    float v[4][C];             // V^k in v[k % 4]
+    DF v64[4][C];              // the double-float quotients behind them
+    unsigned empty[4];         // whether some cluster was empty in the sums behind V^k
+    int4 ctl;                  // x: a wait gave up; y: a sampled change reached eps; z: some
+                               // den_j is too small for the exchange words
     DF J;
     float delta;
     unsigned flags;            // bit 0: bad input
-    int err;
-    float v[C], vp[C];         // V^k and V^{k-1}, for the rare scalar path and the sample
+    WaitLimits lim;
 };
 
-template <int C, int MK>
-__global__ void __launch_bounds__(RUN_NT, 1) k_fcm_run(RunState* __restrict__ st, void* slots_raw, unsigned nonce) {
+// A pixel warp's totals of a sums pass into sh.red.
+template <int C>
+__device__ __forceinline__ void warp_sums(RunShared<C>& sh, float (&a)[pow2_at_least(2 * C)]) {
     constexpr int P = pow2_at_least(2 * C);
-    constexpr bool SCALED = MK == M_ONE_HALF;
+    const int lane = threadIdx.x & 31;
+    warp_totals<P>(a);
+    const int s = slot_of_lane<P>(lane);
+    if ((lane & (32 / P - 1)) == 0 && s < 2 * C) sh.red[threadIdx.x >> 5][s] = a[0];
+}
+
+// A sums pass of a pixel warp from V^k in sh.v[cur]. FIRST: pass 0 from V^0,
+// which reads x and calls see(x) on every pixel.
+template <int C, int MK, bool FIRST, typename See>
+__device__ __forceinline__ void sums_pass_body(const Px& px, RunShared<C>& sh, f2* second, int cur, float m,
+                                               float inv_m1, See&& see) {
+    constexpr int P = pow2_at_least(2 * C);
+    SumAcc<C> a;
+    a.reset();
+    PackedCenters<C, MK> cen;
+    cen.set(sh.v[cur]);
+    f2* const set = second + threadIdx.x;
+    int held = 0;
+    bool folded = false;
+    auto quad = [&](const float4& c, int64_t) {
+        if (FIRST) see(c.x), see(c.y), see(c.z), see(c.w);
+        if (run_pairs(C) == 2) {
+            f2 um[2][C], d2[2][C], J2[2];
+            const f2 xq[2] = {pack2(c.x, c.y), pack2(c.z, c.w)};
+            packed_pairs<C, MK, true, 2>(xq, cen, m, inv_m1, um, d2, J2);
+            a.add(d2[0], um[0]);
+            a.add(d2[1], um[1]);
+        } else {
+            // one pair at a time: two would not fit in the registers
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                f2 um[1][C], d2[1][C], J2[1];
+                const f2 xq[1] = {h ? pack2(c.z, c.w) : pack2(c.x, c.y)};
+                packed_pairs<C, MK, true, 1>(xq, cen, m, inv_m1, um, d2, J2);
+                a.add(d2[0], um[0]);
+            }
+        }
+        if (++held == FOLD) {
+            a.fold(set, px.pt, !folded);
+            folded = true;
+            held = 0;
+        }
+    };
+    if (FIRST) px.stage(quad);
+    else px.quads(quad);
+    px.tail([&](int64_t i) {
+        // a pixel past the last quad: the low halves of the sums
+        const float xi = __ldg(px.x + i);
+        if (FIRST) see(xi);
+        const PixelPair<C> w = scalar_pair<C, MK, true>(xi, xi, cen.vs, m, inv_m1);
+        const f2 xs = cen.of(pack2(xi, xi));
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            const f2 um = pack2(w.a[j], 0.0f);
+            a.num2[j] = fma2(um, sub2(xs, cen.v2[j]), a.num2[j]);
+            a.den2[j] = add2(a.den2[j], um);
+        }
+    });
+    a.finish(set, px.pt, folded);
+    // back from scaled differences (by a power of two: exact)
+    const float back = PackedCenters<C, MK>::SCALED ? rcp_approx(lo2(cen.scale)) : 1.0f;
+    float t[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        const f2 q = i < C ? a.num2[i < C ? i : 0] : a.den2[(i >= C && i < 2 * C) ? i - C : 0];
+        t[i] = i < 2 * C ? lo2(q) + hi2(q) : 0.0f;
+        if (PackedCenters<C, MK>::SCALED && i < C) t[i] *= back;
+    }
+    warp_sums<C>(sh, t);
+}
+
+template <int C, int MK>
+__device__ __forceinline__ void sums_pass(const Px& px, RunShared<C>& sh, f2* second, int cur, float m, float inv_m1) {
+    sums_pass_body<C, MK, false>(px, sh, second, cur, m, inv_m1, [](float) {});
+}
+
+// What an exchange adds up over the blocks.
+enum Exchange : int { X_SUMS0 = 0, X_SUMS = 1, X_J = 2 };  // sums of pass 0 from U^0; centered sums; J
+
+template <int C, int MK>
+__global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
+    k_fcm_run(RunState* __restrict__ st, char* scratch, unsigned nonce, int resident) {
+    constexpr int P = pow2_at_least(2 * C);
+    extern __shared__ __align__(16) f2 second[];  // [2 C][pt] second set of the sums, then the resident quads
     __shared__ RunShared<C> sh;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t t0 = (int64_t)blockIdx.x * RUN_NT + threadIdx.x, nt = (int64_t)gridDim.x * RUN_NT;
+    const int pw = (int)(blockDim.x >> 5) - 1;  // pixel warps; the control warp follows
+    const bool control = warp == pw;
     const int nb = (int)gridDim.x;
     const bool from_u = st->from_u != 0;
     const float* U0 = st->Uprev;  // may be U itself: each pixel is read, then written, by one thread
     float* U = st->U;
+    const int64_t n = st->n;
     Px px;
     px.x = st->x;
-    px.n = st->n;
+    px.xs = reinterpret_cast<float4*>(second + 2 * C * 32 * pw) + threadIdx.x;
+    px.n = n;
+    px.pt = 32 * pw;
+    px.t0 = (int64_t)blockIdx.x * px.pt + threadIdx.x;
+    px.nt = (int64_t)nb * px.pt;
+    px.steps = (n >> 2) > px.t0 ? (int)(((n >> 2) - 1 - px.t0) / px.nt) + 1 : 0;
+    px.resident = min(resident, px.steps);
     px.vec_x = ((uintptr_t)px.x & 15) == 0;
-    px.vec_u = px.vec_x && (px.n & 3) == 0 && ((uintptr_t)U & 15) == 0 && (!from_u || ((uintptr_t)U0 & 15) == 0);
-    const int64_t n = px.n;
+    px.vec_u = px.vec_x && (n & 3) == 0 && ((uintptr_t)U & 15) == 0 && (!from_u || ((uintptr_t)U0 & 15) == 0);
     const float m = st->m, inv_m1 = st->inv_m1, eps = st->eps;
     const int max_iter = st->max_iter;
-    const uint32_t limit = st->lim.grid_spins, phantoms = st->lim.phantoms;
-    double* const trace = st->trace;
-    char* const slots = static_cast<char*>(slots_raw);
+    const bool tracing = st->trace != nullptr;
 
-    if (threadIdx.x < C) sh.v[threadIdx.x] = sh.vp[threadIdx.x] = st->V0[threadIdx.x];
-    if (threadIdx.x == 0) sh.err = 0;
-    __syncthreads();
-    f2 v2[C];
-    DF v64[C];  // the double-float quotients behind V^k
-#pragma unroll
-    for (int j = 0; j < C; ++j) {
-        v2[j] = pack2(sh.v[j], sh.v[j]);
-        v64[j] = DF{sh.v[j], 0.0f};
+    if (threadIdx.x < C) {
+        const float v0 = st->V0[threadIdx.x];
+        sh.v[0][threadIdx.x] = v0;
+        sh.v64[0][threadIdx.x] = DF{v0, 0.0f};
     }
-    int flags = 0;
+    if (threadIdx.x == 0) {
+        sh.ctl = make_int4(0, 0, 0, 0);
+        sh.empty[0] = sh.empty[1] = sh.empty[2] = sh.empty[3] = 0u;
+        sh.lim = st->lim;
+    }
+    __syncthreads();
+    int flags = 0;    // thread 0 of block 0 only
     unsigned nx = 0;  // exchanges so far
 
-    // Publishes this block's totals and collects every block's: the sums (or J)
-    // of sh.red, the maximum of sh.mx and the flags of sh.bad. SUMS: cluster
-    // totals -> sh.vq, sh.empty; otherwise J -> sh.J. centered: the numerators are
-    // relative to V^k. Returns false when a wait gave up.
-    auto exchange = [&](bool sums, bool centered) {
-        __syncthreads();
-        const uint64_t tag = ((uint64_t)nonce << 32) | ++nx;
-        char* const mine = slots + (int64_t)(nx & 1) * (C + 1) * nb * RUN_SLOT_BYTES;
-        const int nq = sums ? C : 1;
-        if (warp < nq) {
-            const int j = warp;
-            float a = lane < RUN_NW ? sh.red[lane][j] : 0.0f, b = (sums && lane < RUN_NW) ? sh.red[lane][C + j] : 0.0f;
-#pragma unroll
-            for (int o = RUN_NW / 2; o > 0; o >>= 1) {
-                a += __shfl_xor_sync(0xffffffffu, a, o);
-                b += __shfl_xor_sync(0xffffffffu, b, o);
-            }
-            char* const row = mine + (int64_t)j * nb * RUN_SLOT_BYTES;
-            if (lane == 0) st_slot(row + (int64_t)blockIdx.x * RUN_SLOT_BYTES, a, b, tag);
-            DF na{0.0f, 0.0f}, da{0.0f, 0.0f};
-            const bool ok = collect(row, nb, tag, limit, phantoms, [&](float p, float q) {
-                df_add(na, p);
-                df_add(da, q);
-            });
-            if (!ok && lane == 0) sh.err = 1;
-            DF d[2] = {na, da};
-            warp_sum_df_n<2>(d);
-            if (lane == 0) {
-                if (sums) {
-                    const bool empty = !(d[1].hi > 0.0f);
-                    DF q = empty ? DF{0.0f, 0.0f} : df_div(d[0], d[1]);
-                    if (centered) {
-                        if (SCALED) {
-                            const float s = __frcp_rn(spread_scale<C>(v2));  // a power of two: exact
-                            q = DF{q.hi * s, q.lo * s};
-                        }
-                        q = df_merge(q, DF{sh.v[j], 0.0f});
-                    }
-                    sh.vq[j] = q;
-                    sh.empty[j] = empty;
-                } else {
-                    sh.J = d[0];
-                }
-            }
-        } else if (warp == C) {
-            unsigned mb = lane < RUN_NW ? __float_as_uint(sh.mx[lane]) : 0u, fb = lane < RUN_NW ? sh.bad[lane] : 0u;
-            mb = __reduce_max_sync(0xffffffffu, mb);  // non-negative floats order as their bits
-            fb = __reduce_or_sync(0xffffffffu, fb);
-            char* const row = mine + (int64_t)C * nb * RUN_SLOT_BYTES;
-            if (lane == 0) st_slot(row + (int64_t)blockIdx.x * RUN_SLOT_BYTES, __uint_as_float(mb), __uint_as_float(fb), tag);
-            unsigned tm = 0u, tf = 0u;
-            const bool ok = collect(row, nb, tag, limit, phantoms, [&](float p, float q) {
-                tm = max(tm, __float_as_uint(p));
-                tf |= __float_as_uint(q);
-            });
-            if (!ok && lane == 0) sh.err = 1;
-            tm = __reduce_max_sync(0xffffffffu, tm);
-            tf = __reduce_or_sync(0xffffffffu, tf);
-            if (lane == 0) {
-                sh.delta = __uint_as_float(tm);
-                sh.flags = tf;
-            }
-        }
-        __syncthreads();
-        return sh.err == 0;
+    // The words of this run's bank (runs alternate between two; each run clears
+    // the other one, which the next run uses): [parity][cluster] pairs and, in row
+    // C, the control word, a 128-byte line each.
+    auto word = [&](unsigned bank, unsigned x, int q) {
+        return reinterpret_cast<uint64_t*>(scratch + RUN_WORD_BYTES * (((bank & 1) * 2 + (x & 1)) * (FCM_MAX_CLUSTERS + 1) + q));
     };
-    // This warp's totals of a sums pass into sh.red / sh.mx / sh.bad.
-    auto warp_publish = [&](const float (&num)[C], const float (&den)[C], float mx, bool bad) {
-        float a[P];
-#pragma unroll
-        for (int i = 0; i < P; ++i) a[i] = i < C ? num[i < C ? i : 0] : i < 2 * C ? den[i < 2 * C && i >= C ? i - C : 0] : 0.0f;
-        warp_totals<P>(a);
-        const int s = slot_of_lane<P>(lane);
-        if ((lane & (32 / P - 1)) == 0 && s < 2 * C) sh.red[warp][s] = a[0];
-        const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
-        const bool any = __any_sync(0xffffffffu, bad);
+    if (blockIdx.x == 0 && threadIdx.x < 2 * (FCM_MAX_CLUSTERS + 1)) {
+        uint64_t* const w = word(nonce + 1, threadIdx.x & 1, threadIdx.x >> 1);
+        w[0] = w[1] = 0ull;
+    }
+    char* const slots_raw = scratch + RUN_WORDS_BYTES;
+    // this warp's words after their last exchange, of even and odd parity
+    uint64_t seen_a0 = 0ull, seen_b0 = 0ull, seen_a1 = 0ull, seen_b1 = 0ull;
+    float to_num = 0.0f, to_den = 0.0f, num_unit = 0.0f, den_unit = 0.0f;  // fixed-point scales
+
+    // This block's row of exchange nx + 1: cluster q's slots, or (q = C) the
+    // maxima's and flags'.
+    auto slot_row = [&](int q, unsigned x) {
+        return slots_raw + ((int64_t)(x & 1) * (C + 1) + q) * nb * RUN_SLOT_BYTES;
+    };
+    // Control warp: publishes the block's maximum and flags and collects every
+    // block's into sh.delta and sh.flags.
+    auto exchange_max = [&](float mx, unsigned fl) {
+        const uint64_t tag = ((uint64_t)nonce << 32) | (nx + 1);
+        char* const row = slot_row(C, nx + 1);
+        unsigned tm = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));  // non-negative floats order as their bits
+        unsigned tf = __reduce_or_sync(0xffffffffu, fl);
+        if (lane == 0) st_slot(row + (int64_t)blockIdx.x * RUN_SLOT_BYTES, __uint_as_float(tm), __uint_as_float(tf), tag);
+        const bool ok = collect(row, nb, tag, sh.lim.grid_spins, sh.lim.phantoms, [&](float p, float r) {
+            tm = max(tm, __float_as_uint(p));
+            tf |= __float_as_uint(r);
+        });
+        tm = __reduce_max_sync(0xffffffffu, tm);
+        tf = __reduce_or_sync(0xffffffffu, tf);
         if (lane == 0) {
-            sh.mx[warp] = __uint_as_float(mb);
-            sh.bad[warp] = any ? 1u : 0u;
+            sh.delta = __uint_as_float(tm);
+            sh.flags = tf;
+            if (!ok) sh.ctl.x = 1;
         }
     };
-
-    // ---- a sums pass from V^k (also pass 0 from V^0, which checks x) ----
-    SumAcc<C> a;
-    auto sums_pass = [&](float dmax, bool check_x) {
-        a.reset();
-        float tn[C], td[C];  // pixels that do not fill a pair
-#pragma unroll
-        for (int j = 0; j < C; ++j) tn[j] = td[j] = 0.0f;
-        bool bad = false;
-        f2 vq2[C], s2;
-        if (SCALED) {
-            const float s = spread_scale<C>(v2);
-            s2 = pack2(s, s);
+    // V^{k+1}_q from the totals (one lane).
+    auto new_center = [&](int q, DF na, DF da, bool centered, int cur, int nxt) {
+        if (da.hi > 0.0f) {
+            DF r = (da.hi > 1e-30f && da.hi < 1e30f) ? df_div_fast(na, da) : df_div(na, da);
+            if (centered) r = df_merge(r, DF{sh.v[cur][q], 0.0f});
+            sh.v[nxt][q] = r.hi;
+            sh.v64[nxt][q] = r;
+        } else {
+            // an empty cluster keeps its center (in pass 0 that is V^0, or 0 from a U^0)
+            sh.v[nxt][q] = centered ? sh.v[cur][q] : 0.0f;
+            sh.v64[nxt][q] = centered ? sh.v64[cur][q] : DF{0.0f, 0.0f};
+            sh.empty[nxt] = 1u;
         }
-#pragma unroll
-        for (int j = 0; j < C; ++j) vq2[j] = SCALED ? mul2(v2[j], s2) : v2[j];
-        auto quad = [&](const float4& c, int64_t) {
-            const f2 xa = pack2(c.x, c.y), xb = pack2(c.z, c.w);
-            if (check_x) bad |= !(finite_f(c.x) && finite_f(c.y) && finite_f(c.z) && finite_f(c.w));
-            f2 um[C], d2[C];
-            powers_pair<C, MK>(xa, SCALED ? mul2(xa, s2) : xa, vq2, m, inv_m1, sh.v, um, d2);
-            a.add(d2, um);
-            powers_pair<C, MK>(xb, SCALED ? mul2(xb, s2) : xb, vq2, m, inv_m1, sh.v, um, d2);
-            a.add(d2, um);
-            if (++a.held == FOLD) a.fold();
-        };
-        auto single = [&](int64_t i) {
-            const float xi = __ldg(px.x + i);
-            if (check_x) bad |= !finite_f(xi);
-            const Powers<C> w = powers_scalar<C, MK>(xi, xi, sh.v, m, inv_m1);
-#pragma unroll
-            for (int j = 0; j < C; ++j) {
-                tn[j] = fmaf(w.a[j], SCALED ? lo2(mul2(pack2(xi, xi), s2)) - lo2(vq2[j]) : xi - lo2(vq2[j]), tn[j]);
-                td[j] += w.a[j];
-            }
-        };
-        if (px.vec_x) for_quads(px, t0, nt, quad, single);
-        else for_tiles(px, t0, nt, quad, single);
-        if (check_x && threadIdx.x < C) bad |= !finite_f(sh.v[threadIdx.x]);
-        a.fold();
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            tn[j] += lo2(a.num[j]) + hi2(a.num[j]);
-            td[j] += lo2(a.den[j]) + hi2(a.den[j]);
-        }
-        warp_publish(tn, td, dmax, bad);
     };
-
+    // Warp q < C (q = 0 for X_J): the block's totals from the warp totals, then
+    // the grid's. X_SUMS*: V^{k+1}_q into sh.v[nxt], sh.v64[nxt]; cur is the slot
+    // of V^k, which centers the numerators. X_J: sh.J.
+    auto exchange_sums = [&](auto kind, int q, int cur, int nxt) {
+        constexpr int K = decltype(kind)::value;
+        const uint64_t tag = ((uint64_t)nonce << 32) | (nx + 1);
+        char* const row = slot_row(q, nx + 1);
+        float a = lane < pw ? sh.red[lane][q] : 0.0f, b = (K != X_J && lane < pw) ? sh.red[lane][C + q] : 0.0f;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (K != X_J) b += __shfl_xor_sync(0xffffffffu, b, o);
+        }
+        if (lane == 0) st_slot(row + (int64_t)blockIdx.x * RUN_SLOT_BYTES, a, b, tag);
+        DF na{0.0f, 0.0f}, da{0.0f, 0.0f};
+        const bool ok = collect(row, nb, tag, sh.lim.grid_spins, sh.lim.phantoms, [&](float p, float r) {
+            df_add(na, p);
+            if (K != X_J) df_add(da, r);
+        });
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            // TwoSum is symmetric: every lane gets the same totals
+            na = df_merge_raw(na, DF{__shfl_xor_sync(0xffffffffu, na.hi, o), __shfl_xor_sync(0xffffffffu, na.lo, o)});
+            if (K != X_J)
+                da = df_merge_raw(da, DF{__shfl_xor_sync(0xffffffffu, da.hi, o), __shfl_xor_sync(0xffffffffu, da.lo, o)});
+        }
+        if (lane != 0) return;
+        if (!ok) sh.ctl.x = 1;
+        na = df_norm(na);
+        if (K == X_J) {
+            sh.J = na;
+            return;
+        }
+        da = df_norm(da);
+        new_center(q, na, da, K == X_SUMS, cur, nxt);
+    };
+    // Polls a pair of words until f(a, b) says that they are complete.
+    auto poll = [&](const uint64_t* w, uint64_t& a, uint64_t& b, auto&& complete) {
+        const uint32_t limit = sh.lim.grid_spins, phantoms = sh.lim.phantoms;
+        for (uint32_t spins = 0;;) {
+            ld_words(w, a, b);
+            if (complete(a, b) && phantoms == 0) return true;
+            if (++spins > limit) return false;
+            if (spins > 256) __nanosleep(100);
+        }
+    };
+    // Warp q < C between iterations: the block's totals into cluster q's words,
+    // then V^{k+1}_q from the complete ones (one lane polls).
+    auto exchange_words = [&](int q, int cur, int nxt) {
+        uint64_t* const w = word(nonce, nx + 1, q);
+        float a = lane < pw ? sh.red[lane][q] : 0.0f, b = lane < pw ? sh.red[lane][C + q] : 0.0f;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, o);
+            b += __shfl_xor_sync(0xffffffffu, b, o);
+        }
+        if (lane != 0) return;
+        red_add_u64(w, (uint64_t)__float2ll_rn(a * to_num) + ARRIVAL);
+        red_add_u64(w + 1, (uint64_t)__float2ll_rn(b * to_den) + ARRIVAL);
+        const bool odd = (nx + 1) & 1;
+        const uint64_t pa = odd ? seen_a1 : seen_a0, pb = odd ? seen_b1 : seen_b0;
+        uint64_t va, vb;
+        const bool ok = poll(w, va, vb, [&](uint64_t x, uint64_t y) {
+            return arrivals(x - pa) == (unsigned)nb && arrivals(y - pb) == (unsigned)nb;
+        });
+        const int64_t sa = (int64_t)(va - pa - (uint64_t)nb * ARRIVAL), sb = (int64_t)(vb - pb - (uint64_t)nb * ARRIVAL);
+        (odd ? seen_a1 : seen_a0) = va;
+        (odd ? seen_b1 : seen_b0) = vb;
+        if (!ok) sh.ctl.x = 1;
+        if (sb < (1ll << 37)) sh.ctl.z = 1;
+        else new_center(q, fixed_to_df(sa, num_unit), fixed_to_df(sb, den_unit), true, cur, nxt);
+    };
+    // Control warp: publishes whether this block's sample of iteration k reached
+    // eps; collects, an iteration later, whether any block's did.
+    auto publish_decision = [&](int k, float mx) {
+        const bool ge = __any_sync(0xffffffffu, mx >= eps);
+        if (lane == 0) red_add_u64(word(nonce, k, C), 1ull + (ge ? 1ull << 16 : 0ull));
+    };
+    auto collect_decision = [&](int k) {
+        if (lane != 0) return;
+        const uint64_t pa = (k & 1) ? seen_a1 : seen_a0;
+        uint64_t va, vb;
+        const bool ok = poll(word(nonce, k, C), va, vb, [&](uint64_t x, uint64_t) { return ((x - pa) & 0xffffu) == (unsigned)nb; });
+        sh.ctl.y = ((va - pa) >> 16) != 0;
+        ((k & 1) ? seen_a1 : seen_a0) = va;
+        if (!ok) sh.ctl.x = 1;
+    };
     // ---- pass 0: V^1 from U^0, or from U^0 = f(x, V^0) ----
-    if (from_u) {
-        // four pixels in FP32, then double-float: the pass waits for memory, and
-        // the separation of the V^1 of a random start is of the order of 1e-5
-        DF sn[C], sd[C];
-        float num[C], den[C];
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            sn[j] = sd[j] = DF{0.0f, 0.0f};
-            num[j] = den[j] = 0.0f;
-        }
+    bool ok;
+    {
         bool bad = false;
-        auto one = [&](float xi, float u0, int j) {
-            bad |= !(u0 >= 0.0f) || !finite_f(u0);
-            const float w = pow_m<MK>(u0, m);
-            num[j] = fmaf(w, xi, num[j]);
-            den[j] += w;
+        float xmax = 0.0f;  // largest |x| (and |V^0|)
+        auto see = [&](float xi) {
+            bad |= !finite_f(xi);
+            xmax = fmaxf(xmax, fabsf(xi));
         };
-        auto fold = [&] {
+        if (control) {
+            if (!from_u && lane < C) see(sh.v[0][lane]);
+        } else if (from_u) {
+            // four pixels in FP32, then double-float: the pass waits for memory, and
+            // the separation of the V^1 of a random start is of the order of 1e-5
+            DF sn[C], sd[C];
+            float num[C], den[C];
 #pragma unroll
             for (int j = 0; j < C; ++j) {
-                df_add(sn[j], num[j]);
-                df_add(sd[j], den[j]);
+                sn[j] = sd[j] = DF{0.0f, 0.0f};
                 num[j] = den[j] = 0.0f;
             }
-        };
-        auto quad_v = [&](const float4& c, int64_t i) {
-            bad |= !(finite_f(c.x) && finite_f(c.y) && finite_f(c.z) && finite_f(c.w));
-            float4 u[C];
+            auto one = [&](float xi, float u0, int j) {
+                bad |= !(u0 >= 0.0f) || !finite_f(u0);
+                const float w = pow_m<MK>(u0, m);
+                num[j] = fmaf(w, xi, num[j]);
+                den[j] += w;
+            };
+            auto fold = [&] {
 #pragma unroll
-            for (int j = 0; j < C; ++j) u[j] = __ldcs(reinterpret_cast<const float4*>(U0 + (int64_t)j * n + i));
+                for (int j = 0; j < C; ++j) {
+                    df_add(sn[j], num[j]);
+                    df_add(sd[j], den[j]);
+                    num[j] = den[j] = 0.0f;
+                }
+            };
+            auto single = [&](int64_t i) {
+                const float xi = __ldg(px.x + i);
+                see(xi);
 #pragma unroll
-            for (int j = 0; j < C; ++j) {
-                one(c.x, u[j].x, j);
-                one(c.y, u[j].y, j);
-                one(c.z, u[j].z, j);
-                one(c.w, u[j].w, j);
+                for (int j = 0; j < C; ++j) one(xi, __ldcs(U0 + (int64_t)j * n + i), j);
+            };
+            if (px.vec_u) {
+                px.stage([&](const float4& c, int64_t i) {
+                    see(c.x), see(c.y), see(c.z), see(c.w);
+                    float4 u[C];
+#pragma unroll
+                    for (int j = 0; j < C; ++j) u[j] = __ldcs(reinterpret_cast<const float4*>(U0 + (int64_t)j * n + i));
+#pragma unroll
+                    for (int j = 0; j < C; ++j) {
+                        one(c.x, u[j].x, j);
+                        one(c.y, u[j].y, j);
+                        one(c.z, u[j].z, j);
+                        one(c.w, u[j].w, j);
+                    }
+                    fold();
+                });
+            } else {
+                px.stage([&](const float4&, int64_t) {});
+                px.tiles(
+                    [&](const float4& c, int64_t i) {
+                        see(c.x), see(c.y), see(c.z), see(c.w);
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) {
+#pragma unroll
+                            for (int j = 0; j < C; ++j) one(comp(c, p), __ldcs(U0 + (int64_t)j * n + i + 32 * p), j);
+                        }
+                        fold();
+                    },
+                    single);
             }
             fold();
-        };
-        auto quad_t = [&](const float4& c, int64_t i) {
-            bad |= !(finite_f(c.x) && finite_f(c.y) && finite_f(c.z) && finite_f(c.w));
+            float t[P];
 #pragma unroll
-            for (int p = 0; p < 4; ++p) {
-#pragma unroll
-                for (int j = 0; j < C; ++j) one(comp(c, p), __ldcs(U0 + (int64_t)j * n + i + 32 * p), j);
+            for (int i = 0; i < P; ++i) {
+                const DF q = i < C ? sn[i < C ? i : 0] : sd[(i >= C && i < 2 * C) ? i - C : 0];
+                t[i] = i < 2 * C ? q.hi + q.lo : 0.0f;
             }
-            fold();
-        };
-        auto single = [&](int64_t i) {
-            const float xi = __ldg(px.x + i);
-            bad |= !finite_f(xi);
-#pragma unroll
-            for (int j = 0; j < C; ++j) one(xi, __ldcs(U0 + (int64_t)j * n + i), j);
-        };
-        if (px.vec_u) for_quads(px, t0, nt, quad_v, single);
-        else for_tiles(px, t0, nt, quad_t, single);
-        fold();
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            num[j] = sn[j].hi + sn[j].lo;
-            den[j] = sd[j].hi + sd[j].lo;
+            warp_sums<C>(sh, t);
+        } else {
+            sums_pass_body<C, MK, true>(px, sh, second, 0, m, inv_m1, see);
         }
-        warp_publish(num, den, 0.0f, bad);
-    } else {
-        sums_pass(0.0f, true);
+        const unsigned wx = __reduce_max_sync(0xffffffffu, __float_as_uint(xmax));
+        const bool wbad = __any_sync(0xffffffffu, bad);
+        if (!control && lane == 0) {
+            sh.bad[warp] = wbad ? 1u : 0u;
+            sh.mx[warp] = __uint_as_float(wx);
+        }
+        __syncthreads();
+        if (control) exchange_max(fmaxf(xmax, lane < pw ? sh.mx[lane] : 0.0f), (wbad ? 1u : 0u) | (lane < pw ? sh.bad[lane] : 0u));
+        else if (warp < C && from_u) exchange_sums(std::integral_constant<int, X_SUMS0>(), warp, 0, 1);
+        else if (warp < C) exchange_sums(std::integral_constant<int, X_SUMS>(), warp, 0, 1);
+        ++nx;
+        __syncthreads();
+        ok = sh.ctl.x == 0;
     }
-    bool ok = exchange(true, !from_u);
-
+    // The fixed-point units: |num_j| <= 2 n max(|x|, |V^0|) and den_j <= n, so the
+    // totals stay below 2^53 units. Images whose FP32 sums could overflow get
+    // scale 0: every total is then thin, and goes through the slots.
+    {
+        const int en = 64 - __clzll(n);                                        // n < 2^en
+        const int ex = max(-100, (__float_as_int(sh.delta) >> 23) - 125);      // 2 max|x| < 2^ex
+        const int e = max(-126, min(126, 53 - en - ex));
+        const bool use = en + ex <= 126;
+        to_num = use ? pow2f(e) : 0.0f;
+        num_unit = pow2f(-e);
+        to_den = use ? pow2f(53 - en) : 0.0f;
+        den_unit = pow2f(en - 53);
+    }
     int status = FCM_NOT_CONVERGED, iters = 0;
     if (!ok) {
         status = FCM_ERR_TIMEOUT;
@@ -491,203 +725,254 @@ __global__ void __launch_bounds__(RUN_NT, 1) k_fcm_run(RunState* __restrict__ st
         status = FCM_ERR_BAD_INPUT;
         ok = false;
     }
-    // V^{k+1} of the last exchange becomes V^k (an empty cluster keeps its
-    // center; in pass 0 that is V^0, or 0 from a U^0).
-    auto advance = [&](bool first) {
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            const float old = lo2(v2[j]);
-            float nv = old;
-            if (sh.empty[j]) {
-                flags |= FCM_FLAG_EMPTY_CLUSTER;
-                if (first && from_u) {
-                    nv = 0.0f;
-                    v64[j] = DF{0.0f, 0.0f};
-                }
-            } else {
-                v64[j] = sh.vq[j];
-                nv = v64[j].hi;
-            }
-            if (threadIdx.x == 0) {
-                sh.vp[j] = old;
-                sh.v[j] = nv;
-            }
-            v2[j] = pack2(nv, nv);
-        }
-        __syncthreads();
-    };
-
-    // The sampled pair of this thread: the first pair that a full pass gives it
-    // (the same pairs, so the sample's changes are bit for bit those of the full
-    // pass), until a full pass has found its pair of largest change.
+    // The control warp samples the change of one pair per lane. The pairs are
+    // spread evenly over the image and are pairs of the full pass (so their
+    // changes are bit for bit the full pass's); after a full pass that did not
+    // stop the run, the lanes of the pixel warps' numbers hold those warps' pairs
+    // of largest change.
     f2 wx = 0;
-    const int64_t wi = px.vec_u ? 4 * t0 : ((t0 >> 5) << 7) + lane;
-    const int ws = px.vec_u ? 1 : 32;
-    bool sampled = px.vec_u ? t0 < (n >> 2) : ((t0 >> 5) << 7) + 128 <= n;
-    bool wide = false;  // every warp samples (after a full pass that did not stop the run)
-    if (sampled) wx = pack2(__ldg(px.x + wi), __ldg(px.x + wi + ws));
+    int64_t wi = 0;
+    int ws = 1;
+    bool sampled = false;
+    if (control) {
+        const double at = ((double)blockIdx.x * 32 + lane) / ((double)nb * 32);
+        const int64_t i = (int64_t)(at * (double)n);
+        if (px.vec_u) {
+            wi = min(i, n - 2) & ~(int64_t)1;
+            sampled = true;
+        } else {
+            const int64_t whole = n >> 7;
+            wi = (min(i >> 7, whole - 1) << 7) + lane;
+            ws = 32;
+            sampled = whole > 0;
+        }
+        if (sampled) wx = pack2(__ldg(px.x + wi), __ldg(px.x + wi + ws));
+    }
+
     // U^k of a pair and its largest |U^k - U^{k-1}|; U^{k-1} is given (u0) or
     // comes from V^{k-1}. J2: the pair's J terms.
-    auto change = [&](f2 xq, f2 (&u2)[C], const f2 (&u0)[C], bool given, f2& J2) {
-        f2 um2[C], uo2[C], vp2[C];
-        J2 = membership_pair<C, MK>(xq, v2, m, inv_m1, sh.v, u2, um2);
+    auto change = [&](f2 xq, const PackedCenters<C, MK>& cen, const PackedCenters<C, MK>& pre, f2 (&u2)[C],
+                      const f2 (&u0)[C], bool given, f2& J2) {
+        f2 w[1][C], o[1][C], t[1][C], j2[1];
+        const f2 xa[1] = {xq};
+        packed_pairs<C, MK, false, 1>(xa, cen, m, inv_m1, w, t, j2);
+        J2 = j2[0];
         if (given) {
 #pragma unroll
-            for (int j = 0; j < C; ++j) uo2[j] = u0[j];
+            for (int j = 0; j < C; ++j) o[0][j] = u0[j];
         } else {
-#pragma unroll
-            for (int j = 0; j < C; ++j) vp2[j] = pack2(sh.vp[j], sh.vp[j]);
-            membership_pair<C, MK>(xq, vp2, m, inv_m1, sh.vp, uo2, um2);
+            packed_pairs<C, MK, false, 1>(xa, pre, m, inv_m1, o, t, j2);
         }
         float d = 0.0f;
 #pragma unroll
         for (int j = 0; j < C; ++j) {
             float da, db;
-            unpack2(sub2(u2[j], uo2[j]), da, db);
+            u2[j] = w[0][j];
+            unpack2(sub2(w[0][j], o[0][j]), da, db);
             d = fmaxf(d, fmaxf(fabsf(da), fabsf(db)));
         }
         return d;
     };
-    if (ok) advance(true);
-    for (int k = 1; ok; ++k) {
-        const bool last = k == max_iter, prev_u0 = from_u && k == 1;
-        bool go_on = false;
-        if (!last) {
-            float dmax = 0.0f;
-            if (sampled && (wide || warp < SAMPLE_WARPS)) {
-                f2 u0[C], u2[C];
-                if (prev_u0) {
-#pragma unroll
-                    for (int j = 0; j < C; ++j)
-                        u0[j] = pack2(__ldcs(U0 + (int64_t)j * n + wi), __ldcs(U0 + (int64_t)j * n + wi + ws));
-                }
-                f2 J2;
-                dmax = change(wx, u2, u0, prev_u0, J2);
-            }
-            sums_pass(dmax, false);
-            if (!exchange(true, true)) {
-                status = FCM_ERR_TIMEOUT;
-                iters = k;
-                break;
-            }
-            go_on = sh.delta >= eps;
-        }
-        if (!go_on || trace) {
-            // ---- full pass: delta_k and J_k over every pixel, U^k ----
-            const bool emit = !go_on;
-            f2 J2 = pack2(0.0f, 0.0f);
-            float J1 = 0.0f, dmax = 0.0f;
+    // The full pass of iteration k: delta_k and J_k over every pixel, and U^k.
+    // False when a wait gave up.
+    auto full_pass = [&](int k) {
+        const int cur = k & 3, prv = (k - 1) & 3;
+        const bool prev_u0 = from_u && k == 1;
+        if (!control) {
+            f2 J2 = pack2(0.0f, 0.0f), best = 0;
+            float J1 = 0.0f, dmax = -1.0f, dtail = 0.0f;
+            PackedCenters<C, MK> cen, pre;
+            cen.set(sh.v[cur]);
+            pre.set(sh.v[prv]);
             auto pair = [&](f2 xq, f2 (&u2)[C], const f2 (&u0)[C]) {
                 f2 j2;
-                const float d = change(xq, u2, u0, prev_u0, j2);
+                const float d = change(xq, cen, pre, u2, u0, prev_u0, j2);
                 J2 = add2(J2, j2);
                 if (d > dmax) {
                     dmax = d;
-                    wx = xq;
-                    sampled = true;
-                }
-            };
-            auto quad_v = [&](const float4& c, int64_t i) {
-                f2 ua[C], ub[C], u0a[C], u0b[C];
-                if (prev_u0) {
-#pragma unroll
-                    for (int j = 0; j < C; ++j) {
-                        const float4 u = __ldcs(reinterpret_cast<const float4*>(U0 + (int64_t)j * n + i));
-                        u0a[j] = pack2(u.x, u.y);
-                        u0b[j] = pack2(u.z, u.w);
-                    }
-                }
-                pair(pack2(c.x, c.y), ua, u0a);
-                pair(pack2(c.z, c.w), ub, u0b);
-                if (emit) {
-#pragma unroll
-                    for (int j = 0; j < C; ++j) st_u4(U + (int64_t)j * n + i, make_float4(lo2(ua[j]), hi2(ua[j]), lo2(ub[j]), hi2(ub[j])));
-                }
-            };
-            auto quad_t = [&](const float4& c, int64_t i) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    f2 u[C], u0[C];
-                    const int64_t ia = i + 64 * h, ib = ia + 32;
-                    if (prev_u0) {
-#pragma unroll
-                        for (int j = 0; j < C; ++j) u0[j] = pack2(__ldcs(U0 + (int64_t)j * n + ia), __ldcs(U0 + (int64_t)j * n + ib));
-                    }
-                    pair(h ? pack2(c.z, c.w) : pack2(c.x, c.y), u, u0);
-                    if (emit) {
-#pragma unroll
-                        for (int j = 0; j < C; ++j) {
-                            __stcs(U + (int64_t)j * n + ia, lo2(u[j]));
-                            __stcs(U + (int64_t)j * n + ib, hi2(u[j]));
-                        }
-                    }
+                    best = xq;
                 }
             };
             auto single = [&](int64_t i) {
                 const float xi = __ldg(px.x + i);
-                float u[C], um[C], up[C], ump[C];
-                float vv[C], vvp[C];
-#pragma unroll
-                for (int j = 0; j < C; ++j) {
-                    vv[j] = sh.v[j];
-                    vvp[j] = sh.vp[j];
-                }
-                J1 += membership<C, MK>(xi, vv, m, inv_m1, u, um);
+                const PixelPair<C> a = scalar_pair<C, MK, false>(xi, xi, cen.vs, m, inv_m1);
+                J1 += a.Ja;
                 if (prev_u0) {
 #pragma unroll
-                    for (int j = 0; j < C; ++j) up[j] = __ldcs(U0 + (int64_t)j * n + i);
+                    for (int j = 0; j < C; ++j) dtail = fmaxf(dtail, fabsf(a.a[j] - __ldcs(U0 + (int64_t)j * n + i)));
                 } else {
-                    membership<C, MK>(xi, vvp, m, inv_m1, up, ump);
-                }
-                float d = 0.0f;
+                    const PixelPair<C> b = scalar_pair<C, MK, false>(xi, xi, pre.vs, m, inv_m1);
 #pragma unroll
-                for (int j = 0; j < C; ++j) {
-                    d = fmaxf(d, fabsf(u[j] - up[j]));
-                    if (emit) __stcs(U + (int64_t)j * n + i, u[j]);
+                    for (int j = 0; j < C; ++j) dtail = fmaxf(dtail, fabsf(a.a[j] - b.a[j]));
                 }
-                dmax = fmaxf(dmax, d);
+                {
+#pragma unroll
+                    for (int j = 0; j < C; ++j) __stcs(U + (int64_t)j * n + i, a.a[j]);
+                }
             };
-            if (px.vec_u) for_quads(px, t0, nt, quad_v, single);
-            else for_tiles(px, t0, nt, quad_t, single);
-            wide = true;
+            if (px.vec_u) {
+                px.quads([&](const float4& c, int64_t i) {
+                    f2 ua[C], ub[C], u0a[C], u0b[C];
+                    if (prev_u0) {
+#pragma unroll
+                        for (int j = 0; j < C; ++j) {
+                            const float4 u = __ldcs(reinterpret_cast<const float4*>(U0 + (int64_t)j * n + i));
+                            u0a[j] = pack2(u.x, u.y);
+                            u0b[j] = pack2(u.z, u.w);
+                        }
+                    }
+                    pair(pack2(c.x, c.y), ua, u0a);
+                    pair(pack2(c.z, c.w), ub, u0b);
+                    {
+#pragma unroll
+                        for (int j = 0; j < C; ++j)
+                            st_u4(U + (int64_t)j * n + i, make_float4(lo2(ua[j]), hi2(ua[j]), lo2(ub[j]), hi2(ub[j])));
+                    }
+                });
+            } else {
+                px.tiles(
+                    [&](const float4& c, int64_t i) {
+#pragma unroll 1
+                        for (int h = 0; h < 2; ++h) {
+                            f2 u[C], u0[C];
+                            const int64_t ia = i + 64 * h, ib = ia + 32;
+                            if (prev_u0) {
+#pragma unroll
+                                for (int j = 0; j < C; ++j)
+                                    u0[j] = pack2(__ldcs(U0 + (int64_t)j * n + ia), __ldcs(U0 + (int64_t)j * n + ib));
+                            }
+                            pair(h ? pack2(c.z, c.w) : pack2(c.x, c.y), u, u0);
+                            {
+#pragma unroll
+                                for (int j = 0; j < C; ++j) {
+                                    __stcs(U + (int64_t)j * n + ia, lo2(u[j]));
+                                    __stcs(U + (int64_t)j * n + ib, hi2(u[j]));
+                                }
+                            }
+                        }
+                    },
+                    single);
+            }
             J1 = warp_sum(J1 + lo2(J2) + hi2(J2));
-            const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(dmax));
+            const float own = fmaxf(dmax, 0.0f);
+            const unsigned wb = __reduce_max_sync(0xffffffffu, __float_as_uint(own));
+            const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(own, dtail)));
+            const unsigned who = __ballot_sync(0xffffffffu, dmax >= 0.0f && __float_as_uint(own) == wb);
+            if (lane == (who ? __ffs(who) - 1 : 0)) sh.wit[warp] = best;
             if (lane == 0) {
                 sh.red[warp][0] = J1;
                 sh.mx[warp] = __uint_as_float(mb);
-                sh.bad[warp] = 0u;
+                sh.bad[warp] = who ? 2u : 0u;
             }
-            if (!exchange(false, false)) {
-                status = FCM_ERR_TIMEOUT;
-                iters = k;
-                break;
-            }
-            const float delta = sh.delta;
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                st->delta = delta;
-                st->J = df_to_double(sh.J);
-                if (trace) {
-                    double* t = trace + (int64_t)(k - 1) * (2 + C);
-                    t[0] = delta;
-                    t[1] = df_to_double(sh.J);
-#pragma unroll
-                    for (int j = 0; j < C; ++j) t[2 + j] = df_to_double(v64[j]);
-                }
-            }
-            if (!go_on && (delta < eps || last)) {
-                status = delta < eps ? FCM_OK : FCM_NOT_CONVERGED;
-                iters = k;
-                break;
-            }
-            // the run goes on from the V^{k+1} of the sums pass (still in sh.vq)
         }
-        advance(false);
+        __syncthreads();
+        if (control) {
+            if (lane < pw && (sh.bad[lane] & 2u)) {
+                wx = sh.wit[lane];
+                sampled = true;
+            }
+            exchange_max(lane < pw ? sh.mx[lane] : 0.0f, 0u);
+        } else if (warp == 0) {
+            exchange_sums(std::integral_constant<int, X_J>(), 0, 0, 0);
+        }
+        ++nx;
+        __syncthreads();
+        if (sh.ctl.x) return false;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            st->delta = sh.delta;
+            st->J = df_to_double(sh.J);
+            if (tracing) {
+                double* t = st->trace + (int64_t)(k - 1) * (2 + C);
+                t[0] = sh.delta;
+                t[1] = df_to_double(sh.J);
+#pragma unroll
+                for (int j = 0; j < C; ++j) t[2 + j] = df_to_double(sh.v64[cur][j]);
+            }
+        }
+        return true;
+    };
+    // Iterations. The decision of iteration k - whether its sample shows that the
+    // run goes on - is collected an iteration later, so that the control warp's
+    // sample and exchange are never waited for: iteration k + 1 runs meanwhile, and
+    // is dropped when the full pass of iteration k stops the run.
+    auto give_up = [&](int k) {
+        status = FCM_ERR_TIMEOUT;
+        iters = k;
+        return false;
+    };
+    if (ok && threadIdx.x == 0 && sh.empty[1]) flags |= FCM_FLAG_EMPTY_CLUSTER;
+    for (int k = 1; ok; ++k) {
+        const bool last = k == max_iter, prev_u0 = from_u && k == 1;
+        const int cur = k & 3, prv = (k - 1) & 3, nxt = (k + 1) & 3;
+        if (!last) {
+            if (control) {
+                float d = 0.0f;
+                if (sampled) {
+                    PackedCenters<C, MK> cen, pre;
+                    cen.set(sh.v[cur]);
+                    pre.set(sh.v[prv]);
+                    f2 u0[C], u2[C], J2;
+                    if (prev_u0) {
+#pragma unroll
+                        for (int j = 0; j < C; ++j)
+                            u0[j] = pack2(__ldcs(U0 + (int64_t)j * n + wi), __ldcs(U0 + (int64_t)j * n + wi + ws));
+                    }
+                    d = change(wx, cen, pre, u2, u0, prev_u0, J2);
+                }
+                publish_decision(k, d);
+                if (k > 1) collect_decision(k - 1);
+                __syncthreads();
+            } else {
+                if (threadIdx.x == 0) sh.empty[nxt] = 0u;
+                sums_pass<C, MK>(px, sh, second, cur, m, inv_m1);
+                __syncthreads();
+                if (warp < C) exchange_words(warp, cur, nxt);
+            }
+        } else {
+            if (control && k > 1) collect_decision(k - 1);
+            __syncthreads();
+        }
+        ++nx;
+        __syncthreads();
+        int4 ctl = sh.ctl;
+        if (ctl.x) {
+            ok = give_up(k);
+            break;
+        }
+        if (ctl.z) {
+            // uniform over the grid: every block has read the same words
+            __syncthreads();
+            if (threadIdx.x == 0) sh.ctl.z = 0;
+            if (warp < C) exchange_sums(std::integral_constant<int, X_SUMS>(), warp, cur, nxt);
+            ++nx;
+            __syncthreads();
+            if (sh.ctl.x) {
+                ok = give_up(k);
+                break;
+            }
+        }
+        // Iteration k - 1's full pass when its sample could not decide, iteration
+        // k's when it is the last (and every one for a trace).
+        const int from = (k > 1 && !ctl.y && !tracing) ? k - 1 : k, to = (last || tracing) ? k : k - 1;
+#pragma unroll 1
+        for (int r = from; ok && r <= to; ++r) {
+            if (!full_pass(r)) {
+                ok = give_up(r);
+            } else if (sh.delta < eps || r == max_iter) {
+                status = sh.delta < eps ? FCM_OK : FCM_NOT_CONVERGED;
+                iters = r;
+                ok = false;
+            } else if (r < k && threadIdx.x == 0 && sh.empty[cur]) {
+                flags |= FCM_FLAG_EMPTY_CLUSTER;
+            }
+        }
+        if (from == k && k > 1 && threadIdx.x == 0 && sh.empty[cur]) flags |= FCM_FLAG_EMPTY_CLUSTER;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
 #pragma unroll
         for (int j = 0; j < C; ++j) {
-            st->V[j] = lo2(v2[j]);
-            st->V64[j] = df_to_double(v64[j]);
+            st->V[j] = sh.v[iters & 3][j];
+            st->V64[j] = df_to_double(sh.v64[iters & 3][j]);
         }
         st->status = status;
         st->iters = iters;

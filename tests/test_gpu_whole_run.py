@@ -82,3 +82,22 @@ def test_largest_change_outside_the_sample(fcm, n, at):
     V0 = np.array([60.3, 150.1])
     g = _check(fcm, x, 2, 2.0, V0=V0)
     assert g.status == 0 and g.delta < EPS
+
+
+def test_cluster_of_one_pixel(fcm):
+    """A cluster whose share of the image is below what the fixed-point exchange
+    words carry goes through the slots, in every iteration."""
+    rng = np.random.default_rng(11)
+    x = np.rint(rng.random(200004) * 100.0)
+    x[77777] = 5000.0
+    g = _check(fcm, x, 3, 2.0, V0=np.array([20.3, 80.1, 4900.5]))
+    assert abs(float(g.V[2]) - 5000.0) < 50.0
+
+
+@pytest.mark.parametrize("m", [2.0, 1.5, 2.5])
+@pytest.mark.parametrize("C", [1, 2, 6, 8])
+def test_cluster_counts(fcm, C, m):
+    means = tuple(12.0 + 32.0 * j for j in range(C))
+    img, _ = phantom.phantom2d(4500 + C, 90, 91, 4.0, means=means)
+    x = img.reshape(-1)
+    _check(fcm, x, C, m, V0=np.array(means) + 3.3)
