@@ -67,7 +67,7 @@ struct BatchedWorkspace {
     // graph serves every batch of a slice count), rank slots and barrier counters
     int4* d_items = nullptr;
     int4* h_items = nullptr;  // pinned
-    float2* d_tslots = nullptr;
+    float4* d_tslots = nullptr;
     unsigned* d_tctr = nullptr;
     int team_cap = 0;
     std::map<int, int> tgrid;  // block -> CTAs of a full cooperative team grid
@@ -315,7 +315,7 @@ int fill_teams(fcm_ctx* h, int n, const fcm_batch_plan& p) {
         const int cap = std::max(n, 64);
         CK(dev_malloc(h, &w->d_items, sizeof(int4) * (size_t)cap * TEAM_MAX));
         CK(host_malloc(h, &w->h_items, sizeof(int4) * (size_t)cap * TEAM_MAX));
-        CK(dev_malloc(h, &w->d_tslots, sizeof(float2) * (size_t)cap * TEAM_MAX * 2 * TEAM_SLOT));
+        CK(dev_malloc(h, &w->d_tslots, sizeof(float4) * (size_t)cap * TEAM_MAX * 2 * TEAM_SLOT));
         CK(dev_malloc(h, &w->d_tctr, sizeof(unsigned) * cap));
         w->team_cap = cap;
     }

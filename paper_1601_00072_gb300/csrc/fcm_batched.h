@@ -164,7 +164,7 @@ struct alignas(16) RoundsHdr {
 // ---- team schedule (a slice shared by any number of CTAs of the grid) ----
 
 constexpr int TEAM_MAX = 32;                        // largest team
-constexpr int TEAM_SLOT = 2 * FCM_MAX_CLUSTERS + 3;  // values a rank publishes per pass
+constexpr int TEAM_SLOT = FCM_MAX_CLUSTERS + 1;  // 16-byte values a rank publishes per pass
 
 struct TeamArgs {
     const SliceDesc* descs;
@@ -173,7 +173,7 @@ struct TeamArgs {
     const int4* items;      // (slice, seat, team size, 0), seats of a slice in a row
     const RoundsHdr* hdr;   // n_slices; max_rounds = number of items; wait_spins, phantoms
     const int* slot_base;   // [n_slices]: first rank slot of each slice
-    float2* slots;          // [sum of team sizes][2][TEAM_SLOT]
+    float4* slots;          // [sum of team sizes][2][TEAM_SLOT]
     unsigned* counters;     // [n_slices] barrier arrivals (zero before the batch)
 };
 

@@ -25,6 +25,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fcm.h"
+
 namespace fcm {
 
 enum MKind : int { M_TWO = 0, M_THREE = 1, M_ONE_HALF = 2, M_GENERIC = 3, M_KINDS = 4 };
@@ -270,6 +272,47 @@ struct PixelPair {
     float a[C], b[C];  // u^m or u of the two pixels
     float Ja, Jb;
 };
+#ifdef FCM_ONE_SCALAR_PAIR
+// One function for every cluster count and fuzzifier, for the kernels that hold
+// all of them (nested calls of 32 variants compile for minutes): the C centers are
+// padded with infinitely distant ones, whose weights are exactly 0.
+static __device__ __noinline__ PixelPair<FCM_MAX_CLUSTERS> scalar_pair_any(float xa, float xb, const float* vs, int C,
+                                                                          int mk, bool powers, float m, float inv_m1) {
+    constexpr int N = FCM_MAX_CLUSTERS;
+    float v[N], u[N], um[N];
+    PixelPair<N> w;
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = j < C ? vs[j] : __int_as_float(0x7f800000);
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        const float x = h ? xb : xa;
+        float J;
+        switch (mk) {
+            case M_TWO: J = membership<N, M_TWO>(x, v, m, inv_m1, u, um); break;
+            case M_THREE: J = membership<N, M_THREE>(x, v, m, inv_m1, u, um); break;
+            case M_ONE_HALF: J = membership<N, M_ONE_HALF>(x, v, m, inv_m1, u, um); break;
+            default: J = membership<N, M_GENERIC>(x, v, m, inv_m1, u, um); break;
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j) (h ? w.b : w.a)[j] = powers ? um[j] : u[j];
+        (h ? w.Jb : w.Ja) = J;
+    }
+    return w;
+}
+template <int C, int MK, bool POWERS>
+__device__ __forceinline__ PixelPair<C> scalar_pair(float xa, float xb, const float* vs, float m, float inv_m1) {
+    const PixelPair<FCM_MAX_CLUSTERS> q = scalar_pair_any(xa, xb, vs, C, MK, POWERS, m, inv_m1);
+    PixelPair<C> w;
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+        w.a[j] = q.a[j];
+        w.b[j] = q.b[j];
+    }
+    w.Ja = q.Ja;
+    w.Jb = q.Jb;
+    return w;
+}
+#else
 template <int C, int MK, bool POWERS>
 __device__ __noinline__ PixelPair<C> scalar_pair(float xa, float xb, const float* vs, float m, float inv_m1) {
     float v[C], t[C];
@@ -285,6 +328,7 @@ __device__ __noinline__ PixelPair<C> scalar_pair(float xa, float xb, const float
     }
     return w;
 }
+#endif
 
 // Power-of-two factor that brings the centers' spread to [1, 2), for the
 // products at m = 1.5 (1 when the spread is 0 or extreme). Scaling by it is
