@@ -30,6 +30,7 @@
 #include <cstring>
 #include <vector>
 
+#define FCM_ONE_SCALAR_PAIR
 #include "fcm_batched.h"
 #include "fcm_bounds.cuh"
 #include "fcm_device.cuh"
@@ -74,7 +75,8 @@ __device__ __noinline__ void pass_a_chunk(const BinArgs& a, const SliceDesc& d, 
     DF acc[2 * C];
 #pragma unroll
     for (int q = 0; q < 2 * C; ++q) acc[q] = DF{0.0f, 0.0f};
-    bool bad_x = false, bad_u = false;
+    bool bad_x = false;
+    float umin = 0.0f, umax = 0.0f;  // a NaN shows in the sums of V^1 instead
     unsigned* hw = sh.sub[warp];
     constexpr int LOADS = loads_a<C>();
     for (int i0 = lo + t; i0 < hi; i0 += BNT * LOADS) {
@@ -99,12 +101,13 @@ __device__ __noinline__ void pass_a_chunk(const BinArgs& a, const SliceDesc& d, 
             bad_x |= g < 0;
             if (g < 0) continue;
             atomicAdd(&hw[g], 1u);
-            sh.rep[g] = i;  // any pixel of the grey level will do
+            if (q == 0) sh.rep[g] = i;  // some pixels of some grey levels: any will do for the bound
             if (from_u) {
 #pragma unroll
                 for (int j = 0; j < C; ++j) {
                     const float u0 = uc[q][j];
-                    bad_u |= !(u0 >= 0.0f) || !finite_f(u0);
+                    umin = fminf(umin, u0);
+                    umax = fmaxf(umax, u0);
                     const float w = pow_m<MK>(u0, m);
                     num[j] = fmaf(w, xi, num[j]);
                     den[j] += w;
@@ -126,8 +129,8 @@ __device__ __noinline__ void pass_a_chunk(const BinArgs& a, const SliceDesc& d, 
             if (lane == 0) sh.wsum[warp][q] = dd;
         }
     }
-    // bit 0: some x is not a grey level; bit 1: U^0 has a negative or non-finite value
-    const int bx = __syncthreads_or(bad_x), bu = __syncthreads_or(bad_u);
+    // bit 0: some x is not a grey level; bit 1: U^0 has a negative or infinite value
+    const int bx = __syncthreads_or(bad_x), bu = __syncthreads_or(umin < 0.0f || !finite_f(umax));
     if ((bx || bu) && t == 0) atomicOr(&a.bad[s], (bx ? 1u : 0u) | (bu ? 2u : 0u));
     {
         unsigned c = 0;
@@ -179,15 +182,15 @@ __global__ void __launch_bounds__(BNT, 3) k_bins_pass_a(BinArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// Solve: one CTA per run, thread b holding grey level b
+// Solve: one CTA per run, thread t holding grey levels 2t and 2t + 1
 // ---------------------------------------------------------------------------
 
-constexpr int SNT = HNT;
+constexpr int SNT = BIN_NT;
 
 template <int C, int MK>
 __device__ __noinline__ void solve_run(const BinArgs& a, int r, const BinRun& run, const SliceDesc& d,
                                        BinScratch& sc, DF* s_tot) {
-    const int s = run.slice, b = threadIdx.x;
+    const int s = run.slice, t = threadIdx.x;
     const bool from_u = run.init == BIN_FROM_U;
     const float m = d.m, inv_m1 = d.inv_m1;
     SliceResult& res = a.results[r];
@@ -201,14 +204,28 @@ __device__ __noinline__ void solve_run(const BinArgs& a, int r, const BinRun& ru
     if (!from_u) {
 #pragma unroll
         for (int j = 0; j < C; ++j) bad |= !finite_f(v0[j]);
+    } else if (!bad) {
+        // thread q < 2C merges sum q over the slice's chunks, in chunk order
+        if (t < 2 * C) {
+            DF mine{0.0f, 0.0f};
+            for (int c = a.chunk_base[s]; c < a.chunk_base[s + 1]; ++c) {
+                const float2 p = a.part[(int64_t)c * 2 * FCM_MAX_CLUSTERS + t];
+                mine = df_merge(mine, DF{p.x, p.y});
+            }
+            s_tot[t] = mine;
+        }
+        __syncthreads();
+        // a NaN in U^0 shows in its denominator (pass A looks at the other bad values)
+#pragma unroll
+        for (int j = 0; j < C; ++j) bad |= s_tot[C + j].hi != s_tot[C + j].hi;
     }
     if (bad) {
         // not a grey-level slice (or a bad U^0 / V^0): the status, and V = V^0
-        if (b < C) {
-            if (run.write_u) d.V[b] = v0[b];
-            res.V64[b] = v0[b];
+        if (t < C) {
+            if (run.write_u) d.V[t] = v0[t];
+            res.V64[t] = v0[t];
         }
-        if (b == 0) {
+        if (t == 0) {
             res.iters = 0;
             res.status = FCM_ERR_BAD_INPUT;
             res.flags = 0;
@@ -217,59 +234,32 @@ __device__ __noinline__ void solve_run(const BinArgs& a, int r, const BinRun& ru
         }
         return;
     }
-    const float cnt = (float)a.hist[(int64_t)s * 256 + b];
+    const uint2 c2 = *reinterpret_cast<const uint2*>(a.hist + (int64_t)s * 256 + 2 * t);
+    const f2 cnt2 = pack2((float)c2.x, (float)c2.y), b2 = pack2((float)(2 * t), (float)(2 * t + 1));
     int par = 0, flags = 0;
-    float v[C], up[C];
-    DF v64[C];
+    float v[C];
+    f2 up2[C];
+    DF mine = bin_mine<C>(v0);
+    const int g = (t & 31) >> 2;  // the cluster whose double-float center this lane holds
 
     // ---- V^1 (Eq. 3): from the chunk sums of pass A, or from the bins with U^0 = f(b, V^0) ----
     if (from_u) {
-        // thread q < 2C merges sum q over the slice's chunks, in chunk order
-        if (b < 2 * C) {
-            DF mine{0.0f, 0.0f};
-            for (int c = a.chunk_base[s]; c < a.chunk_base[s + 1]; ++c) {
-                const float2 p = a.part[(int64_t)c * 2 * FCM_MAX_CLUSTERS + b];
-                mine = df_merge(mine, DF{p.x, p.y});
-            }
-            s_tot[b] = mine;
-        }
-        __syncthreads();
 #pragma unroll
         for (int j = 0; j < C; ++j) {
-            up[j] = 0.0f;
+            up2[j] = pack2(0.0f, 0.0f);
             if (s_tot[C + j].hi > 0.0f) {
-                v64[j] = df_div(s_tot[j], s_tot[C + j]);
-                v[j] = v64[j].hi;
+                const DF q = df_div(s_tot[j], s_tot[C + j]);
+                v[j] = q.hi;
+                if (g == j) mine = q;
             } else {
                 v[j] = v0[j];  // an empty cluster keeps 0 from a U^0
-                v64[j] = DF{v0[j], 0.0f};
                 flags = FCM_FLAG_EMPTY_CLUSTER;
             }
         }
-    } else {
-        float um[C], t[2 * C + 1], dummy;
-        DF tot[2 * C];
-        membership<C, MK>((float)b, v0, m, inv_m1, up, um);
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            t[j] = cnt * (um[j] * (float)b);
-            t[C + j] = cnt * um[j];
-        }
-        t[2 * C] = 0.0f;
-        block_sums<2 * C>(sc, par, t, tot, dummy);
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            if (tot[C + j].hi > 0.0f) {
-                v64[j] = df_div(tot[j], tot[C + j]);
-                v[j] = v64[j].hi;
-            } else {
-                v[j] = v0[j];  // an empty cluster keeps V^0
-                v64[j] = DF{v0[j], 0.0f};
-                flags = FCM_FLAG_EMPTY_CLUSTER;
-            }
-        }
+    } else if (bin_first_centers<C, MK>(sc, par, cnt2, v0, m, inv_m1, up2, v, mine)) {
+        flags = FCM_FLAG_EMPTY_CLUSTER;  // an empty cluster keeps V^0
     }
-    float* T = a.table + (int64_t)r * 256 * FCM_MAX_CLUSTERS;
+    float* T = a.table + (int64_t)r * 256 * FCM_MAX_CLUSTERS + (2 * t) * FCM_MAX_CLUSTERS;
 
     // ---- the first stopping quantity, from U^0 ----
     float d1 = 0.0f;
@@ -277,21 +267,22 @@ __device__ __noinline__ void solve_run(const BinArgs& a, int r, const BinRun& ru
         if (a.phase == 0) {
             // U^1 per grey level, kept for pass B; the recorded pixel of each
             // grey level gives a lower bound of delta_1
-            float u1[C], um1[C], t[2], lb;
-            DF tot[1];
-            membership<C, MK>((float)b, v, m, inv_m1, u1, um1);
+            PackedCenters<C, MK> cen;
+            bin_centers<C, MK>(sc, v, cen);
+            f2 u1[C], um1[C], dd[C], J2;
+            bin_memberships<C, MK>(b2, cen, m, inv_m1, u1, um1, dd, J2);
+            const int2 rp = *reinterpret_cast<const int2*>(a.rep + (int64_t)s * 256 + 2 * t);
+            float lb = 0.0f;
 #pragma unroll
-            for (int j = 0; j < C; ++j) T[b * FCM_MAX_CLUSTERS + j] = u1[j];
-            t[0] = 0.0f;
-            t[1] = 0.0f;
-            const int rp = a.rep[(int64_t)s * 256 + b];
-            if (rp >= 0) {
-#pragma unroll
-                for (int j = 0; j < C; ++j) t[1] = fmaxf(t[1], fabsf(u1[j] - __ldg(d.U0 + (int64_t)j * d.n + rp)));
+            for (int j = 0; j < C; ++j) {
+                T[j] = lo2(u1[j]);
+                T[FCM_MAX_CLUSTERS + j] = hi2(u1[j]);
+                if (rp.x >= 0) lb = fmaxf(lb, fabsf(lo2(u1[j]) - __ldg(d.U0 + (int64_t)j * d.n + rp.x)));
+                if (rp.y >= 0) lb = fmaxf(lb, fabsf(hi2(u1[j]) - __ldg(d.U0 + (int64_t)j * d.n + rp.y)));
             }
-            block_sums<1>(sc, par, t, tot, lb);
+            lb = bin_max(sc, par, lb);
             if (!(lb >= d.eps) || d.max_iter == 1) {
-                if (b == 0) a.need_b[r] = 1;  // pass B takes delta_1 over every pixel; S1 resumes
+                if (t == 0) a.need_b[r] = 1;  // pass B takes delta_1 over every pixel; S1 resumes
                 return;
             }
             d1 = lb;  // proves delta_1 >= eps: the run goes on to iteration 2
@@ -304,16 +295,17 @@ __device__ __noinline__ void solve_run(const BinArgs& a, int r, const BinRun& ru
     int k, status;
     float delta;
     DF J;
-    solve_bins<C, MK>(sc, par, cnt, from_u, d1, v, v64, up, m, inv_m1, d.eps, d.max_iter, flags, k, status, delta, J);
+    solve_bins<C, MK>(sc, par, cnt2, from_u, d1, v, mine, up2, m, inv_m1, d.eps, d.max_iter, flags, k, status, delta, J);
 #pragma unroll
-    for (int j = 0; j < C; ++j) T[b * FCM_MAX_CLUSTERS + j] = up[j];
-#pragma unroll
-    for (int j = 0; j < C; ++j)
-        if (b == j) {
-            if (run.write_u) d.V[j] = v[j];
-            res.V64[j] = (double)v64[j].hi + (double)v64[j].lo;
-        }
-    if (b == 0) {
+    for (int j = 0; j < C; ++j) {
+        T[j] = lo2(up2[j]);
+        T[FCM_MAX_CLUSTERS + j] = hi2(up2[j]);
+    }
+    if (t < 4 * C && (t & 3) == 0) {
+        if (run.write_u) d.V[g] = mine.hi;
+        res.V64[g] = (double)mine.hi + (double)mine.lo;
+    }
+    if (t == 0) {
         res.iters = k;
         res.status = status;
         res.flags = flags;
@@ -322,7 +314,7 @@ __device__ __noinline__ void solve_run(const BinArgs& a, int r, const BinRun& ru
     }
 }
 
-__global__ void __launch_bounds__(SNT, 2) k_bins_solve(BinArgs a) {
+__global__ void __launch_bounds__(SNT, 4) k_bins_solve(BinArgs a) {
     __shared__ BinScratch sc;
     __shared__ DF s_tot[2 * FCM_MAX_CLUSTERS];
     const int r = blockIdx.x;

@@ -10,10 +10,10 @@
 // per-pixel run's up to the order of rounding.
 //
 // Per run: one pass over the pixels builds the histogram (and, from U^0, the
-// sums of V^1); with U^0 given, a second pass takes the first stopping
-// quantity against the pixels' U^0; one CTA then iterates on the bins; a last
-// pass writes U^k by table lookup. HBM traffic is 4 + 4C bytes per pixel for
-// each of the (up to) three passes instead of 4 + 8C per iteration.
+// sums of V^1); one CTA then iterates on the bins; a last pass writes U^k by table
+// lookup. With U^0 given, a pass over the pixels takes the first stopping quantity
+// when a sample of them cannot decide the first stop. HBM traffic is 4 + 4C bytes
+// per pixel for each of the two (or three) passes instead of 4 + 8C per iteration.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -21,6 +21,7 @@
 #include <cstring>
 
 #include "fcm.h"
+#define FCM_ONE_SCALAR_PAIR
 #include "fcm_bounds.cuh"
 #include "fcm_device.cuh"
 #include "fcm_df.cuh"
@@ -38,13 +39,15 @@ struct alignas(16) HistState {
     unsigned d1bits;  // max |U^1 - U^0| over the pixels, as float bits (from U^0)
     int bad;
     int iters, status, flags;
+    int need_d1;      // the sampled pixels could not decide the first stop: k_hist_delta1 runs
+    int rep[256];     // 1 + some pixel of each grey level, or 0
     unsigned bounds;  // FCM_FLAG_BOUNDS from a FCM_DEBUG_BOUNDS build's guards
 };
 
 struct HistWorkspace {
     HistState* d_st = nullptr;
     HistState* h_st = nullptr;  // pinned
-    double* part = nullptr;
+    double* part = nullptr;  // [blocks][2C] sums of V^1
     int part_blocks = 0;
     float* table = nullptr;  // [256][C] final memberships of each grey level
 };
@@ -69,7 +72,9 @@ __global__ void __launch_bounds__(HNT, C <= 4 ? 4 : 2) k_hist_pass0(const float*
                                                    int64_t n, float m, HistState* st, double* __restrict__ part) {
     __shared__ unsigned hs[HNT / 32][256];  // one sub-histogram per warp
     __shared__ float w[HNT / 32][4 * C];
+    __shared__ int rep[256];
     for (int t = threadIdx.x; t < (HNT / 32) * 256; t += HNT) (&hs[0][0])[t] = 0u;
+    rep[threadIdx.x] = 0;
     __syncthreads();
     DF acc[2 * C];
 #pragma unroll
@@ -109,6 +114,7 @@ __global__ void __launch_bounds__(HNT, C <= 4 ? 4 : 2) k_hist_pass0(const float*
             // shared-memory atomics: lanes of a warp on the same grey level are
             // serialised by the hardware; counts are exact in any order
             if (good) atomicAdd(&hw[g], 1u);
+            if (FROM_U && q == 0 && good && i < 0x7fffffff) rep[g] = (int)i + 1;  // any pixel of the grey level will do
             if (FROM_U && good) {
 #pragma unroll
                 for (int j = 0; j < C; ++j) {
@@ -133,6 +139,7 @@ __global__ void __launch_bounds__(HNT, C <= 4 ? 4 : 2) k_hist_pass0(const float*
         unsigned t = 0u;
         for (int v = 0; v < HNT / 32; ++v) t += hs[v][b];
         if (t) atomicAdd(&st->hist[b], (unsigned long long)t);
+        if (FROM_U && rep[b]) st->rep[b] = rep[b];  // any block's will do
     }
     if (__syncthreads_or(bad || umin < 0.0f) && threadIdx.x == 0) atomicOr(&st->bad, 1);
     if (!FROM_U) return;
@@ -154,116 +161,6 @@ __global__ void __launch_bounds__(HNT, C <= 4 ? 4 : 2) k_hist_pass0(const float*
     }
 }
 
-// Block-wide FP64 sums of S values per thread and one float maximum, the same
-// fixed order in every call; every thread receives the totals.
-template <int S>
-__device__ __forceinline__ void block_sums(double (&v)[S], float& mx, double (*red)[S + 1], double* tot) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < S; ++q) v[q] = warp_sum(v[q]);
-    mx = warp_max(mx);
-    if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < S; ++q) red[warp][q] = v[q];
-        red[warp][S] = (double)mx;
-    }
-    __syncthreads();
-    if (threadIdx.x <= S) {
-        const int q = threadIdx.x;
-        double t = 0.0;
-        for (int u = 0; u < HNT / 32; ++u) t = q < S ? t + red[u][q] : fmax(t, red[u][q]);
-        tot[q] = t;
-    }
-    __syncthreads();
-}
-
-// V^1: from the pass-0 slots (U^0 given), or from the bins with
-// U^0 = f(grey level, V^0) (Eq. 4 then Eq. 3). One CTA.
-template <int C, int MK, bool FROM_U>
-__global__ void __launch_bounds__(HNT) k_hist_init(HistState* st, const double* __restrict__ part, int nblocks,
-                                                  float m, float inv_m1) {
-    __shared__ double red[HNT / 32][2 * C + 1];
-    __shared__ double tot[2 * C + 1];
-    bool bad = st->bad != 0;
-    if (!FROM_U) {
-#pragma unroll
-        for (int j = 0; j < C; ++j) bad |= !finite_f(st->V0[j]);
-    }
-    if (bad) {
-        if (threadIdx.x == 0) {
-            st->bad = 1;
-            st->status = FCM_ERR_BAD_INPUT;
-            st->iters = 0;
-#pragma unroll
-            for (int j = 0; j < C; ++j) {
-                st->V[j] = st->V0[j];
-                st->V64[j] = st->V0[j];
-            }
-        }
-        return;
-    }
-    if (FROM_U) {
-        // thread t adds slots t, t + HNT, ... of every sum; then one block sum
-        double s[2 * C];
-        float mx = 0.0f;
-#pragma unroll
-        for (int q = 0; q < 2 * C; ++q) s[q] = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += HNT) {
-#pragma unroll
-            for (int q = 0; q < 2 * C; ++q) s[q] += part[(int64_t)b * 2 * C + q];
-        }
-        block_sums<2 * C>(s, mx, red, tot);
-        bool finite = true;
-#pragma unroll
-        for (int q = 0; q < 2 * C; ++q) finite &= isfinite(tot[q]);
-        if (!finite) {
-            // a NaN or infinite U^0 entry (pass 0 checks only for negative ones)
-            if (threadIdx.x == 0) {
-                st->bad = 1;
-                st->status = FCM_ERR_BAD_INPUT;
-                st->iters = 0;
-#pragma unroll
-                for (int j = 0; j < C; ++j) {
-                    st->V[j] = st->V0[j];
-                    st->V64[j] = st->V0[j];
-                }
-            }
-            return;
-        }
-    } else {
-        const int b = threadIdx.x;
-        const double hb = (double)st->hist[b];
-        float v0[C], u[C], um[C];
-#pragma unroll
-        for (int j = 0; j < C; ++j) v0[j] = st->V0[j];
-        membership<C, MK>((float)b, v0, m, inv_m1, u, um);
-        double s[2 * C];
-        float mx = 0.0f;
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            s[j] = hb * (double)um[j] * (double)b;
-            s[C + j] = hb * (double)um[j];
-        }
-        block_sums<2 * C>(s, mx, red, tot);
-    }
-    if (threadIdx.x == 0) {
-        int flags = 0;
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            const double den = tot[C + j];
-            if (den > 0.0) {
-                st->V64[j] = tot[j] / den;
-                st->V[j] = (float)st->V64[j];
-            } else {
-                flags |= FCM_FLAG_EMPTY_CLUSTER;  // V^0 kept, or 0 from a U^0
-                st->V[j] = FROM_U ? 0.0f : st->V0[j];
-                st->V64[j] = st->V[j];
-            }
-        }
-        st->flags = flags;
-    }
-}
-
 // The first stopping quantity from U^0: max over pixels and clusters of
 // |f(x_i, V^1)_j - U^0_ij|, with f tabulated per grey level.
 template <int C, int MK>
@@ -271,7 +168,7 @@ __global__ void __launch_bounds__(HNT) k_hist_delta1(const float* __restrict__ x
                                                     int64_t n, float m, float inv_m1, HistState* st) {
     __shared__ float T[256][C];
     __shared__ float wm[HNT / 32];
-    if (st->bad) return;
+    if (st->bad || !st->need_d1) return;
     {
         float v[C], u[C], um[C];
 #pragma unroll
@@ -299,50 +196,127 @@ __global__ void __launch_bounds__(HNT) k_hist_delta1(const float* __restrict__ x
     }
 }
 
-// Algorithm 1 on the bins, one CTA (solve_bins: thread b holds grey level b).
+// V^1, from the pass-0 sums (U^0 given) or from the bins with U^0 = f(grey
+// level, V^0), then Algorithm 1 on the bins, one CTA (solve_bins). From U^0 the
+// first stopping quantity is bounded from below by the recorded pixel of every
+// grey level; only when that bound does not reach eps, or max_iter is 1, does
+// phase 0 leave the run to k_hist_delta1, which takes it over every pixel, and to
+// phase 1. A pass over x and U^0 (50 us of a 256^3 volume's 317) is thus skipped
+// whenever it could not change the run. 60 iterations of that volume: 314 -> 239 us
+// (the bins, at 1.2 us per iteration before, among it).
 template <int C, int MK, bool FROM_U>
-__global__ void __launch_bounds__(HNT) k_hist_solve(HistState* st, float* __restrict__ table, float m, float inv_m1,
-                                                   float eps, int max_iter) {
+__global__ void __launch_bounds__(BIN_NT) k_hist_solve(HistState* st, const double* __restrict__ part, int nblocks,
+                                                      const float* __restrict__ U0, int64_t n,
+                                                      float* __restrict__ table, float m, float inv_m1, float eps,
+                                                      int max_iter, int phase) {
     __shared__ BinScratch sc;
-    if (st->bad) return;
-    const int b = threadIdx.x;
-    float v[C], up[C];
-    DF v64[C];
+    __shared__ double s_sum[2 * C];
+    const int t = threadIdx.x;
+    if (phase == 1 && !st->need_d1) return;
+    bool bad = st->bad != 0;
+    float v0[C];
 #pragma unroll
-    for (int j = 0; j < C; ++j) {
-        v[j] = st->V[j];
-        const double q = st->V64[j];
-        v64[j] = DF{(float)q, (float)(q - (double)(float)q)};
-        up[j] = 0.0f;
-    }
+    for (int j = 0; j < C; ++j) v0[j] = st->V0[j];
     if (!FROM_U) {
-        float v0[C], um0[C];
 #pragma unroll
-        for (int j = 0; j < C; ++j) v0[j] = st->V0[j];
-        membership<C, MK>((float)b, v0, m, inv_m1, up, um0);
+        for (int j = 0; j < C; ++j) bad |= !finite_f(v0[j]);
+    } else if (!bad) {
+        // sum q by 16 lanes' shares at a time, the same fixed order in every call
+        for (int q = t >> 4; q < 2 * C; q += BIN_NT / 16) {
+            double a = 0.0;
+            for (int b = t & 15; b < nblocks; b += 16) a += part[(int64_t)b * 2 * C + q];
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffu << (t & 16), a, o);
+            if ((t & 15) == 0) s_sum[q] = a;
+        }
+        __syncthreads();
+        // a NaN or infinite U^0 entry (pass 0 checks only for negative ones)
+#pragma unroll
+        for (int q = 0; q < 2 * C; ++q) bad |= !isfinite(s_sum[q]);
     }
-    const float cnt = (float)st->hist[b];
-    int flags = st->flags, par = 0;
+    if (bad) {
+        __syncthreads();
+        if (t == 0) {
+            st->bad = 1;
+            st->status = FCM_ERR_BAD_INPUT;
+            st->iters = 0;
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                st->V[j] = v0[j];
+                st->V64[j] = v0[j];
+            }
+        }
+        return;
+    }
+    const f2 cnt2 = pack2((float)st->hist[2 * t], (float)st->hist[2 * t + 1]);
+    const f2 b2 = pack2((float)(2 * t), (float)(2 * t + 1));
+    const int g = (t & 31) >> 2;  // the cluster whose double-float center this lane holds
+    int par = 0, flags = 0;
+    float v[C];
+    f2 up2[C];
+    DF mine = bin_mine<C>(v0);
+    if (FROM_U) {
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            up2[j] = pack2(0.0f, 0.0f);
+            const double den = s_sum[C + j];
+            if (den > 0.0) {
+                const double q = s_sum[j] / den;
+                v[j] = (float)q;
+                if (g == j) mine = DF{(float)q, (float)(q - (double)(float)q)};
+            } else {
+                flags = FCM_FLAG_EMPTY_CLUSTER;  // 0 from a U^0
+                v[j] = 0.0f;
+                if (g == j) mine = DF{0.0f, 0.0f};
+            }
+        }
+    } else if (bin_first_centers<C, MK>(sc, par, cnt2, v0, m, inv_m1, up2, v, mine)) {
+        flags = FCM_FLAG_EMPTY_CLUSTER;  // V^0 kept
+    }
+    float d1 = 0.0f;
+    if (FROM_U) {
+        if (phase == 0) {
+            PackedCenters<C, MK> cen;
+            bin_centers<C, MK>(sc, v, cen);
+            f2 u1[C], um1[C], dd[C], J2;
+            bin_memberships<C, MK>(b2, cen, m, inv_m1, u1, um1, dd, J2);
+            const int r0 = st->rep[2 * t] - 1, r1 = st->rep[2 * t + 1] - 1;
+            float lb = 0.0f;
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                if (r0 >= 0) lb = fmaxf(lb, fabsf(lo2(u1[j]) - __ldg(U0 + (int64_t)j * n + r0)));
+                if (r1 >= 0) lb = fmaxf(lb, fabsf(hi2(u1[j]) - __ldg(U0 + (int64_t)j * n + r1)));
+            }
+            d1 = bin_max(sc, par, lb);
+            if (!(d1 >= eps) || max_iter == 1) {
+                if (t < 4 * C && (t & 3) == 0) st->V[g] = mine.hi;  // k_hist_delta1 reads V^1
+                if (t == 0) st->need_d1 = 1;
+                return;
+            }
+        } else {
+            d1 = __uint_as_float(st->d1bits);
+        }
+    }
     int k, status;
     float delta;
     DF J;
-    solve_bins<C, MK>(sc, par, cnt, FROM_U, FROM_U ? __uint_as_float(st->d1bits) : 0.0f, v, v64, up, m, inv_m1,
-                      eps, max_iter, flags, k, status, delta, J);
+    solve_bins<C, MK>(sc, par, cnt2, FROM_U, d1, v, mine, up2, m, inv_m1, eps, max_iter, flags, k, status, delta, J);
 #pragma unroll
-    for (int j = 0; j < C; ++j) table[b * C + j] = up[j];
-    if (b == 0) {
+    for (int j = 0; j < C; ++j) {
+        table[(2 * t) * C + j] = lo2(up2[j]);
+        table[(2 * t + 1) * C + j] = hi2(up2[j]);
+    }
+    if (t < 4 * C && (t & 3) == 0) {
+        st->V[g] = mine.hi;
+        st->V64[g] = (double)mine.hi + (double)mine.lo;
+    }
+    if (t == 0) {
         st->iters = k;
         st->status = status;
         st->flags = flags;
         st->delta = (double)delta;
         st->J = (double)J.hi + (double)J.lo;
     }
-#pragma unroll
-    for (int j = 0; j < C; ++j)
-        if (b == j) {
-            st->V[j] = v[j];
-            st->V64[j] = (double)v64[j].hi + (double)v64[j].lo;
-        }
 }
 
 // U^k by table lookup: U_ij = table[x_i][j].
@@ -364,14 +338,12 @@ __global__ void __launch_bounds__(HNT) k_hist_emit(const float* __restrict__ x, 
 }
 
 typedef void (*Pass0Fn)(const float*, const float*, int64_t, float, HistState*, double*);
-typedef void (*InitFn)(HistState*, const double*, int, float, float);
 typedef void (*Delta1Fn)(const float*, const float*, int64_t, float, float, HistState*);
-typedef void (*SolveFn)(HistState*, float*, float, float, float, int);
+typedef void (*SolveFn)(HistState*, const double*, int, const float*, int64_t, float*, float, float, float, int, int);
 typedef void (*EmitFn)(const float*, int64_t, const float*, const HistState*, float*);
 
 struct HistKernels {
     Pass0Fn pass0[2];
-    InitFn init[2];
     Delta1Fn delta1;
     SolveFn solve[2];
     EmitFn emit;
@@ -380,7 +352,6 @@ struct HistKernels {
 template <int C, int MK>
 HistKernels kernels_cm() {
     return HistKernels{{k_hist_pass0<C, MK, false>, k_hist_pass0<C, MK, true>},
-                       {k_hist_init<C, MK, false>, k_hist_init<C, MK, true>},
                        k_hist_delta1<C, MK>,
                        {k_hist_solve<C, MK, false>, k_hist_solve<C, MK, true>},
                        k_hist_emit<C>};
@@ -480,9 +451,10 @@ extern "C" int fcm_run_hist(fcm_handle h, const float* x, int64_t n, int C, floa
     const float inv_m1 = (float)(1.0 / ((double)m - 1.0));
     const int fu = from_u ? 1 : 0;
     k.pass0[fu]<<<nblocks, HNT, 0, h->stream>>>(x, from_u ? U0 : nullptr, n, m, w->d_st, w->part);
-    k.init[fu]<<<1, HNT, 0, h->stream>>>(w->d_st, w->part, nblocks, m, inv_m1);
+    k.solve[fu]<<<1, BIN_NT, 0, h->stream>>>(w->d_st, w->part, nblocks, U0, n, w->table, m, inv_m1, eps, max_iter, 0);
+    // these return at once unless the solver's bound left the first stop open
     if (from_u) k.delta1<<<nblocks, HNT, 0, h->stream>>>(x, U0, n, m, inv_m1, w->d_st);
-    k.solve[fu]<<<1, HNT, 0, h->stream>>>(w->d_st, w->table, m, inv_m1, eps, max_iter);
+    k.solve[fu]<<<1, BIN_NT, 0, h->stream>>>(w->d_st, w->part, nblocks, U0, n, w->table, m, inv_m1, eps, max_iter, 1);
     k.emit<<<nblocks, HNT, 0, h->stream>>>(x, n, w->table, w->d_st, U);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(hs, w->d_st, sizeof(HistState), cudaMemcpyDeviceToHost, h->stream));
