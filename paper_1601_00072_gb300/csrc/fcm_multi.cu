@@ -94,17 +94,21 @@ extern "C" int fcm_run_multi(fcm_handle h, const float* x, int64_t n, int D, int
     if (!w->h_st) CK(host_malloc(h, &w->h_st, sizeof(MultiState)));
     const MultiTable& t = multi_table();
     const MultiFn fn = t.run[D][C][m == 2.0f ? 0 : 1][from_u ? 0 : 1];
+    const int smem = multi_smem(C, D);
     int per_sm = 0;
     auto it = w->occupancy.find((const void*)fn);
     if (it != w->occupancy.end()) {
         per_sm = it->second;
     } else {
-        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, 256, 0));
+        CK(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, MULTI_NT, smem));
         w->occupancy[(const void*)fn] = per_sm;
     }
     if (per_sm < 1) return ctx_invalid(h, "the multi-feature kernel does not fit on this device");
-    const int64_t want = (n + 256 * 4 - 1) / (256 * 4);
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)per_sm * h->num_sms));
+    // a thread takes two pixels per step: one block per SM at most, fewer for an
+    // image that a single step of them covers
+    const int64_t want = (n + 2 * MULTI_NT - 1) / (2 * MULTI_NT);
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(want, h->num_sms));
     const int64_t S = (int64_t)C * D + C + 1 + 3;
     const int64_t need = 2 * 2 * S * blocks;
     if (w->partial_floats < need) {
@@ -133,7 +137,7 @@ extern "C" int fcm_run_multi(fcm_handle h, const float* x, int64_t n, int D, int
     MultiState* dst = w->d_st;
     float* part = w->partials;
     void* args[2] = {&dst, &part};
-    CK(cudaLaunchCooperativeKernel((const void*)fn, dim3(blocks), dim3(256), args, 0, h->stream));
+    CK(cudaLaunchCooperativeKernel((const void*)fn, dim3(blocks), dim3(MULTI_NT), args, smem, h->stream));
     CK(cudaMemcpyAsync(hs, w->d_st, sizeof(MultiState), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemcpyAsync(V, &w->d_st->V, sizeof(float) * C * D,
                        V_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));

@@ -29,6 +29,10 @@ struct alignas(128) MultiState {
 
 typedef void (*MultiFn)(MultiState*, float*);
 
+constexpr int MULTI_NT = 512;  // threads per block, one block per SM
+// Dynamic shared memory: the second set of the sums.
+constexpr int multi_smem(int C, int D) { return MULTI_NT * 8 * C * (D + 1); }
+
 struct MultiTable {
     // [D][C][0 = m == 2, 1 = any m][0 = from U^0, 1 = from V^0]
     MultiFn run[MULTI_MAX_D + 1][FCM_MAX_CLUSTERS + 1][2][2];
