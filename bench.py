@@ -53,11 +53,10 @@ MAX_ITER = 300
 METRIC = "FCM pixel-iterations/s (256^3 volume, C=4, m=2, eps=1e-5)"
 UNIT = "pixel-iter/s"
 PROFILE = os.path.join(ROOT, "profiles", "fcm_pass_volume256.md")
-KERNEL_SOURCES = ["paper_1601_00072_gb300/csrc/fcm_single_inst.cu",
+KERNEL_SOURCES = ["paper_1601_00072_gb300/csrc/fcm_run_inst.cu",
                   "paper_1601_00072_gb300/csrc/fcm_device.cuh",
-                  "paper_1601_00072_gb300/csrc/fcm_exchange.cuh",
                   "paper_1601_00072_gb300/csrc/fcm_df.cuh",
-                  "paper_1601_00072_gb300/csrc/fcm_tma.cuh",
+                  "paper_1601_00072_gb300/csrc/fcm_run.h",
                   "paper_1601_00072_gb300/csrc/fcm_internal.h"]
 
 
@@ -108,6 +107,28 @@ def issue_roofline(path, sources, ms, iters, sm_mhz):
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "G warp-instr/s", "frac": achieved / peak,
             "instructions_per_launch": inst, "source": path,
             "peak_source": f"{sms} SMs x 4 schedulers x {sm_mhz or 2070.0:.0f} MHz"}
+
+
+def fp32_ops_per_pixel_iter(C, m):
+    """FP32 operations of a sums pass per pixel (packed pairs count as two):
+    differences C, squares C (none at m = 3), co-products 3 (C - 2), their sum
+    C - 1, u^m 2C (one more C at m = 3 and 1.5), numerators and denominators 2C."""
+    ops = C + 3 * max(C - 2, 0) + (C - 1) + 2 * C + 2 * C
+    ops += 0 if m == 3.0 else C
+    ops += C if m in (1.5, 3.0) else 0
+    return ops
+
+
+def fp32_roofline(px_iters, ms, C, m, sm_mhz):
+    """Of the FP32 pipe: 128 lanes per SM and clock."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    mhz = sm_mhz or 2070.0
+    peak = sms * 128 * mhz * 1e6 / 1e12
+    achieved = px_iters * fp32_ops_per_pixel_iter(C, m) / (ms / 1e3) / 1e12
+    return {"bound": "fp32 pipe", "achieved": achieved, "peak": peak, "unit": "T FP32 instr/s", "frac": achieved / peak,
+            "ops_per_pixel_iter": fp32_ops_per_pixel_iter(C, m),
+            "peak_source": f"{sms} SMs x 128 lanes x {mhz:.0f} MHz"}
 
 
 def measured_peak():
@@ -651,10 +672,11 @@ def bench_ours(args):
     units = allreduce(units_local, "sum", world)
     value = units / (ms / 1e3)
 
-    # roofline of the pass kernels over the timed region (algorithmic bytes:
-    # pass 0 reads x and U^0; each iteration reads x and U^{k-1}, writes U^k)
-    bytes_local = sum((4 * n + 4 * C * n) + it * (4 * n + 8 * C * n) for it in iters)
-    achieved = bytes_local / (ms_local / 1e3) / 1e9
+    # rooflines over the timed region: the FP32 pipe bounds the iterations, which
+    # read x alone (from shared memory and the L2); HBM the first pass (x and U^0)
+    # and the last (U^k written once)
+    bytes_local = sum((4 * n + 4 * C * n) + (4 * n + 4 * C * n) for _ in iters)
+    hbm_gbs = bytes_local / (ms_local / 1e3) / 1e9
     peak, peak_kind = measured_peak()
     traffic = profiled_traffic()
 
@@ -703,9 +725,8 @@ def bench_ours(args):
     keep = {"main": (Ud, Vd, r.iters, r.J)}
 
     # the other single-image workloads: the 200x200 and 1024x1024 phantoms
-    # (L2-resident: latency-bound, no HBM roofline) and the volume at the
-    # other fuzzifiers (HBM-bound, roofline as the main line)
-    peak_, _ = measured_peak()
+    # (on chip: latency-bound, no roofline) and the volume at the other
+    # fuzzifiers (roofline as the main line)
     workloads = {}
     if not args.no_workloads:
         import phantom
@@ -730,19 +751,16 @@ def bench_ours(args):
             e1.record(stream)
             torch.cuda.synchronize(dev)
             wms = e0.elapsed_time(e1) / reps
-            wbytes = (4 + 4 * C) * nw + rw.iters * (4 + 8 * C) * nw
             ent = {"workload": workload_name(mm) if name == "volume256" else
                    f"{name}: {int(np.sqrt(nw))}x{int(np.sqrt(nw))} uint8 phantom as f32, C=4, m={mm:g}, eps=1e-5",
                    "n_pixels": nw, "m": mm, "runs": reps, "ms_per_run": wms, "images_per_s": 1e3 / wms,
                    "iters": rw.iters, "pixel_iter_per_s": nw * rw.iters / (wms / 1e3),
                    "us_per_iteration": wms * 1e3 / max(1, rw.iters)}
             if name == "volume256":
-                ent["roofline"] = {"bound": "hbm", "achieved": wbytes / (wms / 1e3) / 1e9, "peak": peak_,
-                                   "unit": "GB/s", "frac": wbytes / (wms / 1e3) / 1e9 / peak_,
-                                   "algorithmic_bytes_per_run": wbytes}
+                ent["roofline"] = fp32_roofline(float(nw) * rw.iters, wms, C, mm, clocks.get("sm_mhz"))
             else:
-                ent["bound"] = (f"latency: working set {(4 + 8 * C) * nw / 1e6:.1f} MB sits in the 129 MB L2; "
-                                "an iteration costs its grid exchange")
+                ent["bound"] = (f"latency: x ({4 * nw / 1e6:.1f} MB) sits in shared memory; "
+                                "an iteration costs its dependent steps and its grid exchange")
             workloads[key] = ent
             keep[key] = (Uw, Vw, rw.iters, rw.J, xw, u0w, mm)
 
@@ -761,8 +779,8 @@ def bench_ours(args):
         e1.record(stream)
         torch.cuda.synchronize(dev)
         hms = e0.elapsed_time(e1) / hs
-        hbytes = 3 * (4 + 4 * C) * n  # histogram + V^1 pass, first-stop pass, U write
-        hist = {"kernel": "fcm_run_hist: pixel passes for the histogram, the first stop and the U write; "
+        hbytes = 2 * (4 + 4 * C) * n  # histogram + V^1 pass, U write
+        hist = {"kernel": "fcm_run_hist: pixel passes for the histogram and the U write; "
                           "the iterations on 256 bins in one CTA",
                 "ms_per_run": hms, "iters": rh.iters, "launches_per_run": rh.launches,
                 "equivalent_pixel_iter_per_s": n * rh.iters / (hms / 1e3),
@@ -786,21 +804,13 @@ def bench_ours(args):
         e1.record(stream)
         torch.cuda.synchronize(dev)
         rms = e0.elapsed_time(e1) / rs
-        rbytes = 2 * (4 + 4 * C) * n + (rr.iters - 1) * 4 * n + (4 + 4 * C) * n
-        recompute = {"kernel": "k_fcm_run_rc: one cooperative launch; U^{k-1} recomputed from V^{k-1}, "
-                               "x read per iteration (L2-resident), U written once",
+        rbytes = 2 * (4 + 4 * C) * n
+        recompute = {"kernel": "k_fcm_run (FCM_OPT_RECOMPUTE insists on it)",
                      "ms_per_run": rms, "iters": rr.iters, "pixel_iter_per_s": n * rr.iters / (rms / 1e3),
-                     "bound": "alu",
+                     "bound": "fp32 pipe",
                      "dram_bytes_per_run_algorithmic": rbytes,
                      "speedup_vs_pixel_path": (ms / args.steps) / rms,
-                     "roofline": issue_roofline("profiles/fcm_recompute_volume256.md",
-                                                ["paper_1601_00072_gb300/csrc/fcm_recompute_inst.cu",
-                                                 "paper_1601_00072_gb300/csrc/fcm_device.cuh",
-                                                 "paper_1601_00072_gb300/csrc/fcm_exchange.cuh",
-                                                 "paper_1601_00072_gb300/csrc/fcm_df.cuh",
-                                                 "paper_1601_00072_gb300/csrc/fcm_tma.cuh",
-                                                 "paper_1601_00072_gb300/csrc/fcm_internal.h"],
-                                                rms, rr.iters, clocks.get("sm_max_mhz"))}
+                     "roofline": fp32_roofline(float(n) * rr.iters, rms, C, m, clocks.get("sm_mhz"))}
         keep["recompute"] = (Ur, Vr, rr.iters, rr.J)
 
     # multi-feature FCM on a 3-channel 2048^2 phantom (shared layout, per-channel
@@ -860,15 +870,12 @@ def bench_ours(args):
                    "parallelism": f"replicas x{world}",
                    "l2": "working set 603 MB > 129 MB L2; no flush"},
         "gpu_launches": launches,
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak, "traffic": traffic,
-                     "peak_source": f"{peak_kind} copy bandwidth",
-                     "kernel": ("k_fcm_run_tma: one cooperative launch per step (pass 0 reads "
-                                "x and U0, 20 B/pixel; each iteration 36 B/pixel at C=4)"
-                                if r.launches == 1 else
-                                "k_fcm_pass_*: one launch per pass (pass 0 20 B/pixel, "
-                                "each iteration 36 B/pixel at C=4)"),
-                     "algorithmic_bytes_per_step": bytes_local / args.steps},
+        "roofline": dict(fp32_roofline(units_local, ms_local, C, m, clocks.get("sm_mhz")), traffic=traffic,
+                         kernel="k_fcm_run: one cooperative launch per step (pass 0 reads x and U0; the "
+                                "iterations read x from shared memory and the L2; U is written once)",
+                         algorithmic_bytes_per_step=bytes_local / args.steps,
+                         hbm={"achieved": hbm_gbs, "peak": peak, "unit": "GB/s", "frac": hbm_gbs / peak,
+                              "peak_source": f"{peak_kind} copy bandwidth"}),
         "clocks": clocks,
         "e2e": e2e,
         "histogram_domain": hist,
