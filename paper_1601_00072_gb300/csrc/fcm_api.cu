@@ -532,12 +532,7 @@ int fcm_run(fcm_handle h, const float* x, int64_t n, int C, float m, float eps, 
     hs->C = C;
     hs->status = STATUS_RUNNING;
     hs->lim = h->limits;
-    hs->from_u = init_mode == FCM_INIT_U;
     if (init_mode == FCM_INIT_V && !V_dev) std::memcpy(hs->V0, V, sizeof(float) * C);
-    CK(cudaMemcpyAsync(h->d_st, hs, sizeof(RunState), cudaMemcpyHostToDevice, h->stream));
-    if (init_mode == FCM_INIT_V && V_dev)
-        CK(cudaMemcpyAsync(&h->d_st->V0, V, sizeof(float) * C, cudaMemcpyDeviceToDevice, h->stream));
-
     const int mk = mkind_of(m);
     const int pass0 = init_mode == FCM_INIT_U ? P_ACCUM0 : P_INITV;
     const bool aligned = (n % 4 == 0) && ((uintptr_t)dx % 16 == 0) && ((uintptr_t)dU % 16 == 0) &&
@@ -551,10 +546,27 @@ int fcm_run(fcm_handle h, const float* x, int64_t n, int C, float m, float eps, 
         shape = run_shape(n, C, max_run_blocks(h, krun, C));
     if (shape.blocks > 0) {
         // the whole run: one cooperative launch (all blocks co-resident)
-        unsigned nonce;
-        if ((rc = next_nonce(h, &nonce))) return rc;
-        int resident = shape.resident;
-        void* args[4] = {&h->d_st, &h->d_slots, &nonce, &resident};
+        RunArgs ra;
+        std::memset(&ra, 0, sizeof(ra));
+        if ((rc = next_nonce(h, &ra.nonce))) return rc;
+        ra.x = dx;
+        ra.U0 = hs->Uprev;
+        ra.U = dU;
+        ra.Vin = init_mode == FCM_INIT_V && V_dev ? V : nullptr;
+        ra.Vout = V_dev ? V : nullptr;
+        ra.trace = hs->trace;
+        ra.out = hs;
+        ra.scratch = h->d_slots;
+        ra.n = n;
+        ra.m = m;
+        ra.inv_m1 = hs->inv_m1;
+        ra.eps = eps;
+        ra.max_iter = max_iter;
+        ra.from_u = init_mode == FCM_INIT_U;
+        ra.resident = shape.resident;
+        ra.lim = h->limits;
+        std::memcpy(ra.V0, hs->V0, sizeof(ra.V0));
+        void* args[1] = {&ra};
         const cudaError_t le =
             cudaLaunchCooperativeKernel(krun, dim3(shape.blocks), dim3(shape.threads), args, shape.smem, h->stream);
         if (le != cudaSuccess) {
@@ -564,6 +576,9 @@ int fcm_run(fcm_handle h, const float* x, int64_t n, int C, float m, float eps, 
         h->last_blocks = shape.blocks;
         h->last_path = 2;
     } else {
+    CK(cudaMemcpyAsync(h->d_st, hs, sizeof(RunState), cudaMemcpyHostToDevice, h->stream));
+    if (init_mode == FCM_INIT_V && V_dev)
+        CK(cudaMemcpyAsync(&h->d_st->V0, V, sizeof(float) * C, cudaMemcpyDeviceToDevice, h->stream));
     Launch L;
     if ((rc = choose_launch(h, n, C, mk, pass0, dx, dU, hs->Uprev, options, &L))) return rc;
     PassFn kfirst = L.kfirst, kiter = L.kiter;
@@ -585,11 +600,13 @@ int fcm_run(fcm_handle h, const float* x, int64_t n, int C, float m, float eps, 
     }
     }
 
-    CK(cudaMemcpyAsync(hs, h->d_st, sizeof(RunState), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(V, &h->d_st->V, sizeof(float) * C,
-                       V_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
+    if (h->last_path != 2) {
+        CK(cudaMemcpyAsync(hs, h->d_st, sizeof(RunState), cudaMemcpyDeviceToHost, h->stream));
+        if (V_dev) CK(cudaMemcpyAsync(V, &h->d_st->V, sizeof(float) * C, cudaMemcpyDeviceToDevice, h->stream));
+    }
     if (!U_dev) CK(cudaMemcpyAsync(U, h->d_stage_U, Ub, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
+    if (!V_dev) std::memcpy(V, hs->V, sizeof(float) * C);
 
     h->last_trace_iters = trace ? hs->iters : 0;
     h->last_C = C;
@@ -684,24 +701,34 @@ int fcm_run_stream(fcm_handle h, int n_images, const float* const* x, int64_t n,
         hs->C = C;
         hs->status = STATUS_RUNNING;
         hs->lim = h->limits;
-        hs->from_u = 1;
         const float* u0 = (U0 && U0[i]) ? U0[i] : U[i];
         // upload, once the download of image i - NS has drained this set
         if (i >= NS) e = cudaStreamWaitEvent(h->pipe_in, out_done[b], 0);
         if (e == cudaSuccess) e = cudaMemcpyAsync(dx, x[i], xb, cudaMemcpyDefault, h->pipe_in);
         if (e == cudaSuccess) e = cudaMemcpyAsync(dU, u0, Ub, cudaMemcpyDefault, h->pipe_in);
         if (e == cudaSuccess) e = cudaEventRecord(in_done[b], h->pipe_in);
-        // the run, with its state uploaded before and read back after
+        // the run; its results go straight to the image's pinned state
         if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, in_done[b], 0);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_st, hs, sizeof(RunState), cudaMemcpyHostToDevice, h->stream);
-        unsigned nonce = 0;
-        if (e == cudaSuccess && next_nonce(h, &nonce)) e = cudaErrorUnknown;
-        int resident = shape.resident;
-        void* args[4] = {&h->d_st, &h->d_slots, &nonce, &resident};
+        RunArgs ra;
+        std::memset(&ra, 0, sizeof(ra));
+        if (e == cudaSuccess && next_nonce(h, &ra.nonce)) e = cudaErrorUnknown;
+        ra.x = dx;
+        ra.U0 = dU;
+        ra.U = dU;
+        ra.out = hs;
+        ra.scratch = h->d_slots;
+        ra.n = n;
+        ra.m = m;
+        ra.inv_m1 = hs->inv_m1;
+        ra.eps = eps;
+        ra.max_iter = max_iter;
+        ra.from_u = 1;
+        ra.resident = shape.resident;
+        ra.lim = h->limits;
+        void* args[1] = {&ra};
         if (e == cudaSuccess)
             e = cudaLaunchCooperativeKernel(krun, dim3(shape.blocks), dim3(shape.threads), args, shape.smem, h->stream);
         if (e != cudaSuccess) h->run_nonce = 0xffffffffu;  // a number may not have been used
-        if (e == cudaSuccess) e = cudaMemcpyAsync(hs, h->d_st, sizeof(RunState), cudaMemcpyDeviceToHost, h->stream);
         if (e == cudaSuccess) e = cudaEventRecord(run_done[b], h->stream);
         // download
         if (e == cudaSuccess) e = cudaStreamWaitEvent(h->pipe_out, run_done[b], 0);

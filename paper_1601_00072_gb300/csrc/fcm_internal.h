@@ -67,7 +67,6 @@ struct alignas(128) RunState {
     unsigned int ticket;  // last-block-done counter of the current pass
     int launches;         // passes started in this run (loop guard)
     WaitLimits lim;
-    int from_u;           // whole-run kernel: 1 from U^0, 0 from V^0
     unsigned int bounds;  // FCM_FLAG_BOUNDS from a FCM_DEBUG_BOUNDS build's guards
 };
 

@@ -130,30 +130,34 @@ extern "C" int fcm_run_noalloc(const float* x, int64_t n, int C, float m, float 
     RunState* st = reinterpret_cast<RunState*>(d.scratch);
     char* slots = reinterpret_cast<char*>(d.scratch + kStateBytes);
 
-    // A fresh state for every call: the status must start at running.
+    RunArgs ra;
+    std::memset(&ra, 0, sizeof(ra));
+    ra.x = x;
+    ra.U0 = Uin;
+    ra.U = U;
+    ra.out = st;
+    ra.scratch = slots;
+    ra.n = n;
+    ra.m = m;
+    ra.inv_m1 = (float)(1.0 / ((double)m - 1.0));
+    ra.eps = eps;
+    ra.max_iter = max_iter;
+    ra.from_u = init_mode == FCM_INIT_U;
+    ra.resident = shape.resident;
+    ra.lim = WaitLimits{DEFAULT_GRID_SPINS, DEFAULT_TMA_POLLS, 0u, 0u};
+    const bool V_dev = on_device(V);
+    if (init_mode == FCM_INIT_V && V_dev) ra.Vin = V;
+    else if (init_mode == FCM_INIT_V) std::memcpy(ra.V0, V, sizeof(float) * C);
+    if (V_dev) ra.Vout = V;
+
+    // the status starts at running
     RunState hs;
     std::memset(&hs, 0, sizeof(hs));
-    hs.x = x;
-    hs.Uprev = Uin;
-    hs.U = U;
-    hs.n = n;
-    hs.m = m;
-    hs.inv_m1 = (float)(1.0 / ((double)m - 1.0));
-    hs.eps = eps;
-    hs.max_iter = max_iter;
-    hs.C = C;
     hs.status = STATUS_RUNNING;
-    hs.lim = WaitLimits{DEFAULT_GRID_SPINS, DEFAULT_TMA_POLLS, 0u, 0u};
-    hs.from_u = init_mode == FCM_INIT_U;
-    const bool V_dev = on_device(V);
-    if (init_mode == FCM_INIT_V && !V_dev) std::memcpy(hs.V0, V, sizeof(float) * C);
-
     cudaError_t e = cudaMemcpyAsync(st, &hs, sizeof(RunState), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess && init_mode == FCM_INIT_V && V_dev)
-        e = cudaMemcpyAsync(&st->V0, V, sizeof(float) * C, cudaMemcpyDeviceToDevice, stream);
     // the run's number, and zeroed slots when the numbers start over (no slot
     // then shows a tag of an earlier run of the same number)
-    unsigned nonce;
+    unsigned& nonce = ra.nonce;
     {
         std::lock_guard<std::mutex> lock(g_mu);
         nonce = ++g_dev[dev].nonce;
@@ -161,8 +165,7 @@ extern "C" int fcm_run_noalloc(const float* x, int64_t n, int C, float m, float 
     }
     if (e == cudaSuccess && nonce == 1) e = cudaMemsetAsync(slots, 0, kSlotBytes, stream);
     if (e == cudaSuccess) {
-        int resident = shape.resident;
-        void* args[4] = {&st, &slots, &nonce, &resident};
+        void* args[1] = {&ra};
         e = cudaLaunchCooperativeKernel((const void*)run_table().run[C][mk], dim3(shape.blocks), dim3(shape.threads), args, shape.smem,
                                         stream);
     }
@@ -172,10 +175,8 @@ extern "C" int fcm_run_noalloc(const float* x, int64_t n, int C, float m, float 
     }
     RunState out;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&out, st, sizeof(RunState), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(V, &st->V, sizeof(float) * C, V_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                            stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (e == cudaSuccess && !V_dev) std::memcpy(V, out.V, sizeof(float) * C);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return FCM_ERR_CUDA;

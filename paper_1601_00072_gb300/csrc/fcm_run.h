@@ -34,8 +34,28 @@ constexpr size_t run_scratch_bytes(int blocks) {
     return RUN_WORDS_BYTES + (size_t)RUN_SLOT_BYTES * run_slots(FCM_MAX_CLUSTERS) * blocks;
 }
 
-// nonce: the run's number on its scratch, counting up by one from run to run.
-typedef void (*WholeRunFn)(RunState*, char* scratch, unsigned nonce, int resident);
+// Arguments of one whole run, by value: a run is one launch, with no upload
+// before it. Its results (V, V64, delta, J, iters, status, flags of RunState) go
+// straight to `out`, pinned host memory or device memory, and V to Vout too.
+struct RunArgs {
+    const float* x;
+    const float* U0;   // the initial memberships (from_u); may equal U
+    float* U;
+    const float* Vin;  // nullable: initial centers in device memory (else V0)
+    float* Vout;       // nullable: device memory
+    double* trace;     // nullable
+    RunState* out;
+    char* scratch;
+    int64_t n;
+    float m, inv_m1, eps;
+    int max_iter;
+    int from_u;        // 1 from U^0, 0 from V^0
+    int resident;      // quads of x per pixel thread kept in shared memory
+    unsigned nonce;    // the run's number on its scratch, counting up by one from run to run
+    WaitLimits lim;
+    float V0[FCM_MAX_CLUSTERS];
+};
+typedef void (*WholeRunFn)(RunArgs);
 
 struct RunTable {
     WholeRunFn run[FCM_MAX_CLUSTERS + 1][4];

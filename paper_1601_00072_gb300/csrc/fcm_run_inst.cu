@@ -428,7 +428,7 @@ enum Exchange : int { X_SUMS0 = 0, X_SUMS = 1, X_J = 2 };  // sums of pass 0 fro
 
 template <int C, int MK>
 __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
-    k_fcm_run(RunState* __restrict__ st, char* scratch, unsigned nonce, int resident) {
+    k_fcm_run(const __grid_constant__ RunArgs ra) {
     constexpr int P = pow2_at_least(2 * C);
     extern __shared__ __align__(16) f2 second[];  // [2 C][pt] second set of the sums, then the resident quads
     __shared__ RunShared<C> sh;
@@ -436,34 +436,37 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     const int pw = (int)(blockDim.x >> 5) - 1;  // pixel warps; the control warp follows
     const bool control = warp == pw;
     const int nb = (int)gridDim.x;
-    const bool from_u = st->from_u != 0;
-    const float* U0 = st->Uprev;  // may be U itself: each pixel is read, then written, by one thread
-    float* U = st->U;
-    const int64_t n = st->n;
+    char* const scratch = ra.scratch;
+    const unsigned nonce = ra.nonce;
+    RunState* const st = ra.out;
+    const bool from_u = ra.from_u != 0;
+    const float* U0 = ra.U0;  // may be U itself: each pixel is read, then written, by one thread
+    float* U = ra.U;
+    const int64_t n = ra.n;
     Px px;
-    px.x = st->x;
+    px.x = ra.x;
     px.xs = reinterpret_cast<float4*>(second + 2 * C * 32 * pw) + threadIdx.x;
     px.n = n;
     px.pt = 32 * pw;
     px.t0 = (int64_t)blockIdx.x * px.pt + threadIdx.x;
     px.nt = (int64_t)nb * px.pt;
     px.steps = (n >> 2) > px.t0 ? (int)(((n >> 2) - 1 - px.t0) / px.nt) + 1 : 0;
-    px.resident = min(resident, px.steps);
+    px.resident = min(ra.resident, px.steps);
     px.vec_x = ((uintptr_t)px.x & 15) == 0;
     px.vec_u = px.vec_x && (n & 3) == 0 && ((uintptr_t)U & 15) == 0 && (!from_u || ((uintptr_t)U0 & 15) == 0);
-    const float m = st->m, inv_m1 = st->inv_m1, eps = st->eps;
-    const int max_iter = st->max_iter;
-    const bool tracing = st->trace != nullptr;
+    const float m = ra.m, inv_m1 = ra.inv_m1, eps = ra.eps;
+    const int max_iter = ra.max_iter;
+    const bool tracing = ra.trace != nullptr;
 
     if (threadIdx.x < C) {
-        const float v0 = st->V0[threadIdx.x];
+        const float v0 = ra.Vin ? ra.Vin[threadIdx.x] : ra.V0[threadIdx.x];
         sh.v[0][threadIdx.x] = v0;
         sh.v64[0][threadIdx.x] = DF{v0, 0.0f};
     }
     if (threadIdx.x == 0) {
         sh.ctl = make_int4(0, 0, 0, 0);
         sh.empty[0] = sh.empty[1] = sh.empty[2] = sh.empty[3] = 0u;
-        sh.lim = st->lim;
+        sh.lim = ra.lim;
     }
     __syncthreads();
     int flags = 0;    // thread 0 of block 0 only
@@ -882,7 +885,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
             st->delta = sh.delta;
             st->J = df_to_double(sh.J);
             if (tracing) {
-                double* t = st->trace + (int64_t)(k - 1) * (2 + C);
+                double* t = ra.trace + (int64_t)(k - 1) * (2 + C);
                 t[0] = sh.delta;
                 t[1] = df_to_double(sh.J);
 #pragma unroll
@@ -972,14 +975,12 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
 #pragma unroll
         for (int j = 0; j < C; ++j) {
             st->V[j] = sh.v[iters & 3][j];
+            if (ra.Vout) ra.Vout[j] = sh.v[iters & 3][j];
             st->V64[j] = df_to_double(sh.v64[iters & 3][j]);
         }
         st->status = status;
         st->iters = iters;
-        st->k = iters;
         st->flags = flags;
-        st->done = 1;
-        st->Uprev = st->U;
     }
 }
 
