@@ -67,8 +67,12 @@ constexpr int HCHUNK = 4;  // pixels per thread whose loads are issued together 
 // overflows FP32).
 // Up to C = 4, four blocks per SM fit in 64 registers (a few bytes spill at
 // C = 4): twice the warps of an unbounded build to cover the loads' latency.
-template <int C, int MK, bool FROM_U>
-__global__ void __launch_bounds__(HNT, C <= 4 ? 4 : 2) k_hist_pass0(const float* __restrict__ x, const float* __restrict__ U0,
+// VEC: rows of 16-byte-aligned quads (n % 4 == 0). A thread then takes two quads
+// of pixels per step with 128-bit loads, a quarter of the load instructions, and
+// folds its sums into double-float every eight pixels instead of four: the pass is
+// bound by its instructions as much as by HBM.
+template <int C, int MK, bool FROM_U, bool VEC>
+__global__ void __launch_bounds__(HNT, C <= 4 ? (VEC ? 3 : 4) : 2) k_hist_pass0(const float* __restrict__ x, const float* __restrict__ U0,
                                                    int64_t n, float m, HistState* st, double* __restrict__ part) {
     __shared__ unsigned hs[HNT / 32][256];  // one sub-histogram per warp
     __shared__ float w[HNT / 32][4 * C];
@@ -84,6 +88,59 @@ __global__ void __launch_bounds__(HNT, C <= 4 ? 4 : 2) k_hist_pass0(const float*
     const int64_t stride = (int64_t)gridDim.x * HNT;
     const int lane_id = threadIdx.x & 31;
     unsigned* hw = hs[threadIdx.x >> 5];
+    if (VEC) {
+        constexpr int Q = 2;  // quads per thread and step
+        const int64_t nq = n >> 2;
+        for (int64_t q0 = (int64_t)blockIdx.x * HNT + threadIdx.x; q0 < nq; q0 += stride * Q) {
+            float4 xc[Q], uc[Q][FROM_U ? C : 1];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int64_t i = q0 + q * stride;
+                const bool in = i < nq;
+                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                xc[q] = in ? __ldg(reinterpret_cast<const float4*>(x) + i) : z;
+                if (FROM_U) {
+#pragma unroll
+                    for (int j = 0; j < C; ++j)
+                        uc[q][j] = in ? __ldg(reinterpret_cast<const float4*>(U0 + (int64_t)j * n) + i) : z;
+                }
+            }
+            float num[C], den[C];
+#pragma unroll
+            for (int j = 0; j < C; ++j) num[j] = den[j] = 0.0f;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int64_t i = q0 + q * stride;
+                if (i >= nq) break;
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const float xi = comp(xc[q], p);
+                    const int g = grey_index(xi);
+                    bad |= g < 0;
+                    if (g < 0) continue;
+                    atomicAdd(&hw[g], 1u);
+                    if (FROM_U && p == 0 && q == 0 && 4 * i < 0x7fffffff) rep[g] = (int)(4 * i) + 1;
+                    if (FROM_U) {
+#pragma unroll
+                        for (int j = 0; j < C; ++j) {
+                            const float u0 = comp(uc[q][j], p);
+                            umin = fminf(umin, u0);  // NaN and infinities show in the sums instead
+                            const float wt = pow_m<MK>(u0, m);
+                            num[j] = fmaf(wt, xi, num[j]);
+                            den[j] += wt;
+                        }
+                    }
+                }
+            }
+            if (FROM_U) {
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                    df_add(acc[j], num[j]);
+                    df_add(acc[C + j], den[j]);
+                }
+            }
+        }
+    } else
     // the loop bounds are the same for all lanes of a warp (its first lane's
     // index); lanes past n load nothing and count nothing
     for (int64_t i0 = (int64_t)blockIdx.x * HNT + threadIdx.x; i0 - lane_id < n; i0 += stride * HCHUNK) {
@@ -320,7 +377,7 @@ __global__ void __launch_bounds__(BIN_NT) k_hist_solve(HistState* st, const doub
 }
 
 // U^k by table lookup: U_ij = table[x_i][j].
-template <int C>
+template <int C, bool VEC>
 __global__ void __launch_bounds__(HNT) k_hist_emit(const float* __restrict__ x, int64_t n,
                                                   const float* __restrict__ table, const HistState* st,
                                                   float* __restrict__ U) {
@@ -329,6 +386,18 @@ __global__ void __launch_bounds__(HNT) k_hist_emit(const float* __restrict__ x, 
     for (int t = threadIdx.x; t < 256 * C; t += HNT) T[t] = table[t];
     __syncthreads();
     const int64_t stride = (int64_t)gridDim.x * HNT;
+    if (VEC) {
+        for (int64_t i = (int64_t)blockIdx.x * HNT + threadIdx.x; i < n >> 2; i += stride) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(x) + i);
+            const int b[4] = {(int)v.x, (int)v.y, (int)v.z, (int)v.w};
+            const bool ok = (unsigned)(b[0] | b[1] | b[2] | b[3]) < 256u;
+            if (!in_bounds(ok, const_cast<unsigned*>(&st->bounds))) continue;
+#pragma unroll
+            for (int j = 0; j < C; ++j)
+                st_u4(U + (int64_t)j * n + 4 * i, make_float4(T[b[0] * C + j], T[b[1] * C + j], T[b[2] * C + j], T[b[3] * C + j]));
+        }
+        return;
+    }
     for (int64_t i = (int64_t)blockIdx.x * HNT + threadIdx.x; i < n; i += stride) {
         const int b = (int)__ldg(x + i);
         if (!in_bounds(b >= 0 && b < 256, const_cast<unsigned*>(&st->bounds))) continue;
@@ -343,18 +412,19 @@ typedef void (*SolveFn)(HistState*, const double*, int, const float*, int64_t, f
 typedef void (*EmitFn)(const float*, int64_t, const float*, const HistState*, float*);
 
 struct HistKernels {
-    Pass0Fn pass0[2];
+    Pass0Fn pass0[2][2];  // [from U^0][quads]
     Delta1Fn delta1;
     SolveFn solve[2];
-    EmitFn emit;
+    EmitFn emit[2];  // [quads]
 };
 
 template <int C, int MK>
 HistKernels kernels_cm() {
-    return HistKernels{{k_hist_pass0<C, MK, false>, k_hist_pass0<C, MK, true>},
+    return HistKernels{{{k_hist_pass0<C, MK, false, false>, k_hist_pass0<C, MK, false, true>},
+                        {k_hist_pass0<C, MK, true, false>, k_hist_pass0<C, MK, true, true>}},
                        k_hist_delta1<C, MK>,
                        {k_hist_solve<C, MK, false>, k_hist_solve<C, MK, true>},
-                       k_hist_emit<C>};
+                       {k_hist_emit<C, false>, k_hist_emit<C, true>}};
 }
 
 template <int C>
@@ -450,12 +520,14 @@ extern "C" int fcm_run_hist(fcm_handle h, const float* x, int64_t n, int C, floa
     const HistKernels k = kernels_for(C, mkind_of(m));
     const float inv_m1 = (float)(1.0 / ((double)m - 1.0));
     const int fu = from_u ? 1 : 0;
-    k.pass0[fu]<<<nblocks, HNT, 0, h->stream>>>(x, from_u ? U0 : nullptr, n, m, w->d_st, w->part);
+    const auto quads = [](const void* p) { return (uintptr_t)p % 16 == 0; };
+    const int v0 = n % 4 == 0 && quads(x) && (!from_u || quads(U0)), v1 = n % 4 == 0 && quads(x) && quads(U);
+    k.pass0[fu][v0]<<<nblocks, HNT, 0, h->stream>>>(x, from_u ? U0 : nullptr, n, m, w->d_st, w->part);
     k.solve[fu]<<<1, BIN_NT, 0, h->stream>>>(w->d_st, w->part, nblocks, U0, n, w->table, m, inv_m1, eps, max_iter, 0);
     // these return at once unless the solver's bound left the first stop open
     if (from_u) k.delta1<<<nblocks, HNT, 0, h->stream>>>(x, U0, n, m, inv_m1, w->d_st);
     k.solve[fu]<<<1, BIN_NT, 0, h->stream>>>(w->d_st, w->part, nblocks, U0, n, w->table, m, inv_m1, eps, max_iter, 1);
-    k.emit<<<nblocks, HNT, 0, h->stream>>>(x, n, w->table, w->d_st, U);
+    k.emit[v1]<<<nblocks, HNT, 0, h->stream>>>(x, n, w->table, w->d_st, U);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(hs, w->d_st, sizeof(HistState), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemcpyAsync(V, &w->d_st->V, sizeof(float) * C, V_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
