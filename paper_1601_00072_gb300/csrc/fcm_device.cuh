@@ -392,9 +392,11 @@ struct PackedCenters {
 //             The products' roundings average out in the sums, but not in a
 //             pixel's u (at C = 8 up to 7e-7, against 2e-7): u itself takes the
 //             weight form, w_j = (d2min / d2_j)^2.
+//   WEIGHTS takes the weight form of u at m = 2 and 3 too (w_j = d2min / d2_j, its
+//   square root): the grey-level kernels, whose 256 bins are a pixel each.
 //   other m   w_j = 2^t_j, t_j = (log2 d2min - log2 d2_j) / (m - 1), S = sum w:
 //             u_j^m = 2^(m (t_j - log2 S)), without the C logarithms of u_j.
-template <int C, int MK, bool POWERS, int N>
+template <int C, int MK, bool POWERS, int N, bool WEIGHTS = MK == M_ONE_HALF>
 __device__ __forceinline__ void packed_pairs(const f2 (&x2)[N], const PackedCenters<C, MK>& c, float m, float inv_m1,
                                              f2 (&w2)[N][C], f2 (&d2)[N][C], f2 (&J2)[N]) {
 #pragma unroll
@@ -403,7 +405,7 @@ __device__ __forceinline__ void packed_pairs(const f2 (&x2)[N], const PackedCent
 #pragma unroll
         for (int j = 0; j < C; ++j) d2[p][j] = sub2(xs, c.v2[j]);
     }
-    if (MK == M_ONE_HALF && !POWERS) {
+    if (MK != M_GENERIC && WEIGHTS && !POWERS) {
         float mn[2 * N], low = __int_as_float(0x7f800000);
         f2 b[N][C];
 #pragma unroll
@@ -411,7 +413,7 @@ __device__ __forceinline__ void packed_pairs(const f2 (&x2)[N], const PackedCent
             mn[2 * p] = mn[2 * p + 1] = __int_as_float(0x7f800000);
 #pragma unroll
             for (int j = 0; j < C; ++j) {
-                b[p][j] = mul2(d2[p][j], d2[p][j]);
+                b[p][j] = (MK == M_THREE) ? abs2(d2[p][j]) : mul2(d2[p][j], d2[p][j]);
                 mn[2 * p] = fminf(mn[2 * p], lo2(b[p][j]));
                 mn[2 * p + 1] = fminf(mn[2 * p + 1], hi2(b[p][j]));
             }
@@ -425,15 +427,21 @@ __device__ __forceinline__ void packed_pairs(const f2 (&x2)[N], const PackedCent
 #pragma unroll
                 for (int j = 0; j < C; ++j) {
                     const f2 q = mul2(mn2, pack2(rcp_approx(lo2(b[p][j])), rcp_approx(hi2(b[p][j]))));
-                    w2[p][j] = mul2(q, q);
+                    w2[p][j] = (MK == M_ONE_HALF) ? mul2(q, q) : q;
                     S = add2(S, w2[p][j]);
                 }
                 const float ra = rcp_approx(lo2(S)), rb = rcp_approx(hi2(S));
 #pragma unroll
                 for (int j = 0; j < C; ++j) w2[p][j] = mul2(w2[p][j], pack2(ra, rb));
-                // d2min S^(-1/2), back from scaled differences
-                const float q = rcp_approx(lo2(c.scale));  // of a power of two: exact
-                J2[p] = mul2(mul2(mn2, pack2(sqrt_approx(ra), sqrt_approx(rb))), pack2(q * q, q * q));
+                if (MK == M_ONE_HALF) {
+                    // d2min S^(-1/2), back from scaled differences
+                    const float q = rcp_approx(lo2(c.scale));  // of a power of two: exact
+                    J2[p] = mul2(mul2(mn2, pack2(sqrt_approx(ra), sqrt_approx(rb))), pack2(q * q, q * q));
+                } else {
+                    // d2min / S (m = 2), d2min / S^2 (m = 3)
+                    J2[p] = mul2(mn2, pack2(ra, rb));
+                    if (MK == M_THREE) J2[p] = mul2(J2[p], J2[p]);
+                }
             }
             return;
         }

@@ -165,7 +165,7 @@ __device__ __forceinline__ void bin_memberships(f2 b2, const PackedCenters<C, MK
                                                 f2 (&u2)[C], f2 (&um2)[C], f2 (&d2)[C], f2& J2) {
     f2 w[1][C], d[1][C], j[1];
     const f2 x[1] = {b2};
-    packed_pairs<C, MK, false, 1>(x, cen, m, inv_m1, w, d, j);
+    packed_pairs<C, MK, false, 1, true>(x, cen, m, inv_m1, w, d, j);
     J2 = j[0];
 #pragma unroll
     for (int q = 0; q < C; ++q) {
