@@ -1,8 +1,11 @@
 // Host runtime and C ABI of the single-image FCM path.
 //
-// A handle owns a device workspace (run state, per-block partials, optional
-// trace, staging buffers for host inputs) and one instantiated CUDA graph per
-// launch shape. A graph is
+// A run is one cooperative launch of k_fcm_run: its arguments go by value and
+// its results to pinned host memory, so nothing else crosses the host link but
+// the copies of host buffers. With FCM_OPT_NO_PERSISTENT, NO_GRAPH or NO_TMA it is
+// one launch per pass instead: a handle owns a device workspace (run state, per-block partials,
+// optional trace, staging buffers for host inputs) and one instantiated CUDA
+// graph per launch shape for these. A graph is
 //
 //     first pass (P_ACCUM0 or P_INITV)  ->  WHILE(cond) { P_ITER pass }
 //
@@ -10,7 +13,7 @@
 // cudaGraphSetConditional, so the whole of Algorithm 1 (arXiv:1601.00072,
 // Sec. 2.1) runs on the device after one graph launch. The paper copies U to
 // the host every iteration to test convergence (Sec. 4.3); here the only
-// host-device traffic of a run is the 200-byte state upload, the state
+// host-device traffic of such a run is the 200-byte state upload, the state
 // read-back and, for host buffers, the input/output copies.
 #include <cuda_runtime.h>
 

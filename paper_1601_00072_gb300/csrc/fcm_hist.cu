@@ -260,7 +260,8 @@ __global__ void __launch_bounds__(HNT) k_hist_delta1(const float* __restrict__ x
 // phase 0 leave the run to k_hist_delta1, which takes it over every pixel, and to
 // phase 1. A pass over x and U^0 (50 us of a 256^3 volume's 317) is thus skipped
 // whenever it could not change the run. 60 iterations of that volume: 314 -> 239 us
-// (the bins, at 1.2 us per iteration before, among it).
+// with this and the bin loop in packed pairs (1.2 us per iteration before); 226 us
+// with 128-bit loads and stores in the pixel passes as well.
 template <int C, int MK, bool FROM_U>
 __global__ void __launch_bounds__(BIN_NT) k_hist_solve(HistState* st, const double* __restrict__ part, int nblocks,
                                                       const float* __restrict__ U0, int64_t n,
