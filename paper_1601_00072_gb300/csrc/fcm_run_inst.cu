@@ -335,8 +335,11 @@ struct RunShared {
     float v[4][C];             // V^k in v[k % 4]
     DF v64[4][C];              // the double-float quotients behind them
     unsigned empty[4];         // whether some cluster was empty in the sums behind V^k
-    int4 ctl;                  // x: a wait gave up; y: a sampled change reached eps; z: some
-                               // den_j is too small for the exchange words
+    // By the parity of the iteration: the control warp writes the next iteration's
+    // while slower warps still read this one's (no barrier is between them).
+    // x: a wait gave up; y: a sampled change reached eps; z: some den_j is too small
+    // for the exchange words.
+    int4 ctl[2];
     DF J;
     float delta;
     unsigned flags;            // bit 0: bad input
@@ -464,13 +467,14 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         sh.v64[0][threadIdx.x] = DF{v0, 0.0f};
     }
     if (threadIdx.x == 0) {
-        sh.ctl = make_int4(0, 0, 0, 0);
+        sh.ctl[0] = sh.ctl[1] = make_int4(0, 0, 0, 0);
         sh.empty[0] = sh.empty[1] = sh.empty[2] = sh.empty[3] = 0u;
         sh.lim = ra.lim;
     }
     __syncthreads();
     int flags = 0;    // thread 0 of block 0 only
     unsigned nx = 0;  // exchanges so far
+    int it = 0;       // parity of the iteration (0 in pass 0)
 
     // The words of this run's bank (runs alternate between two; each run clears
     // the other one, which the next run uses): [parity][cluster] pairs and, in row
@@ -509,7 +513,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         if (lane == 0) {
             sh.delta = __uint_as_float(tm);
             sh.flags = tf;
-            if (!ok) sh.ctl.x = 1;
+            if (!ok) sh.ctl[it].x = 1;
         }
     };
     // V^{k+1}_q from the totals (one lane).
@@ -553,7 +557,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
                 da = df_merge_raw(da, DF{__shfl_xor_sync(0xffffffffu, da.hi, o), __shfl_xor_sync(0xffffffffu, da.lo, o)});
         }
         if (lane != 0) return;
-        if (!ok) sh.ctl.x = 1;
+        if (!ok) sh.ctl[it].x = 1;
         na = df_norm(na);
         if (K == X_J) {
             sh.J = na;
@@ -594,8 +598,8 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         const int64_t sa = (int64_t)(va - pa - (uint64_t)nb * ARRIVAL), sb = (int64_t)(vb - pb - (uint64_t)nb * ARRIVAL);
         (odd ? seen_a1 : seen_a0) = va;
         (odd ? seen_b1 : seen_b0) = vb;
-        if (!ok) sh.ctl.x = 1;
-        if (sb < (1ll << 37)) sh.ctl.z = 1;
+        if (!ok) sh.ctl[it].x = 1;
+        if (sb < (1ll << 37)) sh.ctl[it].z = 1;
         else new_center(q, fixed_to_df(sa, num_unit), fixed_to_df(sb, den_unit), true, cur, nxt);
     };
     // Control warp: publishes whether this block's sample of iteration k reached
@@ -609,9 +613,9 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         const uint64_t pa = (k & 1) ? seen_a1 : seen_a0;
         uint64_t va, vb;
         const bool ok = poll(word(nonce, k, C), va, vb, [&](uint64_t x, uint64_t) { return ((x - pa) & 0xffffu) == (unsigned)nb; });
-        sh.ctl.y = ((va - pa) >> 16) != 0;
+        sh.ctl[it].y = ((va - pa) >> 16) != 0;
         ((k & 1) ? seen_a1 : seen_a0) = va;
-        if (!ok) sh.ctl.x = 1;
+        if (!ok) sh.ctl[it].x = 1;
     };
     // ---- pass 0: V^1 from U^0, or from U^0 = f(x, V^0) ----
     bool ok;
@@ -706,7 +710,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         else if (warp < C) exchange_sums(std::integral_constant<int, X_SUMS>(), warp, 0, 1);
         ++nx;
         __syncthreads();
-        ok = sh.ctl.x == 0;
+        ok = sh.ctl[0].x == 0;
     }
     // The fixed-point units: |num_j| <= 2 n max(|x|, |V^0|) and den_j <= n, so the
     // totals stay below 2^53 units. Images whose FP32 sums could overflow get
@@ -880,7 +884,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         }
         ++nx;
         __syncthreads();
-        if (sh.ctl.x) return false;
+        if (sh.ctl[it].x) return false;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             st->delta = sh.delta;
             st->J = df_to_double(sh.J);
@@ -907,6 +911,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     for (int k = 1; ok; ++k) {
         const bool last = k == max_iter, prev_u0 = from_u && k == 1;
         const int cur = k & 3, prv = (k - 1) & 3, nxt = (k + 1) & 3;
+        it = k & 1;
         if (!last) {
             if (control) {
                 float d = 0.0f;
@@ -937,7 +942,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         }
         ++nx;
         __syncthreads();
-        int4 ctl = sh.ctl;
+        const int4 ctl = sh.ctl[it];
         if (ctl.x) {
             ok = give_up(k);
             break;
@@ -945,11 +950,11 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         if (ctl.z) {
             // uniform over the grid: every block has read the same words
             __syncthreads();
-            if (threadIdx.x == 0) sh.ctl.z = 0;
+            if (threadIdx.x == 0) sh.ctl[it].z = 0;
             if (warp < C) exchange_sums(std::integral_constant<int, X_SUMS>(), warp, cur, nxt);
             ++nx;
             __syncthreads();
-            if (sh.ctl.x) {
+            if (sh.ctl[it].x) {
                 ok = give_up(k);
                 break;
             }

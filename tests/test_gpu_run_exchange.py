@@ -1,0 +1,53 @@
+"""The exchanges and stop decisions of the whole-run kernel (needs a GPU): many
+short runs in a row, whose results must not depend on how the blocks' warps
+happen to be scheduled."""
+import numpy as np
+import pytest
+
+import oracle
+from parity import assert_within, eps32, precision_report
+
+pytestmark = pytest.mark.gpu
+
+EPS = 1e-5
+
+
+@pytest.fixture(scope="module")
+def fcm():
+    from paper_1601_00072_gb300 import _build
+    _build.build()
+    from paper_1601_00072_gb300.fcm import FCM
+    h = FCM(0)
+    yield h
+    h.close()
+
+
+def _cuda(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+
+
+def _lone_pixels(n):
+    """Almost every pixel sits near a center; a few lie between, mostly outside
+    the sampled pairs, so that samples decide some iterations and not others."""
+    rng = np.random.default_rng(n)
+    x = np.where(rng.random(n) < 0.5, 20.0, 200.0) + np.rint(3.0 * rng.standard_normal(n))
+    x[n // 3], x[n // 2 + 1] = 108.0, 113.0
+    return x, np.array([60.3, 150.1])
+
+
+@pytest.mark.parametrize("n", [600, 3001, 40000])
+def test_decisions_repeat(fcm, n):
+    """A block's warps agree on every decision: 200 runs give the same bits."""
+    x, V0 = _lone_pixels(n)
+    o = oracle.fcm(x, 2, 2.0, eps32(EPS), 300, V0=V0)
+    dx, dv = _cuda(x), _cuda(V0)
+    first = None
+    for _ in range(200):
+        g = fcm.run(dx, 2, 2.0, EPS, 300, V0=dv.clone())
+        got = (g.status, g.iters, g.delta, g.J, g.V.cpu().numpy().tobytes())
+        first = first or got
+        assert got == first
+    assert g.status == 0 and abs(g.iters - o["iters"]) <= 1
+    if g.iters == o["iters"]:
+        assert_within(precision_report(g.U.cpu().numpy(), g.V.cpu().numpy(), g.iters, o["U"], o["V"], o["iters"], g.J, o["J"][-1]))
