@@ -936,11 +936,14 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
                 __syncthreads();
                 if (warp < C) exchange_words(warp, cur, nxt);
             }
+            ++nx;
         } else {
+            // no exchange, and so none counted: the full pass's slots are those of
+            // the other parity than the last exchange's, which another block may
+            // still be reading
             if (control && k > 1) collect_decision(k - 1);
             __syncthreads();
         }
-        ++nx;
         __syncthreads();
         const int4 ctl = sh.ctl[it];
         if (ctl.x) {

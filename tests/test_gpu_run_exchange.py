@@ -51,3 +51,34 @@ def test_decisions_repeat(fcm, n):
     assert g.status == 0 and abs(g.iters - o["iters"]) <= 1
     if g.iters == o["iters"]:
         assert_within(precision_report(g.U.cpu().numpy(), g.V.cpu().numpy(), g.iters, o["U"], o["V"], o["iters"], g.J, o["J"][-1]))
+
+
+@pytest.mark.parametrize("n", [520, 4000, 40001])
+@pytest.mark.parametrize("max_iter", [1, 2, 3])
+@pytest.mark.parametrize("kw", [{}, {"trace": True}], ids=["plain", "trace"])
+def test_runs_that_end_at_max_iter(fcm, n, max_iter, kw):
+    """The last iteration has no exchange of sums; its full pass follows an
+    earlier slot exchange at once. Every run ends, alike, and as the oracle's."""
+    x, V0 = _lone_pixels(n)
+    o = oracle.fcm(x, 2, 2.0, 0.0, max_iter, V0=V0)
+    dx, dv = _cuda(x), _cuda(V0)
+    first = None
+    for _ in range(100):
+        g = fcm.run(dx, 2, 2.0, 0.0, max_iter, V0=dv.clone(), **kw)
+        got = (g.status, g.iters, g.delta, g.J, g.V.cpu().numpy().tobytes())
+        first = first or got
+        assert got == first
+    assert g.status == 1 and g.iters == max_iter
+    assert_within(precision_report(g.U.cpu().numpy(), g.V.cpu().numpy(), g.iters, o["U"], o["V"], o["iters"], g.J, o["J"][-1]))
+
+
+def test_undecided_iterations_before_max_iter(fcm):
+    """Full passes of the last three iterations, one after the other."""
+    x, V0 = _lone_pixels(3001)
+    dx, dv = _cuda(x), _cuda(V0)
+    end = fcm.run(dx, 2, 2.0, EPS, 300, V0=dv.clone()).iters
+    for max_iter in range(2, end + 1):
+        o = oracle.fcm(x, 2, 2.0, eps32(EPS), max_iter, V0=V0)
+        for _ in range(20):
+            g = fcm.run(dx, 2, 2.0, EPS, max_iter, V0=dv.clone())
+            assert g.status in (0, 1) and abs(g.iters - o["iters"]) <= 1
