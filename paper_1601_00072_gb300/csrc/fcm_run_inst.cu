@@ -32,9 +32,9 @@
 // 199x201 909 -> 188 us, 1024x1024 716 -> 275 us, 256^3 6.01 -> 1.83 ms.
 //
 // The exchange. Between iterations every block adds its totals of (num_j, den_j)
-// as 64-bit fixed-point numbers to one word each, with a reduction in the L2; the
+// as 64-bit fixed-point numbers to two words and one, with reductions in the L2; the
 // top byte of a word counts the arrivals, so the word itself says when the sum
-// is complete, and the warp that needs cluster j polls these two words and
+// is complete, and the warp that needs cluster j polls these three words and
 // nothing else. Integer sums do not depend on the order of arrival: every block
 // reads the same totals and forms the same V^{k+1}. (Slots that every block
 // polls for every other one cost 5,000 cycles per exchange at 152 blocks, most
@@ -42,10 +42,11 @@
 // The words are never cleared within a run: those of even and odd exchanges
 // alternate, and a sum is the difference from the word's value two exchanges
 // ago, which no block can have moved on from before all have read it. The
-// fixed-point unit comes from n and the largest |x|, |V^0|, known after pass 0;
-// it is 2^-53 of the largest total possible. A cluster whose den_j is below
-// 2^-16 n could lose precision to it: then (the same decision in every block) the
-// totals go through the slots instead, as do pass 0's and J's.
+// fixed-point units come from n and the largest |x|, |V^0|, known after pass 0;
+// num_j is resolved to 2^-97 of the largest total possible, den_j to 2^-46 (its
+// error is relative to the step of the center, not to the center). A cluster whose
+// den_j is below 2^-16 n could lose precision to that: then (the same decision in
+// every block) the totals go through the slots instead, as do pass 0's and J's.
 // Slots: a block's values with a 64-bit tag (the run's number and the exchange's
 // index) in one 16-byte store, polled until each block's shows the tag, added in
 // block order in compensated FP32.
@@ -144,15 +145,25 @@ __device__ __forceinline__ void ld_words(const uint64_t* p, uint64_t& a, uint64_
         : "l"(p)
         : "memory");
 }
+__device__ __forceinline__ uint64_t ld_word(const uint64_t* p) {
+    uint64_t a;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(a) : "l"(p) : "memory");
+    return a;
+}
 // The arrivals in a word's change since an earlier value; the sum in it may be
 // negative, but is below 2^55 in magnitude.
 __device__ __forceinline__ unsigned arrivals(uint64_t change) { return (unsigned)((change + (ARRIVAL >> 1)) >> 56); }
+// v * unit, |v| < 2^55 and unit a power of two: v in three parts of at most 24
+// bits, each exact, so the result is the value to about 48 bits of itself,
+// however small it is.
 __device__ __forceinline__ DF fixed_to_df(int64_t v, float unit) {
-    // the upper 24 bits exactly, the lower 31 rounded; then renormalised
-    const float a = (float)(int)(v >> 31) * 2147483648.0f, b = (float)(int)(v & 0x7fffffff);
-    const float hi = __fadd_rn(a, b);
-    return DF{hi * unit, __fsub_rn(b, __fsub_rn(hi, a)) * unit};
+    const float a = (float)(int)(v >> 32) * 4294967296.0f, b = (float)((unsigned)v >> 8) * 256.0f, c = (float)((unsigned)v & 255u);
+    const float s = __fadd_rn(a, b), e = __fadd_rn(__fsub_rn(b, __fsub_rn(s, a)), c), hi = __fadd_rn(s, e);
+    return DF{hi * unit, __fsub_rn(e, __fsub_rn(hi, s)) * unit};
 }
+// Bits of the sum of an exchange word: |num_j| in units of the high word, the
+// further bits that the low word resolves, and den_j.
+constexpr int NUM_BITS = 53, LOW_BITS = 44, DEN_BITS = 46;
 // 2^e for e in [-126, 127].
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
@@ -340,6 +351,8 @@ struct RunShared {
     // x: a wait gave up; y: a sampled change reached eps; z: some den_j is too small
     // for the exchange words.
     int4 ctl[2];
+    uint64_t seen[2][C][3];    // the words of each cluster after their last exchange, of even and odd parity
+    uint64_t seen_ctl[2];      // and the control word
     DF J;
     float delta;
     unsigned flags;            // bit 0: bad input
@@ -461,6 +474,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     const int max_iter = ra.max_iter;
     const bool tracing = ra.trace != nullptr;
 
+    if (threadIdx.x < 6 * C) (&sh.seen[0][0][0])[threadIdx.x] = 0ull;
     if (threadIdx.x < C) {
         const float v0 = ra.Vin ? ra.Vin[threadIdx.x] : ra.V0[threadIdx.x];
         sh.v[0][threadIdx.x] = v0;
@@ -468,6 +482,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     }
     if (threadIdx.x == 0) {
         sh.ctl[0] = sh.ctl[1] = make_int4(0, 0, 0, 0);
+        sh.seen_ctl[0] = sh.seen_ctl[1] = 0ull;
         sh.empty[0] = sh.empty[1] = sh.empty[2] = sh.empty[3] = 0u;
         sh.lim = ra.lim;
     }
@@ -477,19 +492,17 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     int it = 0;       // parity of the iteration (0 in pass 0)
 
     // The words of this run's bank (runs alternate between two; each run clears
-    // the other one, which the next run uses): [parity][cluster] pairs and, in row
+    // the other one, which the next run uses): [parity][cluster] triples and, in row
     // C, the control word, a 128-byte line each.
     auto word = [&](unsigned bank, unsigned x, int q) {
         return reinterpret_cast<uint64_t*>(scratch + RUN_WORD_BYTES * (((bank & 1) * 2 + (x & 1)) * (FCM_MAX_CLUSTERS + 1) + q));
     };
     if (blockIdx.x == 0 && threadIdx.x < 2 * (FCM_MAX_CLUSTERS + 1)) {
         uint64_t* const w = word(nonce + 1, threadIdx.x & 1, threadIdx.x >> 1);
-        w[0] = w[1] = 0ull;
+        w[0] = w[1] = w[2] = 0ull;
     }
     char* const slots_raw = scratch + RUN_WORDS_BYTES;
-    // this warp's words after their last exchange, of even and odd parity
-    uint64_t seen_a0 = 0ull, seen_b0 = 0ull, seen_a1 = 0ull, seen_b1 = 0ull;
-    float to_num = 0.0f, to_den = 0.0f, num_unit = 0.0f, den_unit = 0.0f;  // fixed-point scales
+    float to_num = 0.0f, to_low = 0.0f, to_den = 0.0f, num_unit = 0.0f, low_unit = 0.0f, den_unit = 0.0f;  // fixed-point scales
 
     // This block's row of exchange nx + 1: cluster q's slots, or (q = C) the
     // maxima's and flags'.
@@ -566,12 +579,11 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         da = df_norm(da);
         new_center(q, na, da, K == X_SUMS, cur, nxt);
     };
-    // Polls a pair of words until f(a, b) says that they are complete.
-    auto poll = [&](const uint64_t* w, uint64_t& a, uint64_t& b, auto&& complete) {
+    // Reads words until they are complete.
+    auto poll = [&](auto&& complete) {
         const uint32_t limit = sh.lim.grid_spins, phantoms = sh.lim.phantoms;
         for (uint32_t spins = 0;;) {
-            ld_words(w, a, b);
-            if (complete(a, b) && phantoms == 0) return true;
+            if (complete() && phantoms == 0) return true;
             if (++spins > limit) return false;
             if (spins > 256) __nanosleep(100);
         }
@@ -587,20 +599,27 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
             b += __shfl_xor_sync(0xffffffffu, b, o);
         }
         if (lane != 0) return;
-        red_add_u64(w, (uint64_t)__float2ll_rn(a * to_num) + ARRIVAL);
+        // what the high word's unit leaves of num_j goes to the low word
+        const float ah = rintf(a * to_num), al = fmaf(-ah, num_unit, a);
+        red_add_u64(w, (uint64_t)__float2ll_rn(ah) + ARRIVAL);
+        red_add_u64(w + 2, (uint64_t)__float2ll_rn(al * to_low) + ARRIVAL);
         red_add_u64(w + 1, (uint64_t)__float2ll_rn(b * to_den) + ARRIVAL);
-        const bool odd = (nx + 1) & 1;
-        const uint64_t pa = odd ? seen_a1 : seen_a0, pb = odd ? seen_b1 : seen_b0;
-        uint64_t va, vb;
-        const bool ok = poll(w, va, vb, [&](uint64_t x, uint64_t y) {
-            return arrivals(x - pa) == (unsigned)nb && arrivals(y - pb) == (unsigned)nb;
+        uint64_t* const seen = sh.seen[(nx + 1) & 1][q];
+        const uint64_t pa = seen[0], pb = seen[1], pc = seen[2];
+        uint64_t va, vb, vc;
+        const bool ok = poll([&] {
+            ld_words(w, va, vb);
+            vc = ld_word(w + 2);
+            return arrivals(va - pa) == (unsigned)nb && arrivals(vb - pb) == (unsigned)nb && arrivals(vc - pc) == (unsigned)nb;
         });
-        const int64_t sa = (int64_t)(va - pa - (uint64_t)nb * ARRIVAL), sb = (int64_t)(vb - pb - (uint64_t)nb * ARRIVAL);
-        (odd ? seen_a1 : seen_a0) = va;
-        (odd ? seen_b1 : seen_b0) = vb;
+        const uint64_t all = (uint64_t)nb * ARRIVAL;
+        const int64_t sa = (int64_t)(va - pa - all), sb = (int64_t)(vb - pb - all), sc = (int64_t)(vc - pc - all);
+        seen[0] = va;
+        seen[1] = vb;
+        seen[2] = vc;
         if (!ok) sh.ctl[it].x = 1;
-        if (sb < (1ll << 37)) sh.ctl[it].z = 1;
-        else new_center(q, fixed_to_df(sa, num_unit), fixed_to_df(sb, den_unit), true, cur, nxt);
+        if (sb < (1ll << (DEN_BITS - 16))) sh.ctl[it].z = 1;
+        else new_center(q, df_merge(fixed_to_df(sa, num_unit), fixed_to_df(sc, low_unit)), fixed_to_df(sb, den_unit), true, cur, nxt);
     };
     // Control warp: publishes whether this block's sample of iteration k reached
     // eps; collects, an iteration later, whether any block's did.
@@ -610,11 +629,15 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     };
     auto collect_decision = [&](int k) {
         if (lane != 0) return;
-        const uint64_t pa = (k & 1) ? seen_a1 : seen_a0;
-        uint64_t va, vb;
-        const bool ok = poll(word(nonce, k, C), va, vb, [&](uint64_t x, uint64_t) { return ((x - pa) & 0xffffu) == (unsigned)nb; });
+        const uint64_t* const w = word(nonce, k, C);
+        const uint64_t pa = sh.seen_ctl[k & 1];
+        uint64_t va;
+        const bool ok = poll([&] {
+            va = ld_word(w);
+            return ((va - pa) & 0xffffu) == (unsigned)nb;
+        });
         sh.ctl[it].y = ((va - pa) >> 16) != 0;
-        ((k & 1) ? seen_a1 : seen_a0) = va;
+        sh.seen_ctl[k & 1] = va;
         if (!ok) sh.ctl[it].x = 1;
     };
     // ---- pass 0: V^1 from U^0, or from U^0 = f(x, V^0) ----
@@ -712,18 +735,25 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         __syncthreads();
         ok = sh.ctl[0].x == 0;
     }
-    // The fixed-point units: |num_j| <= 2 n max(|x|, |V^0|) and den_j <= n, so the
-    // totals stay below 2^53 units. Images whose FP32 sums could overflow get
-    // scale 0: every total is then thin, and goes through the slots.
+    // The fixed-point units: |num_j| <= 2 n max(|x|, |V^0|) < 2^NUM_BITS units of the
+    // high word and den_j <= n. The low word goes on where the high one ends: a few
+    // far outliers, or a masked part at some sentinel value, set the largest |x|,
+    // and the other clusters' numerators may lie wholly below the high word's unit
+    // (one word alone stood still, "converged", from a sentinel of 1e15 on). The
+    // two words together cover 2^-97 of the largest total, or 2^-126. Images whose
+    // FP32 sums could overflow get scale 0: every total is then thin, and goes
+    // through the slots.
     {
         const int en = 64 - __clzll(n);                                        // n < 2^en
         const int ex = max(-100, (__float_as_int(sh.delta) >> 23) - 125);      // 2 max|x| < 2^ex
-        const int e = max(-126, min(126, 53 - en - ex));
+        const int e = min(126, NUM_BITS - en - ex), el = min(126, e + LOW_BITS);
         const bool use = en + ex <= 126;
         to_num = use ? pow2f(e) : 0.0f;
-        num_unit = pow2f(-e);
-        to_den = use ? pow2f(53 - en) : 0.0f;
-        den_unit = pow2f(en - 53);
+        to_low = use ? pow2f(el) : 0.0f;
+        num_unit = use ? pow2f(-e) : 0.0f;
+        low_unit = use ? pow2f(-el) : 0.0f;
+        to_den = use ? pow2f(DEN_BITS - en) : 0.0f;
+        den_unit = pow2f(en - DEN_BITS);
     }
     int status = FCM_NOT_CONVERGED, iters = 0;
     if (!ok) {

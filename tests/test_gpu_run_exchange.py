@@ -82,3 +82,51 @@ def test_undecided_iterations_before_max_iter(fcm):
         for _ in range(20):
             g = fcm.run(dx, 2, 2.0, EPS, max_iter, V0=dv.clone())
             assert g.status in (0, 1) and abs(g.iters - o["iters"]) <= 1
+
+
+def _tissues(n, seed):
+    rng = np.random.default_rng(seed)
+    x = np.where(rng.random(n) < 0.5, 30.0, 90.0) + 6.0 * rng.standard_normal(n)
+    return x.astype(np.float32).astype(np.float64), rng
+
+
+def _check_centers(fcm, x, C, m, V0, eps=EPS, max_iter=60):
+    """Against the oracle at the same iteration count."""
+    V0 = np.asarray(V0, np.float32).astype(np.float64)
+    g = fcm.run(_cuda(x), C, m, eps, max_iter, V0=_cuda(V0))
+    o = oracle.fcm(x, C, m, eps32(eps), max_iter, V0=V0)
+    assert abs(g.iters - o["iters"]) <= 1
+    k = min(g.iters, o["iters"])
+    if g.iters != o["iters"]:
+        g = fcm.run(_cuda(x), C, m, eps, k, V0=_cuda(V0))
+        o = oracle.fcm(x, C, m, eps32(eps), k, V0=V0)
+    assert_within(precision_report(g.U.cpu().numpy(), g.V.cpu().numpy(), g.iters, o["U"], o["V"], o["iters"]))
+    return g
+
+
+@pytest.mark.parametrize("m", [2.0, 1.5, 2.5])
+@pytest.mark.parametrize("share", [0.0, 0.01, 0.3], ids=["one", "1pc", "30pc"])
+@pytest.mark.parametrize("value", [1e6, -1e10, 1e12, 1e15, 1e18])
+def test_tissues_beside_a_sentinel(fcm, value, share, m):
+    """One far outlier, or a masked part at a sentinel value, with a cluster of
+    its own: the other centers move as if it were not there."""
+    n = 200004
+    x, rng = _tissues(n, 3)
+    if share:
+        x[rng.random(n) < share] = np.float32(value)
+    else:
+        x[n // 3] = np.float32(value)
+    _check_centers(fcm, x, 3, m, [20.0, 80.0, value])
+    _check_centers(fcm, x, 3, m, [20.0, 80.0, value], eps=0.0, max_iter=9)
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-20, 1e-12])
+def test_tiny_intensities(fcm, scale):
+    """All totals far below the largest unit."""
+    x, _ = _tissues(40000, 5)
+    x = (x * scale).astype(np.float32)
+    V0 = np.array([20.0, 80.0]) * scale
+    g = fcm.run(_cuda(x), 2, 2.0, 0.0, 8, V0=_cuda(V0))
+    o = oracle.fcm(x.astype(np.float64), 2, 2.0, 0.0, 8, V0=V0.astype(np.float32).astype(np.float64))
+    assert np.max(np.abs(g.V.cpu().numpy() - o["V"]) / o["V"]) <= 1e-5
+    assert np.max(np.abs(g.U.cpu().numpy() - o["U"])) <= 1e-5
