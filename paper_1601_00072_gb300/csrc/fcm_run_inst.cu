@@ -164,6 +164,7 @@ __device__ __forceinline__ DF fixed_to_df(int64_t v, float unit) {
 // Bits of the sum of an exchange word: |num_j| in units of the high word, the
 // further bits that the low word resolves, and den_j.
 constexpr int NUM_BITS = 53, LOW_BITS = 44, DEN_BITS = 46;
+constexpr uint64_t DEN_MARK = 2ull << DEN_BITS;  // 255 of them stay below 2^55
 // 2^e for e in [-126, 127].
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
@@ -600,10 +601,14 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         }
         if (lane != 0) return;
         // what the high word's unit leaves of num_j goes to the low word
-        const float ah = rintf(a * to_num), al = fmaf(-ah, num_unit, a);
-        red_add_u64(w, (uint64_t)__float2ll_rn(ah) + ARRIVAL);
-        red_add_u64(w + 2, (uint64_t)__float2ll_rn(al * to_low) + ARRIVAL);
-        red_add_u64(w + 1, (uint64_t)__float2ll_rn(b * to_den) + ARRIVAL);
+        const float ah = rintf(a * to_num), al = fmaf(-ah, num_unit, a), bd = b * to_den;
+        // Totals that are no fixed-point numbers (infinite or NaN: overflowed
+        // squares, an infinite center) must not reach the words' arrival counts:
+        // such a block adds only den_j's mark, beyond every possible sum of them.
+        const bool fits = fabsf(ah) <= (float)(1ull << NUM_BITS) && fabsf(al) <= 0.5f * num_unit && bd <= 1.25f * (float)(1ull << DEN_BITS);
+        red_add_u64(w, (fits ? (uint64_t)__float2ll_rn(ah) : 0ull) + ARRIVAL);
+        red_add_u64(w + 2, (fits ? (uint64_t)__float2ll_rn(al * to_low) : 0ull) + ARRIVAL);
+        red_add_u64(w + 1, (fits ? (uint64_t)__float2ll_rn(bd) : DEN_MARK) + ARRIVAL);
         uint64_t* const seen = sh.seen[(nx + 1) & 1][q];
         const uint64_t pa = seen[0], pb = seen[1], pc = seen[2];
         uint64_t va, vb, vc;
@@ -618,7 +623,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         seen[1] = vb;
         seen[2] = vc;
         if (!ok) sh.ctl[it].x = 1;
-        if (sb < (1ll << (DEN_BITS - 16))) sh.ctl[it].z = 1;
+        if (sb < (1ll << (DEN_BITS - 16)) || sb >= (int64_t)DEN_MARK) sh.ctl[it].z = 1;
         else new_center(q, df_merge(fixed_to_df(sa, num_unit), fixed_to_df(sc, low_unit)), fixed_to_df(sb, den_unit), true, cur, nxt);
     };
     // Control warp: publishes whether this block's sample of iteration k reached
@@ -741,8 +746,8 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     // and the other clusters' numerators may lie wholly below the high word's unit
     // (one word alone stood still, "converged", from a sentinel of 1e15 on). The
     // two words together cover 2^-97 of the largest total, or 2^-126. Images whose
-    // FP32 sums could overflow get scale 0: every total is then thin, and goes
-    // through the slots.
+    // FP32 sums could overflow get scale 0: every total is then thin or marked, and
+    // goes through the slots.
     {
         const int en = 64 - __clzll(n);                                        // n < 2^en
         const int ex = max(-100, (__float_as_int(sh.delta) >> 23) - 125);      // 2 max|x| < 2^ex

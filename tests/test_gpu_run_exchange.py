@@ -130,3 +130,29 @@ def test_tiny_intensities(fcm, scale):
     o = oracle.fcm(x.astype(np.float64), 2, 2.0, 0.0, 8, V0=V0.astype(np.float32).astype(np.float64))
     assert np.max(np.abs(g.V.cpu().numpy() - o["V"]) / o["V"]) <= 1e-5
     assert np.max(np.abs(g.U.cpu().numpy() - o["U"])) <= 1e-5
+
+
+def test_overflowed_totals(fcm):
+    """Totals that are infinite or NaN: squares beyond FP32 where no center sits
+    on the pixel, an infinite center. The run ends as the one that launches a
+    kernel per pass does, without waiting for sums that never arrive."""
+    n = 40004
+    x, rng = _tissues(n, 6)
+    far = x.copy()
+    far[rng.random(n) < 0.01] = 1e20
+    u0 = oracle.memberships(x, np.array([20.0, 80.0]), 2.0)
+    cases = [(far, {"V0": np.array([20.0, 80.0])}), (x, {"V0": np.array([20.0, 3e38])}), (1e9 * x, {"U0": 1e15 * u0}),
+             (far, {"U0": u0})]
+    for xs, start in cases:
+        got = []
+        for persistent in (True, False):
+            g = fcm.run(_cuda(xs), 2, 2.0, 0.0, 5, persistent=persistent, **{k: _cuda(v) for k, v in start.items()})
+            got.append(g)
+        a, b = got
+        assert (a.status, a.iters, a.flags) == (b.status, b.iters, b.flags)
+        va, vb = a.V.cpu().numpy(), b.V.cpu().numpy()
+        # (an overflowed quotient is NaN in compensated FP32 and infinite in FP64)
+        ok = np.isfinite(va)
+        assert np.array_equal(ok, np.isfinite(vb)) and np.allclose(va[ok], vb[ok], rtol=1e-5, atol=1e-5)
+    # and the handle goes on as before
+    _check_centers(fcm, x, 2, 2.0, [20.0, 80.0])
