@@ -32,9 +32,9 @@
 // 199x201 909 -> 188 us, 1024x1024 716 -> 275 us, 256^3 6.01 -> 1.83 ms.
 //
 // The exchange. Between iterations every block adds its totals of (num_j, den_j)
-// as 64-bit fixed-point numbers to two words and one, with reductions in the L2; the
+// as 64-bit fixed-point numbers to one word each, with a reduction in the L2; the
 // top byte of a word counts the arrivals, so the word itself says when the sum
-// is complete, and the warp that needs cluster j polls these three words and
+// is complete, and the warp that needs cluster j polls these two words and
 // nothing else. Integer sums do not depend on the order of arrival: every block
 // reads the same totals and forms the same V^{k+1}. (Slots that every block
 // polls for every other one cost 5,000 cycles per exchange at 152 blocks, most
@@ -42,11 +42,17 @@
 // The words are never cleared within a run: those of even and odd exchanges
 // alternate, and a sum is the difference from the word's value two exchanges
 // ago, which no block can have moved on from before all have read it. The
-// fixed-point units come from n and the largest |x|, |V^0|, known after pass 0;
-// num_j is resolved to 2^-97 of the largest total possible, den_j to 2^-46 (its
-// error is relative to the step of the center, not to the center). A cluster whose
-// den_j is below 2^-16 n could lose precision to that: then (the same decision in
-// every block) the totals go through the slots instead, as do pass 0's and J's.
+// fixed-point units come from n and the largest |x|, |V^0|, known after pass 0:
+// 2^-53 of the largest num_j possible, 2^-46 of n (the error of den_j is relative
+// to the center's step). A few outliers or a masked part at some sentinel value set
+// the largest |x|, and the other clusters' totals may lie wholly below the unit: a
+// block whose total loses more than its center's FP32 resolution to the rounding
+// says so in the word, and so does one whose total is no number; den_j below 2^-16 n
+// counts alike. Then (the same decision in every block) the totals go through the
+// slots, in FP32, and so do the next ones until the words would hold them. (A
+// second word for what the first one leaves of num_j is exact without that, but
+// costs every run: 40,000 pixels 151.6 -> 161.2 us on a line of its own, 172 on the
+// same line.) Pass 0's totals and J's always go through the slots.
 // Slots: a block's values with a 64-bit tag (the run's number and the exchange's
 // index) in one 16-byte store, polled until each block's shows the tag, added in
 // block order in compensated FP32.
@@ -153,18 +159,30 @@ __device__ __forceinline__ uint64_t ld_word(const uint64_t* p) {
 // The arrivals in a word's change since an earlier value; the sum in it may be
 // negative, but is below 2^55 in magnitude.
 __device__ __forceinline__ unsigned arrivals(uint64_t change) { return (unsigned)((change + (ARRIVAL >> 1)) >> 56); }
-// v * unit, |v| < 2^55 and unit a power of two: v in three parts of at most 24
-// bits, each exact, so the result is the value to about 48 bits of itself,
-// however small it is.
+// v * unit, |v| < 2^55 and unit a power of two, to 2^-25 of itself or better: the
+// upper part exactly, the lower 31 bits (signed) rounded; then renormalised.
 __device__ __forceinline__ DF fixed_to_df(int64_t v, float unit) {
-    const float a = (float)(int)(v >> 32) * 4294967296.0f, b = (float)((unsigned)v >> 8) * 256.0f, c = (float)((unsigned)v & 255u);
-    const float s = __fadd_rn(a, b), e = __fadd_rn(__fsub_rn(b, __fsub_rn(s, a)), c), hi = __fadd_rn(s, e);
-    return DF{hi * unit, __fsub_rn(e, __fsub_rn(hi, s)) * unit};
+    const int top = (int)((v + (1ll << 30)) >> 31);
+    const float a = (float)top * 2147483648.0f, b = (float)(int)(v - ((int64_t)top << 31));
+    const float hi = __fadd_rn(a, b);
+    return DF{hi * unit, __fsub_rn(b, __fsub_rn(hi, a)) * unit};
 }
-// Bits of the sum of an exchange word: |num_j| in units of the high word, the
-// further bits that the low word resolves, and den_j.
-constexpr int NUM_BITS = 53, LOW_BITS = 44, DEN_BITS = 46;
+// Bits of the sum of an exchange word.
+constexpr int NUM_BITS = 53, DEN_BITS = 46;
 constexpr uint64_t DEN_MARK = 2ull << DEN_BITS;  // 255 of them stay below 2^55
+// The units of the fixed-point numbers.
+struct Fixed {
+    float to_num, to_den, num_unit, den_unit;
+    float num_max, den_max;  // no block's totals are above these
+    // Whether the words hold a block's totals a = num_j, b = den_j about the center
+    // v: no infinity or NaN, and the rounding of a to the unit is below 2^-16 of a, or
+    // moves the block's part of the center by less than 2^-26 of it. slack > 1 asks
+    // for that much more room.
+    __device__ __forceinline__ bool holds(float a, float b, float v, float slack) const {
+        const float half = (0.5f * slack) * num_unit;
+        return (fabsf(a) >= 0x1p16f * half || b * fabsf(v) >= 0x1p26f * half || a == 0.0f) && fabsf(a) <= num_max && b <= den_max;
+    }
+};
 // 2^e for e in [-126, 127].
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
@@ -349,10 +367,11 @@ struct RunShared {
     unsigned empty[4];         // whether some cluster was empty in the sums behind V^k
     // By the parity of the iteration: the control warp writes the next iteration's
     // while slower warps still read this one's (no barrier is between them).
-    // x: a wait gave up; y: a sampled change reached eps; z: some den_j is too small
-    // for the exchange words.
+    // x: a wait gave up; y: a sampled change reached eps; z: the exchange words do not
+    // hold the sums, or (of an exchange through the slots) would not; w: some cluster
+    // is empty.
     int4 ctl[2];
-    uint64_t seen[2][C][3];    // the words of each cluster after their last exchange, of even and odd parity
+    uint64_t seen[2][C][2];    // the words of each cluster after their last exchange, of even and odd parity
     uint64_t seen_ctl[2];      // and the control word
     DF J;
     float delta;
@@ -475,7 +494,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     const int max_iter = ra.max_iter;
     const bool tracing = ra.trace != nullptr;
 
-    if (threadIdx.x < 6 * C) (&sh.seen[0][0][0])[threadIdx.x] = 0ull;
+    if (threadIdx.x < 4 * C) (&sh.seen[0][0][0])[threadIdx.x] = 0ull;
     if (threadIdx.x < C) {
         const float v0 = ra.Vin ? ra.Vin[threadIdx.x] : ra.V0[threadIdx.x];
         sh.v[0][threadIdx.x] = v0;
@@ -493,17 +512,18 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     int it = 0;       // parity of the iteration (0 in pass 0)
 
     // The words of this run's bank (runs alternate between two; each run clears
-    // the other one, which the next run uses): [parity][cluster] triples and, in row
+    // the other one, which the next run uses): [parity][cluster] pairs and, in row
     // C, the control word, a 128-byte line each.
     auto word = [&](unsigned bank, unsigned x, int q) {
         return reinterpret_cast<uint64_t*>(scratch + RUN_WORD_BYTES * (((bank & 1) * 2 + (x & 1)) * (FCM_MAX_CLUSTERS + 1) + q));
     };
     if (blockIdx.x == 0 && threadIdx.x < 2 * (FCM_MAX_CLUSTERS + 1)) {
         uint64_t* const w = word(nonce + 1, threadIdx.x & 1, threadIdx.x >> 1);
-        w[0] = w[1] = w[2] = 0ull;
+        w[0] = w[1] = 0ull;
     }
     char* const slots_raw = scratch + RUN_WORDS_BYTES;
-    float to_num = 0.0f, to_low = 0.0f, to_den = 0.0f, num_unit = 0.0f, low_unit = 0.0f, den_unit = 0.0f;  // fixed-point scales
+    Fixed fx{0.0f, 0.0f, 0.0f, 0.0f, -1.0f, -1.0f};  // holds nothing
+    float thick = 0.0f;  // least den_j, in slots, that the words may have again
 
     // This block's row of exchange nx + 1: cluster q's slots, or (q = C) the
     // maxima's and flags'.
@@ -542,6 +562,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
             sh.v[nxt][q] = centered ? sh.v[cur][q] : 0.0f;
             sh.v64[nxt][q] = centered ? sh.v64[cur][q] : DF{0.0f, 0.0f};
             sh.empty[nxt] = 1u;
+            sh.ctl[it].w = 1;
         }
     };
     // Warp q < C (q = 0 for X_J): the block's totals from the warp totals, then
@@ -559,10 +580,13 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         }
         if (lane == 0) st_slot(row + (int64_t)blockIdx.x * RUN_SLOT_BYTES, a, b, tag);
         DF na{0.0f, 0.0f}, da{0.0f, 0.0f};
+        bool slots = false;  // some block's totals do not fit the words with room to spare
         const bool ok = collect(row, nb, tag, sh.lim.grid_spins, sh.lim.phantoms, [&](float p, float r) {
+            if (K == X_SUMS) slots |= !fx.holds(p, r, sh.v[cur][q], 4.0f);
             df_add(na, p);
             if (K != X_J) df_add(da, r);
         });
+        if (K == X_SUMS) slots = __any_sync(0xffffffffu, slots);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             // TwoSum is symmetric: every lane gets the same totals
@@ -578,6 +602,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
             return;
         }
         da = df_norm(da);
+        if (slots || !(da.hi >= thick)) sh.ctl[it].z = 1;
         new_center(q, na, da, K == X_SUMS, cur, nxt);
     };
     // Reads words until they are complete.
@@ -593,6 +618,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     // then V^{k+1}_q from the complete ones (one lane polls).
     auto exchange_words = [&](int q, int cur, int nxt) {
         uint64_t* const w = word(nonce, nx + 1, q);
+        const float v = sh.v[cur][q];
         float a = lane < pw ? sh.red[lane][q] : 0.0f, b = lane < pw ? sh.red[lane][C + q] : 0.0f;
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) {
@@ -600,31 +626,24 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
             b += __shfl_xor_sync(0xffffffffu, b, o);
         }
         if (lane != 0) return;
-        // what the high word's unit leaves of num_j goes to the low word
-        const float ah = rintf(a * to_num), al = fmaf(-ah, num_unit, a), bd = b * to_den;
-        // Totals that are no fixed-point numbers (infinite or NaN: overflowed
-        // squares, an infinite center) must not reach the words' arrival counts:
-        // such a block adds only den_j's mark, beyond every possible sum of them.
-        const bool fits = fabsf(ah) <= (float)(1ull << NUM_BITS) && fabsf(al) <= 0.5f * num_unit && bd <= 1.25f * (float)(1ull << DEN_BITS);
-        red_add_u64(w, (fits ? (uint64_t)__float2ll_rn(ah) : 0ull) + ARRIVAL);
-        red_add_u64(w + 2, (fits ? (uint64_t)__float2ll_rn(al * to_low) : 0ull) + ARRIVAL);
-        red_add_u64(w + 1, (fits ? (uint64_t)__float2ll_rn(bd) : DEN_MARK) + ARRIVAL);
+        // Totals that the words do not hold add only a mark to den_j, beyond every
+        // possible sum of them: nothing but numbers reaches the arrival counts.
+        const bool fits = fx.holds(a, b, v, 1.0f);
+        red_add_u64(w, (uint64_t)__float2ll_rn(fits ? a * fx.to_num : 0.0f) + ARRIVAL);
+        red_add_u64(w + 1, (uint64_t)__float2ll_rn(fits ? b * fx.to_den : (float)DEN_MARK) + ARRIVAL);
         uint64_t* const seen = sh.seen[(nx + 1) & 1][q];
-        const uint64_t pa = seen[0], pb = seen[1], pc = seen[2];
-        uint64_t va, vb, vc;
+        const uint64_t pa = seen[0], pb = seen[1];
+        uint64_t va, vb;
         const bool ok = poll([&] {
             ld_words(w, va, vb);
-            vc = ld_word(w + 2);
-            return arrivals(va - pa) == (unsigned)nb && arrivals(vb - pb) == (unsigned)nb && arrivals(vc - pc) == (unsigned)nb;
+            return arrivals(va - pa) == (unsigned)nb && arrivals(vb - pb) == (unsigned)nb;
         });
-        const uint64_t all = (uint64_t)nb * ARRIVAL;
-        const int64_t sa = (int64_t)(va - pa - all), sb = (int64_t)(vb - pb - all), sc = (int64_t)(vc - pc - all);
+        const int64_t sa = (int64_t)(va - pa - (uint64_t)nb * ARRIVAL), sb = (int64_t)(vb - pb - (uint64_t)nb * ARRIVAL);
         seen[0] = va;
         seen[1] = vb;
-        seen[2] = vc;
         if (!ok) sh.ctl[it].x = 1;
         if (sb < (1ll << (DEN_BITS - 16)) || sb >= (int64_t)DEN_MARK) sh.ctl[it].z = 1;
-        else new_center(q, df_merge(fixed_to_df(sa, num_unit), fixed_to_df(sc, low_unit)), fixed_to_df(sb, den_unit), true, cur, nxt);
+        else new_center(q, fixed_to_df(sa, fx.num_unit), fixed_to_df(sb, fx.den_unit), true, cur, nxt);
     };
     // Control warp: publishes whether this block's sample of iteration k reached
     // eps; collects, an iteration later, whether any block's did.
@@ -740,26 +759,17 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         __syncthreads();
         ok = sh.ctl[0].x == 0;
     }
-    // The fixed-point units: |num_j| <= 2 n max(|x|, |V^0|) < 2^NUM_BITS units of the
-    // high word and den_j <= n. The low word goes on where the high one ends: a few
-    // far outliers, or a masked part at some sentinel value, set the largest |x|,
-    // and the other clusters' numerators may lie wholly below the high word's unit
-    // (one word alone stood still, "converged", from a sentinel of 1e15 on). The
-    // two words together cover 2^-97 of the largest total, or 2^-126. Images whose
-    // FP32 sums could overflow get scale 0: every total is then thin or marked, and
-    // goes through the slots.
-    {
-        const int en = 64 - __clzll(n);                                        // n < 2^en
-        const int ex = max(-100, (__float_as_int(sh.delta) >> 23) - 125);      // 2 max|x| < 2^ex
-        const int e = min(126, NUM_BITS - en - ex), el = min(126, e + LOW_BITS);
-        const bool use = en + ex <= 126;
-        to_num = use ? pow2f(e) : 0.0f;
-        to_low = use ? pow2f(el) : 0.0f;
-        num_unit = use ? pow2f(-e) : 0.0f;
-        low_unit = use ? pow2f(-el) : 0.0f;
-        to_den = use ? pow2f(DEN_BITS - en) : 0.0f;
-        den_unit = pow2f(en - DEN_BITS);
+    // The fixed-point units: |num_j| <= 2 n max(|x|, |V^0|) < 2^NUM_BITS units and
+    // den_j <= n. Images whose FP32 sums could overflow never use the words.
+    const int en = 64 - __clzll(n);                                        // n < 2^en
+    const int ex = max(-100, (__float_as_int(sh.delta) >> 23) - 125);      // 2 max|x| < 2^ex
+    const bool fixed = en + ex <= 126;
+    if (fixed) {
+        const int e = min(126, NUM_BITS - en - ex);
+        fx = Fixed{pow2f(e), pow2f(DEN_BITS - en), pow2f(-e), pow2f(en - DEN_BITS), pow2f(min(127, en + ex)), 1.25f * pow2f(en)};
+        thick = pow2f(en - 15);
     }
+    bool words = fixed;  // the next exchange of sums goes through the words (the same in every block)
     int status = FCM_NOT_CONVERGED, iters = 0;
     if (!ok) {
         status = FCM_ERR_TIMEOUT;
@@ -943,6 +953,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         return false;
     };
     if (ok && threadIdx.x == 0 && sh.empty[1]) flags |= FCM_FLAG_EMPTY_CLUSTER;
+    bool empty = false;  // some cluster is in the sums behind V^k, k > 1
     for (int k = 1; ok; ++k) {
         const bool last = k == max_iter, prev_u0 = from_u && k == 1;
         const int cur = k & 3, prv = (k - 1) & 3, nxt = (k + 1) & 3;
@@ -966,10 +977,16 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
                 if (k > 1) collect_decision(k - 1);
                 __syncthreads();
             } else {
-                if (threadIdx.x == 0) sh.empty[nxt] = 0u;
+                if (threadIdx.x == 0) {
+                    sh.empty[nxt] = 0u;
+                    sh.ctl[it].z = sh.ctl[it].w = 0;
+                }
                 sums_pass<C, MK>(px, sh, second, cur, m, inv_m1);
                 __syncthreads();
-                if (warp < C) exchange_words(warp, cur, nxt);
+                if (warp < C) {
+                    if (words) exchange_words(warp, cur, nxt);
+                    else exchange_sums(std::integral_constant<int, X_SUMS>(), warp, cur, nxt);
+                }
             }
             ++nx;
         } else {
@@ -981,14 +998,18 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         }
         __syncthreads();
         const int4 ctl = sh.ctl[it];
+        // nothing but the next iteration to do: one test, every warp waits for it
+        const bool plain = words && !last && !tracing && !empty && (ctl.x | ctl.z | ctl.w) == 0 && (k == 1 || ctl.y);
+        if (plain) continue;
+        empty = ctl.w != 0;  // behind V^{k+1}
         if (ctl.x) {
             ok = give_up(k);
             break;
         }
-        if (ctl.z) {
+        if (!last && words && ctl.z) {
             // uniform over the grid: every block has read the same words
+            words = false;
             __syncthreads();
-            if (threadIdx.x == 0) sh.ctl[it].z = 0;
             if (warp < C) exchange_sums(std::integral_constant<int, X_SUMS>(), warp, cur, nxt);
             ++nx;
             __syncthreads();
@@ -996,6 +1017,8 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
                 ok = give_up(k);
                 break;
             }
+        } else if (!last && !words) {
+            words = fixed && !ctl.z;
         }
         // Iteration k - 1's full pass when its sample could not decide, iteration
         // k's when it is the last (and every one for a trace).
