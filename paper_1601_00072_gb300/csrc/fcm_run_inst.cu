@@ -224,7 +224,8 @@ __device__ __forceinline__ int slot_of_lane(int lane) {
 // The numerators are centered: num_j = sum u_j^m (x - v_j^k), so that
 // v_j^{k+1} = v_j^k + num_j / den_j. The differences are at hand, and the FP32
 // rounding of the sums is then relative to the pixels' distance from the center
-// and not to their grey level, and vanishes from den as the run converges.
+// and not to their grey level, and vanishes from den as the run converges. (A
+// center that moves by more than it is worth takes its sums again: rebased_pass.)
 //
 // Sums in two levels: pairs into num2/den2, those into a second set after every
 // FOLD quads. A thread's share of a 256^3 volume is 27 quads; many of its terms
@@ -356,6 +357,23 @@ struct Px {
     }
 };
 
+// This thread's pixels. second: the block's dynamic shared memory.
+template <int C>
+__device__ __forceinline__ Px run_px(const RunArgs& ra, f2* second) {
+    Px px;
+    px.x = ra.x;
+    px.n = ra.n;
+    px.pt = (int)blockDim.x - 32;
+    px.xs = reinterpret_cast<float4*>(second + 2 * C * px.pt) + threadIdx.x;
+    px.t0 = (int64_t)blockIdx.x * px.pt + threadIdx.x;
+    px.nt = (int64_t)gridDim.x * px.pt;
+    px.steps = (px.n >> 2) > px.t0 ? (int)(((px.n >> 2) - 1 - px.t0) / px.nt) + 1 : 0;
+    px.resident = min(ra.resident, px.steps);
+    px.vec_x = ((uintptr_t)px.x & 15) == 0;
+    px.vec_u = px.vec_x && (px.n & 3) == 0 && ((uintptr_t)ra.U & 15) == 0 && (!ra.from_u || ((uintptr_t)ra.U0 & 15) == 0);
+    return px;
+}
+
 template <int C>
 struct RunShared {
     float red[RUN_MAX_PW][2 * C];  // warp totals of a sums pass; J in red[w][0] of a full pass
@@ -369,7 +387,7 @@ struct RunShared {
     // while slower warps still read this one's (no barrier is between them).
     // x: a wait gave up; y: a sampled change reached eps; z: the exchange words do not
     // hold the sums, or (of an exchange through the slots) would not; w: some cluster
-    // is empty.
+    // is empty, or a center moved by more than REBASE times its new value.
     int4 ctl[2];
     uint64_t seen[2][C][2];    // the words of each cluster after their last exchange, of even and odd parity
     uint64_t seen_ctl[2];      // and the control word
@@ -459,8 +477,66 @@ __device__ __forceinline__ void sums_pass(const Px& px, RunShared<C>& sh, f2* se
     sums_pass_body<C, MK, false>(px, sh, second, cur, m, inv_m1, [](float) {});
 }
 
+// The sums of a sums pass once more, with the numerators centered on sh.v[basis]:
+// for a center that moved by far more than it is now away from 0 (an initial
+// center far outside the image, a center between two parts that are far apart),
+// whose differences x - v^k have lost the bits of x. Called, not inlined, so that
+// the usual passes keep their registers.
+template <int C, int MK>
+__device__ __noinline__ void rebased_pass(const RunArgs& ra, RunShared<C>& sh, f2* second, int cur, int basis) {
+    constexpr int P = pow2_at_least(2 * C);
+    const Px px = run_px<C>(ra, second);
+    const float m = ra.m, inv_m1 = ra.inv_m1;
+    SumAcc<C> a;
+    a.reset();
+    PackedCenters<C, MK> cen;
+    cen.set(sh.v[cur]);
+    f2* const set = second + threadIdx.x;
+    int held = 0;
+    bool folded = false;
+    auto pair = [&](f2 x) {
+        f2 um[1][C], d2[1][C], J2[1];
+        const f2 xq[1] = {x};
+        packed_pairs<C, MK, true, 1>(xq, cen, m, inv_m1, um, d2, J2);
+#pragma unroll
+        for (int j = 0; j < C; ++j) d2[0][j] = sub2(x, pack2(sh.v[basis][j], sh.v[basis][j]));
+        a.add(d2[0], um[0]);
+    };
+    px.quads([&](const float4& c, int64_t) {
+        pair(pack2(c.x, c.y));
+        pair(pack2(c.z, c.w));
+        if (++held == FOLD) {
+            a.fold(set, px.pt, !folded);
+            folded = true;
+            held = 0;
+        }
+    });
+    px.tail([&](int64_t i) {
+        const float xi = __ldg(px.x + i);
+        const PixelPair<C> w = scalar_pair<C, MK, true>(xi, xi, cen.vs, m, inv_m1);
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            const f2 um = pack2(w.a[j], 0.0f);
+            a.num2[j] = fma2(um, pack2(xi - sh.v[basis][j], 0.0f), a.num2[j]);
+            a.den2[j] = add2(a.den2[j], um);
+        }
+    });
+    a.finish(set, px.pt, folded);
+    float t[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        const f2 q = i < C ? a.num2[i < C ? i : 0] : a.den2[(i >= C && i < 2 * C) ? i - C : 0];
+        t[i] = i < 2 * C ? lo2(q) + hi2(q) : 0.0f;
+    }
+    warp_sums<C>(sh, t);
+}
+
 // What an exchange adds up over the blocks.
 enum Exchange : int { X_SUMS0 = 0, X_SUMS = 1, X_J = 2 };  // sums of pass 0 from U^0; centered sums; J
+
+// The FP32 differences x - v_j^k round by 2^-24 of the step at most, so up to this
+// factor the new center keeps about 18 bits; beyond it, the pass is taken again.
+constexpr float REBASE = 64.0f;
 
 template <int C, int MK>
 __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
@@ -479,17 +555,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     const float* U0 = ra.U0;  // may be U itself: each pixel is read, then written, by one thread
     float* U = ra.U;
     const int64_t n = ra.n;
-    Px px;
-    px.x = ra.x;
-    px.xs = reinterpret_cast<float4*>(second + 2 * C * 32 * pw) + threadIdx.x;
-    px.n = n;
-    px.pt = 32 * pw;
-    px.t0 = (int64_t)blockIdx.x * px.pt + threadIdx.x;
-    px.nt = (int64_t)nb * px.pt;
-    px.steps = (n >> 2) > px.t0 ? (int)(((n >> 2) - 1 - px.t0) / px.nt) + 1 : 0;
-    px.resident = min(ra.resident, px.steps);
-    px.vec_x = ((uintptr_t)px.x & 15) == 0;
-    px.vec_u = px.vec_x && (n & 3) == 0 && ((uintptr_t)U & 15) == 0 && (!from_u || ((uintptr_t)U0 & 15) == 0);
+    const Px px = run_px<C>(ra, second);
     const float m = ra.m, inv_m1 = ra.inv_m1, eps = ra.eps;
     const int max_iter = ra.max_iter;
     const bool tracing = ra.trace != nullptr;
@@ -554,9 +620,11 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     auto new_center = [&](int q, DF na, DF da, bool centered, int cur, int nxt) {
         if (da.hi > 0.0f) {
             DF r = (da.hi > 1e-30f && da.hi < 1e30f) ? df_div_fast(na, da) : df_div(na, da);
+            const float step = fabsf(r.hi);
             if (centered) r = df_merge(r, DF{sh.v[cur][q], 0.0f});
             sh.v[nxt][q] = r.hi;
             sh.v64[nxt][q] = r;
+            if (centered && step > REBASE * fabsf(r.hi)) sh.ctl[it].w = 1;
         } else {
             // an empty cluster keeps its center (in pass 0 that is V^0, or 0 from a U^0)
             sh.v[nxt][q] = centered ? sh.v[cur][q] : 0.0f;
@@ -664,6 +732,21 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         sh.seen_ctl[k & 1] = va;
         if (!ok) sh.ctl[it].x = 1;
     };
+    // V^{k+1} in slot nxt again, with sums centered on what it holds, if a center moved
+    // far. False when a wait gave up.
+    auto rebase = [&](int cur, int nxt) {
+        bool far = false;
+#pragma unroll
+        for (int j = 0; j < C; ++j) far |= fabsf(sh.v[nxt][j] - sh.v[cur][j]) > REBASE * fabsf(sh.v[nxt][j]);
+        if (!far) return true;
+        __syncthreads();
+        if (!control) rebased_pass<C, MK>(ra, sh, second, cur, nxt);
+        __syncthreads();
+        if (warp < C) exchange_sums(std::integral_constant<int, X_SUMS>(), warp, nxt, nxt);
+        ++nx;
+        __syncthreads();
+        return sh.ctl[it].x == 0;
+    };
     // ---- pass 0: V^1 from U^0, or from U^0 = f(x, V^0) ----
     bool ok;
     {
@@ -758,6 +841,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         ++nx;
         __syncthreads();
         ok = sh.ctl[0].x == 0;
+        if (ok && !from_u && !(sh.flags & 1u)) ok = rebase(0, 1);
     }
     // The fixed-point units: |num_j| <= 2 n max(|x|, |V^0|) < 2^NUM_BITS units and
     // den_j <= n. Images whose FP32 sums could overflow never use the words.
@@ -1001,7 +1085,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         // nothing but the next iteration to do: one test, every warp waits for it
         const bool plain = words && !last && !tracing && !empty && (ctl.x | ctl.z | ctl.w) == 0 && (k == 1 || ctl.y);
         if (plain) continue;
-        empty = ctl.w != 0;  // behind V^{k+1}
+        empty = ctl.w != 0;  // perhaps, behind V^{k+1}
         if (ctl.x) {
             ok = give_up(k);
             break;
@@ -1019,6 +1103,10 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
             }
         } else if (!last && !words) {
             words = fixed && !ctl.z;
+        }
+        if (!last && !rebase(cur, nxt)) {
+            ok = give_up(k);
+            break;
         }
         // Iteration k - 1's full pass when its sample could not decide, iteration
         // k's when it is the last (and every one for a trace).

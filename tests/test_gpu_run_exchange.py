@@ -120,6 +120,31 @@ def test_tissues_beside_a_sentinel(fcm, value, share, m):
     _check_centers(fcm, x, 3, m, [20.0, 80.0, value], eps=0.0, max_iter=9)
 
 
+@pytest.mark.parametrize("m", [2.0, 1.5, 2.5])
+def test_a_far_initial_center(fcm, m):
+    """Differences from a center far outside the image have lost the bits of the
+    pixels; the center that is formed from them has not."""
+    x, _ = _tissues(200004, 4)
+    for k in (1, 2, 12):
+        _check_centers(fcm, x, 3, m, [20.0, 80.0, 1e6], eps=0.0, max_iter=k)
+        if m == 2.0:
+            _check_centers(fcm, x, 3, m, [20.0, 80.0, 1e10], eps=0.0, max_iter=k)
+
+
+@pytest.mark.parametrize("n", [4001, 200004])
+def test_a_center_that_leaves_a_sentinel(fcm, n):
+    """A start that mixes tissue and a sentinel puts a center between them; it
+    falls back to the tissue within two iterations, by 10^4 times its value."""
+    x, rng = _tissues(n, 7)
+    far = rng.random(n) < 0.3
+    x[far] = 1e8
+    u0 = np.where(far, np.array([[0.2], [0.8]]), np.array([[0.9], [0.1]])).astype(np.float32)
+    for k in (1, 2, 3, 4, 8):
+        g = fcm.run(_cuda(x), 2, 2.0, 0.0, k, U0=_cuda(u0))
+        o = oracle.fcm(x, 2, 2.0, 0.0, k, U0=u0)
+        assert_within(precision_report(g.U.cpu().numpy(), g.V.cpu().numpy(), g.iters, o["U"], o["V"], o["iters"]))
+
+
 @pytest.mark.parametrize("scale", [1e-30, 1e-20, 1e-12])
 def test_tiny_intensities(fcm, scale):
     """All totals far below the largest unit."""
