@@ -270,7 +270,7 @@ __device__ __noinline__ void solve_run(const BinArgs& a, int r, const BinRun& ru
             PackedCenters<C, MK> cen;
             bin_centers<C, MK>(sc, v, cen);
             f2 u1[C], um1[C], dd[C], J2;
-            bin_memberships<C, MK>(b2, cen, m, inv_m1, u1, um1, dd, J2);
+            bin_memberships<C, MK>(b2, cen, v, m, inv_m1, u1, um1, dd, J2);
             const int2 rp = *reinterpret_cast<const int2*>(a.rep + (int64_t)s * 256 + 2 * t);
             float lb = 0.0f;
 #pragma unroll

@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(BIN_NT) k_hist_solve(HistState* st, const doub
             PackedCenters<C, MK> cen;
             bin_centers<C, MK>(sc, v, cen);
             f2 u1[C], um1[C], dd[C], J2;
-            bin_memberships<C, MK>(b2, cen, m, inv_m1, u1, um1, dd, J2);
+            bin_memberships<C, MK>(b2, cen, v, m, inv_m1, u1, um1, dd, J2);
             const int r0 = st->rep[2 * t] - 1, r1 = st->rep[2 * t + 1] - 1;
             float lb = 0.0f;
 #pragma unroll

@@ -91,13 +91,13 @@ __device__ __forceinline__ void bin_centers(BinScratch& sc, const float (&v)[C],
 }
 
 // The CTA's sums of num and den (per thread, both grey levels) and its maximum;
-// then the centers. base: the centers that the numerators are relative to. mine:
+// then the centers. base: what the numerators are relative to (bin_base). mine:
 // the double-float center of cluster lane >> 2, kept where that cluster is empty.
 // On return v and mine hold the new centers, mx the maximum, and the result tells
 // whether some cluster was empty. All BIN_NT threads must call it.
 template <int C>
 __device__ __forceinline__ bool bin_reduce(BinScratch& sc, int& par, const f2 (&num2)[C], const f2 (&den2)[C],
-                                           float back, float& mx, const float (&base)[C], float (&v)[C], DF& mine) {
+                                           float& mx, const float (&base)[C], float (&v)[C], DF& mine) {
     constexpr int P = bin_pow2(2 * C);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float t[P];
@@ -105,7 +105,6 @@ __device__ __forceinline__ bool bin_reduce(BinScratch& sc, int& par, const f2 (&
     for (int i = 0; i < P; ++i) {
         const f2 q = i < C ? num2[i < C ? i : 0] : den2[(i >= C && i < 2 * C) ? i - C : 0];
         t[i] = i < 2 * C ? lo2(q) + hi2(q) : 0.0f;
-        if (i < C) t[i] *= back;
     }
     const int slot = bin_warp_totals<P>(t);
     const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));  // non-negative
@@ -158,11 +157,16 @@ __device__ __forceinline__ float bin_max(BinScratch& sc, int& par, float mx) {
     return mx;
 }
 
+// What cluster j's numerator is centered on: its center, or the end of the grey
+// scale that is nearest to it. Differences from a center far outside the scale (an
+// initial one) would have lost the bits of the grey levels.
+__device__ __forceinline__ float bin_base(float v) { return fminf(fmaxf(v, 0.0f), 255.0f); }
+
 // u of this thread's grey levels b2 = (2t, 2t + 1), the J terms, and u^m with
-// the (scaled) differences.
+// the differences from the bases.
 template <int C, int MK>
-__device__ __forceinline__ void bin_memberships(f2 b2, const PackedCenters<C, MK>& cen, float m, float inv_m1,
-                                                f2 (&u2)[C], f2 (&um2)[C], f2 (&d2)[C], f2& J2) {
+__device__ __forceinline__ void bin_memberships(f2 b2, const PackedCenters<C, MK>& cen, const float (&base)[C], float m,
+                                                float inv_m1, f2 (&u2)[C], f2 (&um2)[C], f2 (&d2)[C], f2& J2) {
     f2 w[1][C], d[1][C], j[1];
     const f2 x[1] = {b2};
     packed_pairs<C, MK, false, 1, true>(x, cen, m, inv_m1, w, d, j);
@@ -170,7 +174,7 @@ __device__ __forceinline__ void bin_memberships(f2 b2, const PackedCenters<C, MK
 #pragma unroll
     for (int q = 0; q < C; ++q) {
         u2[q] = w[0][q];
-        d2[q] = d[0][q];
+        d2[q] = sub2(b2, pack2(base[q], base[q]));
         um2[q] = (MK == M_TWO)     ? mul2(u2[q], u2[q])
                  : (MK == M_THREE) ? mul2(mul2(u2[q], u2[q]), u2[q])
                                    : pack2(pow_m<MK>(lo2(u2[q]), m), pow_m<MK>(hi2(u2[q]), m));
@@ -185,17 +189,19 @@ __device__ __forceinline__ bool bin_first_centers(BinScratch& sc, int& par, f2 c
     const f2 b2 = pack2((float)(2 * threadIdx.x), (float)(2 * threadIdx.x + 1));
     PackedCenters<C, MK> cen;
     bin_centers<C, MK>(sc, v0, cen);
+    float base[C];
+#pragma unroll
+    for (int j = 0; j < C; ++j) base[j] = bin_base(v0[j]);
     f2 um2[C], d2[C], J2, num2[C];
-    bin_memberships<C, MK>(b2, cen, m, inv_m1, up2, um2, d2, J2);
+    bin_memberships<C, MK>(b2, cen, base, m, inv_m1, up2, um2, d2, J2);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
         um2[j] = mul2(cnt2, um2[j]);
         num2[j] = mul2(um2[j], d2[j]);
     }
     float mx = 0.0f;
-    const float back = PackedCenters<C, MK>::SCALED ? rcp_approx(lo2(cen.scale)) : 1.0f;
     mine = bin_mine<C>(v0);
-    return bin_reduce<C>(sc, par, num2, um2, back, mx, v0, v, mine);
+    return bin_reduce<C>(sc, par, num2, um2, mx, base, v, mine);
 }
 
 // Iterations k = 1, 2, ... of Algorithm 1 on the bins of one run, in one CTA.
@@ -220,8 +226,11 @@ __device__ __forceinline__ void solve_bins(BinScratch& sc, int& par, f2 cnt2, bo
     for (k = 1;; ++k) {
         PackedCenters<C, MK> cen;
         bin_centers<C, MK>(sc, v, cen);
+        float base[C];
+#pragma unroll
+        for (int j = 0; j < C; ++j) base[j] = bin_base(v[j]);
         f2 u2[C], um2[C], d2[C], num2[C];
-        bin_memberships<C, MK>(b2, cen, m, inv_m1, u2, um2, d2, J2);
+        bin_memberships<C, MK>(b2, cen, base, m, inv_m1, u2, um2, d2, J2);
         float ma = 0.0f, mb = 0.0f;
 #pragma unroll
         for (int j = 0; j < C; ++j) {
@@ -234,10 +243,9 @@ __device__ __forceinline__ void solve_bins(BinScratch& sc, int& par, f2 cnt2, bo
             num2[j] = mul2(um2[j], d2[j]);
         }
         float mx = fmaxf(in0 ? ma : 0.0f, in1 ? mb : 0.0f);
-        const float back = PackedCenters<C, MK>::SCALED ? rcp_approx(lo2(cen.scale)) : 1.0f;
         float vn[C];
         DF next = mine;
-        const bool empty = bin_reduce<C>(sc, par, num2, um2, back, mx, v, vn, next);
+        const bool empty = bin_reduce<C>(sc, par, num2, um2, mx, base, vn, next);
         delta = (from_u && k == 1) ? d1 : mx;
         if (delta < eps) {
             status = FCM_OK;

@@ -1,0 +1,68 @@
+"""Starts whose centers lie far from the image, or between parts of it that are
+far apart (needs a GPU): a center then moves by many times its new value in one
+iteration. Against the FP64 oracle at the same iteration."""
+import numpy as np
+import pytest
+
+import oracle
+from parity import assert_within, center_err, precision_report
+
+pytestmark = pytest.mark.gpu
+
+STEPS = (1, 2, 12)
+
+
+@pytest.fixture(scope="module")
+def fcm():
+    from paper_1601_00072_gb300 import _build
+    _build.build()
+    from paper_1601_00072_gb300.fcm import FCM
+    h = FCM(0)
+    yield h
+    h.close()
+
+
+def _cuda(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+
+
+def tissues(n, seed, grey=False):
+    rng = np.random.default_rng(seed)
+    x = np.where(rng.random(n) < 0.5, 30.0, 90.0) + 6.0 * rng.standard_normal(n)
+    x = np.clip(np.rint(x), 0, 255) if grey else x
+    return x.astype(np.float32).astype(np.float64), rng
+
+
+def mixed_start(n, seed):
+    """Tissue beside a sentinel of 1e8, and memberships that mix them."""
+    x, rng = tissues(n, seed)
+    far = rng.random(n) < 0.3
+    x[far] = 1e8
+    return x, np.where(far, np.array([[0.2], [0.8]]), np.array([[0.9], [0.1]])).astype(np.float32)
+
+
+def check(g, o):
+    assert_within(precision_report(g.U.cpu().numpy(), g.V.cpu().numpy(), g.iters, o["U"], o["V"], o["iters"]))
+
+
+@pytest.mark.parametrize("m", [2.0, 1.5, 2.5])
+@pytest.mark.parametrize("far", [1e6, -300.0])
+def test_histogram_run(fcm, far, m):
+    x, _ = tissues(40001, 1, grey=True)
+    V0 = np.array([20.0, 80.0, far])
+    for k in STEPS:
+        g = fcm.run_hist(_cuda(x), 3, m, 0.0, k, V0=_cuda(V0))
+        check(g, oracle.fcm(x, 3, m, 0.0, k, V0=V0))
+
+
+@pytest.mark.parametrize("far", [1e6, -300.0])
+def test_batched_histogram_run(fcm, far):
+    from paper_1601_00072_gb300.fcm import Slice
+    V0 = [20.0, 80.0, far]
+    for k in STEPS:
+        xs = [tissues(n, n, grey=True)[0] for n in (4001, 40000)]
+        sl = [Slice(x=_cuda(x), C=3, m=2.0, eps=0.0, max_iter=k, V0=V0) for x in xs]
+        fcm.run_batched_hist(sl)
+        for s, x in zip(sl, xs):
+            check(s, oracle.fcm(x, 3, 2.0, 0.0, k, V0=np.array(V0)))
