@@ -93,6 +93,7 @@ struct BatchShared {
     float delta;
     unsigned flags;                   // bit 0: bad input
     unsigned empty;                   // some cluster of the latest sums pass was empty
+    unsigned far;                     // some center moved by more than REBASE times its new value
     int idx;
     int team_err;             // a team barrier gave up
     int item[3];              // team schedule: slice, seat, team size
@@ -189,7 +190,12 @@ __device__ __forceinline__ DF lanes_sum(DF d, int n) {
 // What one pass leaves: X_SUMS0 the sums of pass 0 from U^0, X_SUMS centered sums
 // (V^{k+1} into sh.v[nxt]), X_FULL J and the exact maximum. All with the maximum
 // (sh.delta) and the flags.
-enum Exchange : int { X_SUMS0 = 0, X_SUMS = 1, X_FULL = 2 };
+// X_REBASED: sums centered on what slot nxt holds already.
+enum Exchange : int { X_SUMS0 = 0, X_SUMS = 1, X_FULL = 2, X_REBASED = 3 };
+// The FP32 differences x - v_j^k round by 2^-24 of the step at most, so up to this
+// factor the new center keeps about 18 bits; beyond it, the sums are taken again
+// (rebased_sums), as in the whole-run kernel of a single image.
+constexpr float REBASE = 64.0f;
 
 // Totals of one pass over the slice: warp totals (already in sh.w, sh.mx, sh.bad),
 // the CTA's, then (K > 1) the K CTAs' through distributed shared memory or, in a
@@ -207,13 +213,17 @@ static __device__ __noinline__ void slice_reduce(BatchShared& sh, int C, int X, 
     auto center = [&](int q, DF num, DF den) {
         if (den.hi > 0.0f) {
             DF v = df_div(num, den);
-            if (X == X_SUMS) v = df_merge(v, DF{sh.v[cur][q], 0.0f});
+            const float step = fabsf(v.hi);
+            if (X == X_SUMS || X == X_REBASED) v = df_merge(v, DF{sh.v[X == X_SUMS ? cur : nxt][q], 0.0f});
+            if (X == X_SUMS && step > REBASE * fabsf(v.hi)) sh.far = 1u;
             sh.v[nxt][q] = v.hi;
             sh.v64[nxt][q] = v;
         } else {
             // an empty cluster keeps its center (in pass 0 that is V^0, or 0 from a U^0)
-            sh.v[nxt][q] = X == X_SUMS ? sh.v[cur][q] : 0.0f;
-            sh.v64[nxt][q] = X == X_SUMS ? sh.v64[cur][q] : DF{0.0f, 0.0f};
+            if (X != X_REBASED) {
+                sh.v[nxt][q] = X == X_SUMS ? sh.v[cur][q] : 0.0f;
+                sh.v64[nxt][q] = X == X_SUMS ? sh.v64[cur][q] : DF{0.0f, 0.0f};
+            }
             sh.empty = 1u;
         }
     };
@@ -330,6 +340,36 @@ struct XSrc {
     }
 };
 
+// The warps' totals of a sums pass from V^k in slot cur, with the numerators centered
+// on slot nxt, into sh.w: for a center that moved by far more than it is now away
+// from 0, whose differences x - v^k have lost the bits of x. Rare: one function
+// for every cluster count and fuzzifier, in the scalar form.
+static __device__ __noinline__ void rebased_sums(BatchShared& sh, const XSrc& xl, int cnt, int C, int mk, float m,
+                                                 float inv_m1, int cur, int nxt) {
+    constexpr int N = FCM_MAX_CLUSTERS;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    DF t[2 * N];
+#pragma unroll
+    for (int i = 0; i < 2 * N; ++i) t[i] = DF{0.0f, 0.0f};
+    for (int i = threadIdx.x; i < cnt; i += NTB) {
+        const float xi = xl.at(i);
+        const PixelPair<N> w = scalar_pair_any(xi, xi, sh.v[cur], C, mk, true, m, inv_m1);
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            if (j >= C) break;
+            df_add(t[j], w.a[j] * (xi - sh.v[nxt][j]));
+            df_add(t[N + j], w.a[j]);
+        }
+    }
+    warp_totals_df<2 * N>(t);
+    // the lane's value: bit i of its number from the top is bit 4 - i of the lane
+    int s = 0;
+#pragma unroll
+    for (int w = 2 * N, o = 16; w > 1; w >>= 1, o >>= 1) s += (lane & o) ? w / 2 : 0;
+    const int j = s % N;
+    if ((lane & 1) == 0 && j < C) sh.w[warp][s < N ? j : C + j] = t[0];
+}
+
 template <int C, int MK>
 __device__ __noinline__ void process_slice(const SliceDesc& d, SliceResult& res, unsigned r, unsigned K, float* xs,
                                            BatchShared& sh, bool resume, int cap, const TeamCtx& tc) {
@@ -349,7 +389,7 @@ __device__ __noinline__ void process_slice(const SliceDesc& d, SliceResult& res,
     }
     if (threadIdx.x == 0) {
         sh.team_err = 0;
-        sh.empty = 0u;
+        sh.empty = sh.far = 0u;
     }
     XSrc xl{d.x + lo, reinterpret_cast<const uint8_t*>(xs), false};
     if (cnt <= XCAP) {
@@ -444,6 +484,14 @@ __device__ __noinline__ void process_slice(const SliceDesc& d, SliceResult& res,
         if (check && threadIdx.x < C) bad |= !finite_f(sh.v[cur][threadIdx.x]);
         warp_publish<C>(sh, a, dmax, bad);
         reduce(X_SUMS);
+        if (sh.far && !sh.team_err) {
+            // the same in every CTA that shares the slice; the maximum and the flags
+            // are still in sh.mx and sh.bad
+            __syncthreads();
+            if (threadIdx.x == 0) sh.far = 0u;
+            rebased_sums(sh, xl, cnt, C, MK, m, inv_m1, cur, nxt);
+            reduce(X_REBASED);
+        }
     };
     // U^k of a pair and its largest |U^k - U^{k-1}|; U^{k-1} is given (u0) or
     // comes from V^{k-1}. J2: the pair's J terms.

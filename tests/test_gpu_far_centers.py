@@ -66,3 +66,32 @@ def test_batched_histogram_run(fcm, far):
         fcm.run_batched_hist(sl)
         for s, x in zip(sl, xs):
             check(s, oracle.fcm(x, 3, 2.0, 0.0, k, V0=np.array(V0)))
+
+
+PLANS = {"queue": dict(block=256), "clusters": dict(block=512, cluster=4, big=2000),
+         "teams": dict(schedule="teams", block=256, tile=10)}
+
+
+@pytest.mark.parametrize("plan", PLANS.values(), ids=PLANS)
+def test_batch(fcm, plan):
+    """A far initial center, and a start that mixes tissue and a sentinel, in
+    one CTA, in a cluster and in a team."""
+    from paper_1601_00072_gb300.fcm import Slice
+    fcm.set_batched_plan(**plan)
+    try:
+        for k in STEPS + (3, 4):
+            sl, want = [], []
+            for n in (37, 4001, 40000):
+                x, _ = tissues(n, n)
+                for m, far in ((2.0, 1e10), (2.0, -1e6), (1.5, 1e6), (2.5, 1e6)):
+                    V0 = [20.0, 80.0, far]
+                    sl.append(Slice(x=_cuda(x), C=3, m=m, eps=0.0, max_iter=k, V0=V0))
+                    want.append(oracle.fcm(x, 3, m, 0.0, k, V0=np.array(V0)))
+                x, u0 = mixed_start(n, n)
+                sl.append(Slice(x=_cuda(x), C=2, m=2.0, eps=0.0, max_iter=k, U0=_cuda(u0)))
+                want.append(oracle.fcm(x, 2, 2.0, 0.0, k, U0=u0))
+            fcm.run_batched(sl)
+            for s, o in zip(sl, want):
+                check(s, o)
+    finally:
+        fcm.set_batched_plan()
