@@ -36,6 +36,10 @@ constexpr int MNT = MULTI_NT;
 constexpr int MNW = MNT / 32;
 constexpr int MFOLD = 8;         // pairs added in registers before they go to the second set of sums
 constexpr int MSAMPLE_WARPS = 2; // warps per block that sample delta_k
+// The FP32 differences x - v_j^k round by 2^-24 of the step at most, so up to this
+// factor (of the largest channel of the new center) the center keeps about 18 bits;
+// beyond it, the sums are taken again, centered on the new one.
+constexpr float REBASE = 64.0f;
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
     unsigned v;
@@ -194,6 +198,33 @@ __device__ __forceinline__ int warp_totals8(float (&a)[8]) {
     return slot;
 }
 
+// A warp's sums from the centers `cur`, centered on `base`, into w[0..C D + C).
+// Called, not inlined: rare, and the usual passes keep their registers.
+template <int C, int MK>
+__device__ __noinline__ void rebased_sums(const float* x, int64_t n, int64_t t0, int64_t nt, const float* cur,
+                                          const float* base, float m, float inv_m1, DF* w) {
+    for (int j = 0; j < C; ++j) {
+        DF acc[D + 1];
+#pragma unroll
+        for (int d = 0; d <= D; ++d) acc[d] = DF{0.0f, 0.0f};
+        for (int64_t i = t0; i < n; i += nt) {
+            float xv[D], u[C];
+#pragma unroll
+            for (int d = 0; d < D; ++d) xv[d] = __ldg(x + (int64_t)d * n + i);
+            pixel_memberships<C, MK>(xv, cur, m, inv_m1, u);
+            const float um = (MK == M_TWO) ? u[j] * u[j] : ex2_approx(m * lg2_approx(u[j]));
+            df_add(acc[D], um);
+#pragma unroll
+            for (int d = 0; d < D; ++d) df_add(acc[d], um * (xv[d] - base[j * D + d]));
+        }
+#pragma unroll
+        for (int d = 0; d <= D; ++d) {
+            const DF t = warp_sum_df(acc[d]);
+            if ((threadIdx.x & 31) == 0) w[d < D ? j * D + d : C * D + j] = t;
+        }
+    }
+}
+
 // Pass 0 is INIT (V^1 from U^0, or from U^0 = f(x, V^0)).
 template <int C, int MK, bool FROM_U>
 __global__ void __launch_bounds__(MNT, 1) k_fcm_run_multi(MultiState* __restrict__ st, float* __restrict__ partials) {
@@ -209,7 +240,7 @@ __global__ void __launch_bounds__(MNT, 1) k_fcm_run_multi(MultiState* __restrict
     __shared__ DF s_df[NV];
     __shared__ float s_mx[2];
     __shared__ float s_wit[MNW][D];               // each warp's pixel of largest change in a full pass
-    __shared__ int s_err, s_empty;
+    __shared__ int s_err, s_empty, s_far;
 
     const float* __restrict__ x = st->x;
     const float* U0 = st->U0;  // may be U itself: each pixel is read, then written, by one thread
@@ -223,7 +254,7 @@ __global__ void __launch_bounds__(MNT, 1) k_fcm_run_multi(MultiState* __restrict
         s_v[0][t] = st->V0[t];
         s_v64[0][t] = DF{st->V0[t], 0.0f};
     }
-    if (threadIdx.x == 0) s_err = s_empty = 0;
+    if (threadIdx.x == 0) s_err = s_empty = s_far = 0;
     int flags = 0, parity = 0;
     unsigned arrived = 0;
     __syncthreads();
@@ -314,7 +345,8 @@ __global__ void __launch_bounds__(MNT, 1) k_fcm_run_multi(MultiState* __restrict
         return true;
     };
     // V^{k+1} into slot nxt from the sums; cur: the slot the numerators are centered
-    // on, or -1. An empty cluster keeps its center (pass 0: V^0, or 0 from a U^0).
+    // on (nxt itself for rebased sums), or -1. An empty cluster keeps its center
+    // (pass 0: V^0, or 0 from a U^0).
     auto centers = [&](int cur, int nxt) {
         if (threadIdx.x < C * D) {
             const int t = threadIdx.x, j = t / D;
@@ -322,7 +354,11 @@ __global__ void __launch_bounds__(MNT, 1) k_fcm_run_multi(MultiState* __restrict
             DF v = cur >= 0 ? s_v64[cur][t] : DF{0.0f, 0.0f};
             if (den.hi > 0.0f) {
                 v = df_div(s_df[t], den);
-                if (cur >= 0) v = df_merge(v, DF{s_v[cur][t], 0.0f});
+                if (cur >= 0) {
+                    const float step = fabsf(v.hi);
+                    v = df_merge(v, DF{s_v[cur][t], 0.0f});
+                    if (step > REBASE * fabsf(v.hi)) s_far = 1;
+                }
             } else {
                 s_empty = 1;
             }
@@ -330,6 +366,29 @@ __global__ void __launch_bounds__(MNT, 1) k_fcm_run_multi(MultiState* __restrict
             s_v64[nxt][t] = v;
         }
         __syncthreads();
+    };
+    // s_far says that some channel of a center moved far: whether one moved by more
+    // than its largest channel is worth, and then V^{k+1} again from sums centered on
+    // slot nxt (the scalar form: rare). False when the barrier gave up.
+    auto rebase = [&](int cur, int nxt) {
+        bool far = false;
+        for (int j = 0; j < C; ++j) {
+            float step = 0.0f, size = 0.0f;
+            for (int d = 0; d < D; ++d) {
+                step = fmaxf(step, fabsf(s_v[nxt][j * D + d] - s_v[cur][j * D + d]));
+                size = fmaxf(size, fabsf(s_v[nxt][j * D + d]));
+            }
+            far |= step > REBASE * size;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) s_far = 0;
+        if (!far) return true;
+        rebased_sums<C, MK>(x, n, t0, nt, s_v[cur], s_v[nxt], m, inv_m1, s_w[warp]);
+        if (!exchange(NV)) return false;
+        centers(nxt, nxt);
+        __syncthreads();
+        if (threadIdx.x == 0) s_far = 0;
+        return true;
     };
     auto publish = [&](float (&a)[NP], float mx, bool bad) {
 #pragma unroll
@@ -471,6 +530,10 @@ __global__ void __launch_bounds__(MNT, 1) k_fcm_run_multi(MultiState* __restrict
         ok = false;
     } else {
         centers(FROM_U ? -1 : 0, 1);
+        if (!FROM_U && s_far && !rebase(0, 1)) {
+            status = FCM_ERR_TIMEOUT;
+            ok = false;
+        }
     }
     auto advance = [&] {
         if (s_empty) flags |= FCM_FLAG_EMPTY_CLUSTER;
@@ -516,6 +579,19 @@ __global__ void __launch_bounds__(MNT, 1) k_fcm_run_multi(MultiState* __restrict
             }
             const bool go_on = s_mx[0] >= eps;
             centers(cur, nxt);
+            if (go_on && !(s_far | s_empty)) {
+                // as advance(), with no flag to note or clear
+                const int t = prv;
+                prv = cur;
+                cur = nxt;
+                nxt = t;
+                continue;
+            }
+            if (s_far && !rebase(cur, nxt)) {
+                status = FCM_ERR_TIMEOUT;
+                iters = k;
+                break;
+            }
             if (go_on) {
                 advance();
                 continue;

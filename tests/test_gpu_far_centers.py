@@ -95,3 +95,22 @@ def test_batch(fcm, plan):
                 check(s, o)
     finally:
         fcm.set_batched_plan()
+
+
+@pytest.mark.parametrize("m", [2.0, 2.5])
+@pytest.mark.parametrize("D", [1, 3])
+@pytest.mark.parametrize("n", [37, 40001])
+def test_multi_feature_run(fcm, n, D, m):
+    """Far in one channel and in all, and a start that mixes tissue and a sentinel."""
+    xs = np.stack([tissues(n, 10 + d)[0] for d in range(D)])
+    for k in STEPS:
+        for far in (np.full(D, 1e6), np.r_[1e6, np.full(D - 1, 50.0)]):
+            V0 = np.stack([np.full(D, 20.0), np.full(D, 80.0), far])
+            g = fcm.run_multi(_cuda(xs), 3, m, 0.0, k, V0=_cuda(V0))
+            check(g, oracle.fcm_multi(xs, 3, m, 0.0, k, V0=V0))
+    x, u0 = mixed_start(n, 5)
+    xs[0] = x
+    for k in (1, 2, 3, 4):
+        g = fcm.run_multi(_cuda(xs), 2, m, 0.0, k, U0=_cuda(u0))
+        o = oracle.fcm_multi(xs, 2, m, 0.0, k, U0=u0)
+        assert center_err(g.V.cpu().numpy(), o["V"]) <= 1e-5
