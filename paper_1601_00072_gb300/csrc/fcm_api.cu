@@ -28,6 +28,7 @@
 #include <tuple>
 
 #include "fcm.h"
+#include "fcm_bounds.cuh"
 #include "fcm_device.cuh"
 #include "fcm_internal.h"
 #include "fcm_run.h"
@@ -120,6 +121,12 @@ RunShape run_shape(int64_t n, int C, int64_t max_blocks) {
     const int64_t blocks = std::max<int64_t>(1, (quads + steps * pt - 1) / (steps * pt));
     const int resident = (int)std::min<int64_t>((quads + blocks * pt - 1) / (blocks * pt), run_max_resident(C, (int)pt));
     return RunShape{(int)blocks, (int)pt + 32, resident, run_smem(C, (int)pt, resident)};
+}
+
+int64_t run_guard_n(int64_t n) {
+    if (kBoundsChecks)
+        if (const char* e = std::getenv("FCM_DEBUG_BOUNDS_SHORT")) return n - std::max(0ll, std::atoll(e));
+    return n;
 }
 
 int ctx_fail(fcm_ctx* h, cudaError_t e, const char* what) {
@@ -567,6 +574,8 @@ int fcm_run(fcm_handle h, const float* x, int64_t n, int C, float m, float eps, 
         ra.max_iter = max_iter;
         ra.from_u = init_mode == FCM_INIT_U;
         ra.resident = shape.resident;
+        ra.max_blocks = max_run_sms(h);
+        ra.guard_n = run_guard_n(n);
         ra.lim = h->limits;
         std::memcpy(ra.V0, hs->V0, sizeof(ra.V0));
         void* args[1] = {&ra};
@@ -727,6 +736,8 @@ int fcm_run_stream(fcm_handle h, int n_images, const float* const* x, int64_t n,
         ra.max_iter = max_iter;
         ra.from_u = 1;
         ra.resident = shape.resident;
+        ra.max_blocks = max_run_sms(h);
+        ra.guard_n = run_guard_n(n);
         ra.lim = h->limits;
         void* args[1] = {&ra};
         if (e == cudaSuccess)

@@ -144,6 +144,8 @@ extern "C" int fcm_run_noalloc(const float* x, int64_t n, int C, float m, float 
     ra.max_iter = max_iter;
     ra.from_u = init_mode == FCM_INIT_U;
     ra.resident = shape.resident;
+    ra.max_blocks = std::min<int>(FCM_NOALLOC_MAX_BLOCKS, RUN_MAX_BLOCKS);
+    ra.guard_n = run_guard_n(n);
     ra.lim = WaitLimits{DEFAULT_GRID_SPINS, DEFAULT_TMA_POLLS, 0u, 0u};
     const bool V_dev = on_device(V);
     if (init_mode == FCM_INIT_V && V_dev) ra.Vin = V;
@@ -185,7 +187,7 @@ extern "C" int fcm_run_noalloc(const float* x, int64_t n, int C, float m, float 
         std::memset(rep, 0, sizeof(*rep));
         rep->iters = out.iters;
         rep->status = out.status;
-        rep->flags = out.flags;
+        rep->flags = out.flags | (int)out.bounds;
         rep->C = C;
         rep->delta = out.delta;
         rep->J = out.J;

@@ -54,6 +54,8 @@ struct RunArgs {
     int max_iter;
     int from_u;        // 1 from U^0, 0 from V^0
     int resident;      // quads of x per pixel thread kept in shared memory
+    int max_blocks;    // blocks that the scratch has room for
+    int64_t guard_n;   // n, or fewer: what a FCM_DEBUG_BOUNDS build's guards take for n (run_guard_n)
     unsigned nonce;    // the run's number on its scratch, counting up by one from run to run
     WaitLimits lim;
     float V0[FCM_MAX_CLUSTERS];
@@ -86,5 +88,10 @@ struct RunShape {
     int blocks, threads, resident, smem;
 };
 RunShape run_shape(int64_t n, int C, int64_t max_blocks);
+
+// n; in a FCM_DEBUG_BOUNDS build FCM_DEBUG_BOUNDS_SHORT in the environment takes
+// that many pixels off, so that a test can see the guards at work: they then skip
+// accesses that are in bounds, and report them.
+int64_t run_guard_n(int64_t n);
 
 }  // namespace fcm

@@ -60,6 +60,7 @@
 // FCM_ERR_TIMEOUT.
 #include <type_traits>
 
+#include "fcm_bounds.cuh"
 #include "fcm_device.cuh"
 #include "fcm_df.cuh"
 #include "fcm_internal.h"
@@ -286,9 +287,14 @@ struct Px {
     int steps, resident;  // this thread's quads; how many of them are kept
     bool vec_x;           // x is 16-byte aligned
     bool vec_u;           // so are the rows of U and U^0, and n % 4 == 0
+    int64_t guard_n;      // a FCM_DEBUG_BOUNDS build checks every index against it
+    unsigned* bounds;     // and reports here
 
+    // Whether the pixels i .. i + count - 1 may be accessed.
+    __device__ __forceinline__ bool in(int64_t i, int count) const { return in_bounds(i >= 0 && i + count <= guard_n, bounds); }
     __device__ __forceinline__ float4 load(int step) const {
         const int64_t q = t0 + (int64_t)step * nt;
+        if (!in(4 * q, 4)) return make_float4(0.f, 0.f, 0.f, 0.f);
         if (vec_x) return __ldg(reinterpret_cast<const float4*>(x) + q);
         const float* p = x + 4 * q;
         return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
@@ -298,7 +304,8 @@ struct Px {
     __device__ __forceinline__ void tail(T&& f) const {
         if (t0 == (n >> 2) % nt) {
 #pragma unroll 1
-            for (int64_t i = n & ~(int64_t)3; i < n; ++i) f(i);
+            for (int64_t i = n & ~(int64_t)3; i < n; ++i)
+                if (in(i, 1)) f(i);
         }
     }
     // Reads the quads from global memory, two steps ahead, keeps the resident
@@ -314,7 +321,8 @@ struct Px {
             a = b;
             if (s + 2 < steps) b = load(s + 2);
             if (s < resident) xs[s * pt] = c;
-            f(c, 4 * (t0 + (int64_t)s * nt));
+            const int64_t i = 4 * (t0 + (int64_t)s * nt);
+            if (in(i, 4)) f(c, i);
         }
     }
     // The same, once the resident quads are in place.
@@ -335,7 +343,8 @@ struct Px {
                 a = b;
                 if (s + 2 < steps) b = load(s + 2);
             }
-            f(c, 4 * (t0 + (int64_t)s * nt));
+            const int64_t i = 4 * (t0 + (int64_t)s * nt);
+            if (in(i, 4)) f(c, i);
         }
     }
     // For unaligned rows of U: a warp takes 128 consecutive pixels, a lane the
@@ -348,10 +357,11 @@ struct Px {
         for (int64_t w = t0 >> 5; w < all; w += nw) {
             const int64_t i = (w << 7) + (threadIdx.x & 31);
             if ((w << 7) + 128 <= n) {
-                f(make_float4(__ldg(x + i), __ldg(x + i + 32), __ldg(x + i + 64), __ldg(x + i + 96)), i);
+                if (in(w << 7, 128)) f(make_float4(__ldg(x + i), __ldg(x + i + 32), __ldg(x + i + 64), __ldg(x + i + 96)), i);
             } else {
 #pragma unroll 1
-                for (int64_t k = i; k < n; k += 32) g(k);
+                for (int64_t k = i; k < n; k += 32)
+                    if (in(k, 1)) g(k);
             }
         }
     }
@@ -369,6 +379,14 @@ __device__ __forceinline__ Px run_px(const RunArgs& ra, f2* second) {
     px.nt = (int64_t)gridDim.x * px.pt;
     px.steps = (px.n >> 2) > px.t0 ? (int)(((px.n >> 2) - 1 - px.t0) / px.nt) + 1 : 0;
     px.resident = min(ra.resident, px.steps);
+    px.guard_n = ra.guard_n;
+    px.bounds = &ra.out->bounds;
+    if (kBoundsChecks) {
+        // the places of the resident quads lie in the block's dynamic shared memory
+        unsigned smem;
+        asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(smem));
+        if (!in_bounds((unsigned)(px.pt * 16 * (C + ra.resident)) <= smem, px.bounds)) px.resident = 0;
+    }
     px.vec_x = ((uintptr_t)px.x & 15) == 0;
     px.vec_u = px.vec_x && (px.n & 3) == 0 && ((uintptr_t)ra.U & 15) == 0 && (!ra.from_u || ((uintptr_t)ra.U0 & 15) == 0);
     return px;
@@ -544,6 +562,8 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     constexpr int P = pow2_at_least(2 * C);
     extern __shared__ __align__(16) f2 second[];  // [2 C][pt] second set of the sums, then the resident quads
     __shared__ RunShared<C> sh;
+    // the scratch has room for the grid's slots, and the words can count its blocks
+    if (!in_bounds((int)gridDim.x <= ra.max_blocks, &ra.out->bounds)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int pw = (int)(blockDim.x >> 5) - 1;  // pixel warps; the control warp follows
     const bool control = warp == pw;
@@ -875,12 +895,12 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         const int64_t i = (int64_t)(at * (double)n);
         if (px.vec_u) {
             wi = min(i, n - 2) & ~(int64_t)1;
-            sampled = true;
+            sampled = px.in(wi, 2);
         } else {
             const int64_t whole = n >> 7;
             wi = (min(i >> 7, whole - 1) << 7) + lane;
             ws = 32;
-            sampled = whole > 0;
+            sampled = whole > 0 && px.in(wi, ws + 1);
         }
         if (sampled) wx = pack2(__ldg(px.x + wi), __ldg(px.x + wi + ws));
     }
