@@ -76,7 +76,9 @@ __device__ __noinline__ void pass_a_chunk(const BinArgs& a, const SliceDesc& d, 
 #pragma unroll
     for (int q = 0; q < 2 * C; ++q) acc[q] = DF{0.0f, 0.0f};
     bool bad_x = false;
-    float umin = 0.0f, umax = 0.0f;  // a NaN shows in the sums of V^1 instead
+    // U^0 is bad where its bits, with -0 made 0, are above the largest finite
+    // number's: infinities, NaN and, by their sign, negative values
+    unsigned umax = 0u;
     unsigned* hw = sh.sub[warp];
     constexpr int LOADS = loads_a<C>();
     for (int i0 = lo + t; i0 < hi; i0 += BNT * LOADS) {
@@ -106,8 +108,7 @@ __device__ __noinline__ void pass_a_chunk(const BinArgs& a, const SliceDesc& d, 
 #pragma unroll
                 for (int j = 0; j < C; ++j) {
                     const float u0 = uc[q][j];
-                    umin = fminf(umin, u0);
-                    umax = fmaxf(umax, u0);
+                    umax = max(umax, __float_as_uint(__fadd_rn(u0, 0.0f)));
                     const float w = pow_m<MK>(u0, m);
                     num[j] = fmaf(w, xi, num[j]);
                     den[j] += w;
@@ -129,8 +130,8 @@ __device__ __noinline__ void pass_a_chunk(const BinArgs& a, const SliceDesc& d, 
             if (lane == 0) sh.wsum[warp][q] = dd;
         }
     }
-    // bit 0: some x is not a grey level; bit 1: U^0 has a negative or infinite value
-    const int bx = __syncthreads_or(bad_x), bu = __syncthreads_or(umin < 0.0f || !finite_f(umax));
+    // bit 0: some x is not a grey level; bit 1: U^0 has a negative or non-finite value
+    const int bx = __syncthreads_or(bad_x), bu = __syncthreads_or(umax >= 0x7f800000u);
     if ((bx || bu) && t == 0) atomicOr(&a.bad[s], (bx ? 1u : 0u) | (bu ? 2u : 0u));
     {
         unsigned c = 0;
@@ -215,9 +216,6 @@ __device__ __noinline__ void solve_run(const BinArgs& a, int r, const BinRun& ru
             s_tot[t] = mine;
         }
         __syncthreads();
-        // a NaN in U^0 shows in its denominator (pass A looks at the other bad values)
-#pragma unroll
-        for (int j = 0; j < C; ++j) bad |= s_tot[C + j].hi != s_tot[C + j].hi;
     }
     if (bad) {
         // not a grey-level slice (or a bad U^0 / V^0): the status, and V = V^0
