@@ -218,11 +218,12 @@ int ensure_single_workspace(fcm_ctx* h) {
 // the numbers start over, so no slot can show a tag of an earlier run of the
 // same number.
 int next_nonce(fcm_ctx* h, unsigned* nonce) {
-    if (++h->run_nonce == 0) {
+    if (h->run_nonce == 0xffffffffu) {
+        // (a memset that fails leaves the number: the next run tries again)
         CK(cudaMemsetAsync(h->d_slots, 0, run_scratch_bytes(max_run_sms(h)), h->stream));
-        h->run_nonce = 2;  // even, as 0: the banks go on alternating
+        h->run_nonce = 1;
     }
-    *nonce = h->run_nonce;
+    *nonce = ++h->run_nonce;
     return 0;
 }
 
