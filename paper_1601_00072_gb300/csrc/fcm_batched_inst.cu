@@ -108,7 +108,7 @@ struct BatchShared {
 struct TeamCtx {
     float4* slots;        // [T][2][TEAM_SLOT], this slice's
     unsigned* ctr;        // this slice's barrier counter (zero before the batch)
-    uint32_t spins;       // polls, 128 ns apart, before the barrier gives up
+    uint32_t spins;       // polls, 64 ns and an L2 round trip apart, before the barrier gives up
     uint32_t phantoms;    // arrivals beyond the team's (0 unless a test injects a barrier that never fills)
 };
 

@@ -18,14 +18,14 @@ constexpr int STATUS_RUNNING = 2;
 // (fcm_set_limits). Every spin or suspension loop counts against one of them
 // and, when it runs out, the kernel records FCM_ERR_TIMEOUT and returns.
 struct WaitLimits {
-    uint32_t grid_spins;  // polls, about 128 ns apart, of a grid-wide barrier
+    uint32_t grid_spins;  // polls, a fraction of a microsecond apart, of a grid-wide wait
     uint32_t tma_polls;   // suspensions, up to about 1 ms each, of a wait for TMA bytes
     uint32_t phantoms;    // arrivals every grid-wide barrier waits for beyond the
                           // grid's own: 0 in normal use; a test sets 1 to make
                           // every barrier give up (fault injection on the host side)
     uint32_t pad;
 };
-constexpr uint32_t DEFAULT_GRID_SPINS = 1u << 23;  // about 1 s
+constexpr uint32_t DEFAULT_GRID_SPINS = 1u << 23;  // a few seconds
 constexpr uint32_t DEFAULT_TMA_POLLS = 2048;       // about 2 s
 
 // Which half-step a launch of the pass performs.

@@ -26,8 +26,8 @@
 // in flight each: 23 or 31 warps with fewer registers were slower). x is kept in
 // shared memory up to 7 million pixels; beyond that, the rest of x comes from the
 // L2, two steps ahead of its use. On a small image it is the latency of an
-// iteration (1.9 us at 40,000 pixels): about 1 us of dependent steps in a block
-// and as much for the exchange. 60 iterations on a GB300, before (U stored; plain
+// iteration (1.9 us at 40,000 pixels): a single block of 512 pixels, whose exchange is
+// an L2 round trip that no other block contends for, takes 1.4. 60 iterations on a GB300, before (U stored; plain
 // loads and a launch per pass where n % 4 != 0) and after: 200x200 376 -> 151 us,
 // 199x201 909 -> 188 us, 1024x1024 716 -> 275 us, 256^3 6.01 -> 1.83 ms.
 //
@@ -45,14 +45,16 @@
 // fixed-point units come from n and the largest |x|, |V^0|, known after pass 0:
 // 2^-53 of the largest num_j possible, 2^-46 of n (the error of den_j is relative
 // to the center's step). A few outliers or a masked part at some sentinel value set
-// the largest |x|, and the other clusters' totals may lie wholly below the unit: a
-// block whose total loses more than its center's FP32 resolution to the rounding
-// says so in the word, and so does one whose total is no number; den_j below 2^-16 n
-// counts alike. Then (the same decision in every block) the totals go through the
-// slots, in FP32, and so do the next ones until the words would hold them. (A
-// second word for what the first one leaves of num_j is exact without that, but
-// costs every run: 40,000 pixels 151.6 -> 161.2 us on a line of its own, 172 on the
-// same line.) Pass 0's totals and J's always go through the slots.
+// the largest |x|, and the other clusters' totals may lie wholly below the unit:
+// when all blocks' roundings together could move a center by 2^-26 of it and are
+// not below 2^-16 of its step, when den_j is below 2^-16 n, or when some block's
+// total is no number (it adds a mark instead), then (the same decision in every
+// block) the totals go through the slots, in FP32, and so do the next ones until
+// the words would do. Measured there: 40,000 pixels 1.9 -> 2.8 us per iteration,
+// 1 M 3.8 -> 6.0. (A second word for what the first one leaves of num_j needs none
+// of that, but costs every run: 40,000 pixels, 60 iterations, 151.6 -> 161.2 us with
+// a line of its own, 172 on the same line.) Pass 0's totals and J's always go
+// through the slots.
 // Slots: a block's values with a 64-bit tag (the run's number and the exchange's
 // index) in one 16-byte store, polled until each block's shows the tag, added in
 // block order in compensated FP32.
@@ -171,17 +173,21 @@ __device__ __forceinline__ DF fixed_to_df(int64_t v, float unit) {
 // Bits of the sum of an exchange word.
 constexpr int NUM_BITS = 53, DEN_BITS = 46;
 constexpr uint64_t DEN_MARK = 2ull << DEN_BITS;  // 255 of them stay below 2^55
+// Iterations that a cluster's totals are taken to be resolved after an exchange
+// through the slots has shown that they are.
+constexpr int TRUST = 16;
 // The units of the fixed-point numbers.
 struct Fixed {
     float to_num, to_den, num_unit, den_unit;
     float num_max, den_max;  // no block's totals are above these
-    // Whether the words hold a block's totals a = num_j, b = den_j about the center
-    // v: no infinity or NaN, and the rounding of a to the unit is below 2^-16 of a, or
-    // moves the block's part of the center by less than 2^-26 of it. slack > 1 asks
-    // for that much more room.
-    __device__ __forceinline__ bool holds(float a, float b, float v, float slack) const {
-        const float half = (0.5f * slack) * num_unit;
-        return (fabsf(a) >= 0x1p16f * half || b * fabsf(v) >= 0x1p26f * half || a == 0.0f) && fabsf(a) <= num_max && b <= den_max;
+    float lost;              // all blocks' roundings to the unit, at most
+    float thick;             // least den_j, in slots, that the words may have again
+    // Whether a block's totals are numbers that the words can add.
+    __device__ __forceinline__ bool fits(float a, float b) const { return fabsf(a) <= num_max && b <= den_max; }
+    // Whether the roundings move a center v with the sums a, b by less than 2^-26 of
+    // it, or are below 2^-16 of what moves it. slack > 1 asks for that much more room.
+    __device__ __forceinline__ bool resolves(float a, float b, float v, float slack) const {
+        return b * fabsf(v) >= (0x1p26f * slack) * lost || fabsf(a) >= (0x1p16f * slack) * lost;
     }
 };
 // 2^e for e in [-126, 127].
@@ -409,6 +415,7 @@ struct RunShared {
     int4 ctl[2];
     uint64_t seen[2][C][2];    // the words of each cluster after their last exchange, of even and odd parity
     uint64_t seen_ctl[2];      // and the control word
+    int trust[C];              // see TRUST
     DF J;
     float delta;
     unsigned flags;            // bit 0: bad input
@@ -580,6 +587,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     const int max_iter = ra.max_iter;
     const bool tracing = ra.trace != nullptr;
 
+    if (threadIdx.x < C) sh.trust[threadIdx.x] = 0;
     if (threadIdx.x < 4 * C) (&sh.seen[0][0][0])[threadIdx.x] = 0ull;
     if (threadIdx.x < C) {
         const float v0 = ra.Vin ? ra.Vin[threadIdx.x] : ra.V0[threadIdx.x];
@@ -608,8 +616,7 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         w[0] = w[1] = 0ull;
     }
     char* const slots_raw = scratch + RUN_WORDS_BYTES;
-    Fixed fx{0.0f, 0.0f, 0.0f, 0.0f, -1.0f, -1.0f};  // holds nothing
-    float thick = 0.0f;  // least den_j, in slots, that the words may have again
+    Fixed fx{0.0f, 0.0f, 0.0f, 0.0f, -1.0f, -1.0f, 0.0f, 0.0f};  // nothing fits
 
     // This block's row of exchange nx + 1: cluster q's slots, or (q = C) the
     // maxima's and flags'.
@@ -668,13 +675,20 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         }
         if (lane == 0) st_slot(row + (int64_t)blockIdx.x * RUN_SLOT_BYTES, a, b, tag);
         DF na{0.0f, 0.0f}, da{0.0f, 0.0f};
-        bool slots = false;  // some block's totals do not fit the words with room to spare
+        bool fits = true;
+        float amax = 0.0f;  // the largest block's |num_j|
         const bool ok = collect(row, nb, tag, sh.lim.grid_spins, sh.lim.phantoms, [&](float p, float r) {
-            if (K == X_SUMS) slots |= !fx.holds(p, r, sh.v[cur][q], 4.0f);
+            if (K == X_SUMS) {
+                fits &= fx.fits(p, r);
+                amax = fmaxf(amax, fabsf(p));
+            }
             df_add(na, p);
             if (K != X_J) df_add(da, r);
         });
-        if (K == X_SUMS) slots = __any_sync(0xffffffffu, slots);
+        if (K == X_SUMS) {
+            fits = __all_sync(0xffffffffu, fits);
+            amax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(amax)));
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             // TwoSum is symmetric: every lane gets the same totals
@@ -690,7 +704,14 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
             return;
         }
         da = df_norm(da);
-        if (slots || !(da.hi >= thick)) sh.ctl[it].z = 1;
+        if (K == X_SUMS) {
+            // Would the words do? A center near 0 that hardly moves any more is
+            // resolved where the roundings are small against the largest block's part
+            // of the sum (parts that cancel), or every part is 0.
+            const bool ok2 = fx.resolves(amax, da.hi, sh.v[cur][q], 4.0f) || amax == 0.0f;
+            sh.trust[q] = fits && ok2 ? TRUST : 0;
+            if (!fits || !ok2 || !(da.hi >= fx.thick)) sh.ctl[it].z = 1;
+        }
         new_center(q, na, da, K == X_SUMS, cur, nxt);
     };
     // Reads words until they are complete.
@@ -714,9 +735,9 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
             b += __shfl_xor_sync(0xffffffffu, b, o);
         }
         if (lane != 0) return;
-        // Totals that the words do not hold add only a mark to den_j, beyond every
-        // possible sum of them: nothing but numbers reaches the arrival counts.
-        const bool fits = fx.holds(a, b, v, 1.0f);
+        // Totals that are no numbers, or too large, add only a mark to den_j, beyond
+        // every possible sum of them: nothing else may reach the arrival counts.
+        const bool fits = fx.fits(a, b);
         red_add_u64(w, (uint64_t)__float2ll_rn(fits ? a * fx.to_num : 0.0f) + ARRIVAL);
         red_add_u64(w + 1, (uint64_t)__float2ll_rn(fits ? b * fx.to_den : (float)DEN_MARK) + ARRIVAL);
         uint64_t* const seen = sh.seen[(nx + 1) & 1][q];
@@ -730,8 +751,13 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
         seen[0] = va;
         seen[1] = vb;
         if (!ok) sh.ctl[it].x = 1;
-        if (sb < (1ll << (DEN_BITS - 16)) || sb >= (int64_t)DEN_MARK) sh.ctl[it].z = 1;
-        else new_center(q, fixed_to_df(sa, fx.num_unit), fixed_to_df(sb, fx.den_unit), true, cur, nxt);
+        if (sb < (1ll << (DEN_BITS - 16)) || sb >= (int64_t)DEN_MARK) {
+            sh.ctl[it].z = 1;
+        } else {
+            const DF na = fixed_to_df(sa, fx.num_unit), da = fixed_to_df(sb, fx.den_unit);
+            new_center(q, na, da, true, cur, nxt);
+            if (!fx.resolves(na.hi, da.hi, v, 1.0f) && --sh.trust[q] < 0) sh.ctl[it].z = 1;
+        }
     };
     // Control warp: publishes whether this block's sample of iteration k reached
     // eps; collects, an iteration later, whether any block's did.
@@ -870,8 +896,8 @@ __global__ void __launch_bounds__(run_max_pt(C) + 32, 1)
     const bool fixed = en + ex <= 126;
     if (fixed) {
         const int e = min(126, NUM_BITS - en - ex);
-        fx = Fixed{pow2f(e), pow2f(DEN_BITS - en), pow2f(-e), pow2f(en - DEN_BITS), pow2f(min(127, en + ex)), 1.25f * pow2f(en)};
-        thick = pow2f(en - 15);
+        fx = Fixed{pow2f(e), pow2f(DEN_BITS - en), pow2f(-e), pow2f(en - DEN_BITS), pow2f(min(127, en + ex)), 1.25f * pow2f(en),
+                   (0.5f * (float)nb) * pow2f(-e), pow2f(en - 15)};
     }
     bool words = fixed;  // the next exchange of sums goes through the words (the same in every block)
     int status = FCM_NOT_CONVERGED, iters = 0;

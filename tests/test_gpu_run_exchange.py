@@ -181,3 +181,18 @@ def test_overflowed_totals(fcm):
         assert np.array_equal(ok, np.isfinite(vb)) and np.allclose(va[ok], vb[ok], rtol=1e-5, atol=1e-5)
     # and the handle goes on as before
     _check_centers(fcm, x, 2, 2.0, [20.0, 80.0])
+
+
+@pytest.mark.parametrize("n", [4000, 40001, 700000])
+@pytest.mark.parametrize("m", [2.0, 1.2])
+def test_masked_background(fcm, n, m):
+    """An exact background whose center goes to 0, in blocks that hold nothing
+    else, with and without a sentinel beside it; and a center that sits on 0."""
+    x, _ = _tissues(n, 8)
+    x[:n // 2] = 0.0
+    _check_centers(fcm, x, 3, m, [3.0, 25.0, 80.0], max_iter=40)
+    far = x.copy()
+    far[:n // 8] = 1e9
+    _check_centers(fcm, far, 4, m, [0.0, 25.0, 80.0, 1e9], eps=0.0, max_iter=24)
+    levels = np.where(x > 60.0, 255.0, np.where(x > 0.0, 100.0, 0.0))
+    _check_centers(fcm, levels, 3, m, [10.0, 90.0, 240.0], eps=0.0, max_iter=24)
