@@ -517,30 +517,34 @@ def bench_batched(h, dev, steps, warmup, plan=None, keep_results=False, n_slices
     h.model_load(warmstart.MODEL_PATH)
     stream = torch.cuda.current_stream(dev)
 
-    def timed(fn, reps):
+    spread = {}  # median and largest of the single calls behind each mean
+
+    def timed(fn, reps, name):
         for _ in range(warmup):
             fn()
         torch.cuda.synchronize(dev)
-        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        e0.record(stream)
-        for _ in range(reps):
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(reps + 1)]
+        ev[0].record(stream)
+        for e in ev[1:]:
             fn()
-        e1.record(stream)
+            e.record(stream)
         torch.cuda.synchronize(dev)
-        return e0.elapsed_time(e1) / reps
+        each = [a.elapsed_time(b) for a, b in zip(ev, ev[1:])]
+        spread[name] = {"ms_median": float(np.median(each)), "ms_max": float(max(each))}
+        return ev[0].elapsed_time(ev[-1]) / reps
 
     if plan:
         h.set_batched_plan(**plan)
     cold = Batch(cold)
     # results land in each Batch's host array; the Slice fields are filled
     # once after timing (the warm call's judge and reruns are inside its time)
-    ms_cold = timed(lambda: h.run_batched(cold, read_back=False), steps)
+    ms_cold = timed(lambda: h.run_batched(cold, read_back=False), steps, "cold")
     cold.read_back()
     plan_used = h.batched_plan()
     # the same cold batch, ordered and split by cost: each slice's iteration
     # count comes from a run on its grey-level histogram inside the call
     cold_p = Batch([Slice(x=x, C=c, U0=u) for x, c, u in zip(xs, Cs, u0s)])
-    ms_cold_p = timed(lambda: h.run_batched(cold_p, read_back=False, presolve=True), steps)
+    ms_cold_p = timed(lambda: h.run_batched(cold_p, read_back=False, presolve=True), steps, "cold_presolved")
     cold_p.read_back()
     plan_cold_p = h.batched_plan()
     warm = Batch([Slice(x=x, C=c, U0=u) for x, c, u in zip(xs, Cs, u0s)])
@@ -549,7 +553,7 @@ def bench_batched(h, dev, steps, warmup, plan=None, keep_results=False, n_slices
     def run_warm():
         n_ran_cold[0] = h.run_batched_warm(warm, read_back=False)[1]
 
-    ms_warm = timed(run_warm, steps)
+    ms_warm = timed(run_warm, steps, "warm")
     warm.read_back()
     plan_warm = h.batched_plan()
     # every returned slice against the cold batch by the acceptance rule; the
@@ -562,7 +566,7 @@ def bench_batched(h, dev, steps, warmup, plan=None, keep_results=False, n_slices
     ms_charge = 0.0
     if bad_i.size:
         bad = Batch([Slice(x=xs[i], C=Cs[i], U0=u0s[i]) for i in bad_i])
-        ms_charge = timed(lambda: h.run_batched(bad, read_back=False), steps)
+        ms_charge = timed(lambda: h.run_batched(bad, read_back=False), steps, "charged")
     it_c = np.array([s.iters for s in cold.slices])
     it_w = np.array([s.iters for s in warm.slices])
     ran_cold = np.array([s.init == "U" for s in warm.slices])
@@ -571,7 +575,7 @@ def bench_batched(h, dev, steps, warmup, plan=None, keep_results=False, n_slices
     # the same cold batch on each slice's 256-bin histogram (one CTA per
     # slice): the same iterates up to rounding, compared with the cold run
     hist = Batch([Slice(x=x, C=c, U0=u) for x, c, u in zip(xs, Cs, u0s)])
-    ms_hist = timed(lambda: h.run_batched_hist(hist, read_back=False), steps)
+    ms_hist = timed(lambda: h.run_batched_hist(hist, read_back=False), steps, "histogram_domain")
     hist.read_back()
     it_h = np.array([s.iters for s in hist.slices])
     verr = np.array([np.max(np.abs(np.asarray(a.V64) - np.asarray(c.V64)) / np.maximum(np.abs(np.asarray(c.V64)), 1.0))
@@ -597,6 +601,7 @@ def bench_batched(h, dev, steps, warmup, plan=None, keep_results=False, n_slices
                            "mean_iters": float(np.mean([s.iters for s in cold_p.slices])), "plan": plan_cold_p},
         "warm_over_cold": warm_ips / cold_ips,
         "warm_over_cold_presolved": warm_ips / (n_img / (ms_cold_p / 1e3)),
+        "warm_over_cold_presolved_medians": spread["cold_presolved"]["ms_median"] / (spread["warm"]["ms_median"] + ms_charge),
         "plan": plan_used,
         "plan_warm": plan_warm,
         "histogram_domain": {
@@ -608,6 +613,9 @@ def bench_batched(h, dev, steps, warmup, plan=None, keep_results=False, n_slices
             "iters_within_1_of_cold": float(np.mean(np.abs(it_h - it_c) <= 1)),
             "center_rel_err_vs_cold": {"max": float(verr.max()), "fraction_within_1e-5": float(np.mean(verr <= 1e-5))}},
     }
+    for name, v in spread.items():
+        if name in res:
+            res[name].update(v)
     if keep_results:
         return res, (cold.slices, warm.slices, hist.slices, host, Cs, cold_p.slices)
     return res

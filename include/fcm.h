@@ -27,14 +27,27 @@
  *     step 3); the run stops with (U^k, V^k) when delta_k < eps (strict),
  *     else V^{k+1} = centers(U^k). V^1 comes from the initial U^0, or from
  *     U^0 = membership(V^0) when initial centers are given.
- *   - Arithmetic: memberships and per-thread sums in FP32; the sums across
- *     threads and blocks (center numerators/denominators and J) in
- *     compensated FP32 (double-float, about 44 bits) or FP64, in a fixed
- *     order. A run is deterministic: the same call gives the same bits.
- *     The histogram-domain entry points form V^1 the same way from the
- *     pixels; their loop over the 256 bins sums non-negative terms in FP32
- *     within each warp (a fixed tree, at most five roundings) and combines
- *     the warp totals in double-float.
+ *   - Arithmetic: memberships in FP32. V^1 from a given U^0: FP32 over at
+ *     most 16 pixels per thread, then compensated FP32 (double-float, about 44
+ *     bits). Between iterations the numerators of Eq. 3 are centered on V^k
+ *     (num_j = sum u^m (x - v_j), v_j moves by num_j / den_j), so that the
+ *     rounding of the sums is relative to the pixels' distance from the center
+ *     and that of den_j to the center's step; a center that moves by more than
+ *     64 times its new value has its sums taken again, centered on the new one.
+ *     Within a block the single-image and multi-feature runs add in FP32 (two
+ *     levels per thread, a tree over lanes, and over warps in the single-image
+ *     run); batched slices in FP32 over 32 pixels per thread, then in
+ *     double-float. Across blocks the sums are double-float; the single-image
+ *     run adds them as 64-bit fixed-point integers where the rounding of every
+ *     block's total to the unit is below 2^-16 of that total or below 2^-26 of
+ *     the center, and in double-float elsewhere. J is FP32 within a block of the
+ *     single-image run and double-float elsewhere. Center quotients are
+ *     double-float. The histogram-domain loop adds two bins per thread, an FP32
+ *     tree of five levels in each warp, and the four warp totals in
+ *     double-float, with numerators centered within the grey scale. The passes
+ *     that FCM_OPT_NO_PERSISTENT, NO_GRAPH and NO_TMA select add uncentered FP32
+ *     sums per thread and block, in FP64 across blocks. Every order is fixed (or
+ *     the sums are integers): the same call gives the same bits.
  *   - Ownership: the caller owns x, U, V and every output array; the library
  *     never frees them. A handle owns its device workspace, CUDA graphs and
  *     autotuning cache, and frees them in fcm_destroy.
@@ -89,7 +102,9 @@ extern "C" {
                                  between iterations (an iteration reads only x; U^k
                                  is written once at the end): refused unless
                                  n % 4 == 0 and the rows are 16-byte aligned; takes
-                                 precedence over the three options above */
+                                 precedence over the three options above. (On a device
+                                 that the kernel does not fit, the passes with a stored
+                                 U run all the same.) */
 #define FCM_OPT_DETERMINISTIC 32 /* bit-reproducible results; every run is (kept for
                                      callers that ask for it) */
 

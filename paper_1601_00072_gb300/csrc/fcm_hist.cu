@@ -69,8 +69,9 @@ constexpr int HCHUNK = 4;  // pixels per thread whose loads are issued together 
 // C = 4): twice the warps of an unbounded build to cover the loads' latency.
 // VEC: rows of 16-byte-aligned quads (n % 4 == 0). A thread then takes two quads
 // of pixels per step with 128-bit loads, a quarter of the load instructions, and
-// folds its sums into double-float every eight pixels instead of four: the pass is
-// bound by its instructions as much as by HBM.
+// folds its sums into double-float every eight pixels instead of four (the error of
+// V^1 against 64 bits is the same over 2^12 to 2^24 pixels): the pass is bound by
+// its instructions as much as by HBM.
 template <int C, int MK, bool FROM_U, bool VEC>
 __global__ void __launch_bounds__(HNT, C <= 4 ? (VEC ? 3 : 4) : 2) k_hist_pass0(const float* __restrict__ x, const float* __restrict__ U0,
                                                    int64_t n, float m, HistState* st, double* __restrict__ part) {

@@ -28,8 +28,8 @@
 // L2, two steps ahead of its use. On a small image it is the latency of an
 // iteration (1.9 us at 40,000 pixels): a single block of 512 pixels, whose exchange is
 // an L2 round trip that no other block contends for, takes 1.4. 60 iterations on a GB300, before (U stored; plain
-// loads and a launch per pass where n % 4 != 0) and after: 200x200 376 -> 151 us,
-// 199x201 909 -> 188 us, 1024x1024 716 -> 275 us, 256^3 6.01 -> 1.83 ms.
+// loads and a launch per pass where n % 4 != 0) and after: 200x200 374 -> 153 us,
+// 199x201 902 -> 191 us, 1024x1024 717 -> 273 us, 256^3 6.02 -> 1.77 ms.
 //
 // The exchange. Between iterations every block adds its totals of (num_j, den_j)
 // as 64-bit fixed-point numbers to one word each, with a reduction in the L2; the
